@@ -210,11 +210,11 @@ def run(st: dict):
 
 
 def _env_bytes(n: int, side: int, h: int, w: int, sprites: int, steps: int, gray: int) -> float:
-    """One launch over n envs: per step the frame (and its grayscale plane), the action, reward and done
-    flag; per launch the state fields read and the pose written, and the map at the one bit a cell that
-    movement and rays need."""
-    per_step = 3 * h * w + (h * w if gray else 0) + 6
-    per_launch = 53 + 9 * sprites + 19 + side * side / 8
+    """One launch over n envs: per step the frame, the action, reward and done flag; per launch the state
+    fields read and the pose written, the grayscale planes it leaves (of the last four frames at most), and
+    the map at the one bit a cell that movement and rays need."""
+    per_step = 3 * h * w + 6
+    per_launch = 53 + 9 * sprites + 19 + side * side / 8 + (min(steps, 4) * h * w if gray else 0)
     return float(n) * (steps * per_step + per_launch)
 
 
