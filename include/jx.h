@@ -327,8 +327,8 @@ jx_status jx_set_state(jx_env* env, const void* h_buf, size_t bytes);
 jx_status jx_sync_status(jx_env* env, void* stream);
 
 /* Number of kernel launches this env has issued since creation. For maze
- * configs with a next-episode block (see jx_create), jx_reset, jx_step and
- * jx_rollout each also launch the three kernels that build episodes ahead (a
+ * configs with a next-episode block (see jx_create) and batches of many envs
+ * (at least 3 x 28 per SM), jx_reset, jx_step and jx_rollout each also launch the three kernels that build episodes ahead (a
  * count, the walls of builds that start, then the build's share of the launch,
  * after a 4-byte cudaMemsetAsync on the same stream; all capturable in a CUDA
  * graph). */

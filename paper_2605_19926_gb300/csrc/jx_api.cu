@@ -173,7 +173,7 @@ jx_status run(jx_env* env, const jx::Params& p, int mode, void* stream) {
   DeviceGuard g(env->device);
   if (g.err != cudaSuccess) return cuda_fail(g.err, "cudaSetDevice");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (p.nx_ep && (mode == jx::MODE_STEP || mode == jx::MODE_ROLLOUT || mode == jx::MODE_RESET)) {
+  if (jx::pregen_runs(p) && (mode == jx::MODE_STEP || mode == jx::MODE_ROLLOUT || mode == jx::MODE_RESET)) {
     cudaError_t err = jx::pregen_launch(p, mode == jx::MODE_ROLLOUT ? p.steps : 1, mode == jx::MODE_RESET, s);
     if (err != cudaSuccess) return cuda_fail(err, "pre-generation launch");
     env->launches.fetch_add(jx::kPregenKernels, std::memory_order_relaxed);

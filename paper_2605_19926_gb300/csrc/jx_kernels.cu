@@ -151,7 +151,7 @@ __global__ void __launch_bounds__(128) pregen_count_kernel(const __grid_constant
 // draws of all cells at once, with the GPU's full occupancy; the walk needs
 // them laid before its first step).
 __global__ void __launch_bounds__(256) pregen_walls_kernel(const __grid_constant__ Params p, int reset) {
-  if (p.nx_count[1] == 0u || p.n < p.nx_min) return;  // the whole grid: no build starts
+  if (p.nx_count[1] == 0u) return;  // the whole grid: no build starts
   const int per_env = p.S * p.S / 16;
   const int64_t items = (int64_t)p.n * per_env;
   for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < items;
@@ -175,7 +175,7 @@ __global__ void __launch_bounds__(256) pregen_walls_kernel(const __grid_constant
 // block for side 128) and in the words array between launches.
 __global__ void __launch_bounds__(kPregenThreads) pregen_kernel(const __grid_constant__ Params p, int steps, int reset) {
   extern __shared__ uint32_t pregen_sm[];
-  if (*p.nx_count == 0u || p.n < p.nx_min) return;  // the whole grid
+  if (*p.nx_count == 0u) return;  // the whole grid
   const LaneSlot L = lane_slot(p.S);
   const LaneWords W = lane_words(pregen_sm + threadIdx.x, blockDim.x, L);
   const int total = 2 * L.n - 1;
@@ -316,7 +316,7 @@ size_t pregen_work_bytes(int S) {
 }
 
 cudaError_t pregen_launch(const Params& p, int steps, bool reset, cudaStream_t stream) {
-  if (p.nx_ep == nullptr || p.nx_lanes <= 0) return cudaSuccess;
+  if (!pregen_runs(p)) return cudaSuccess;
   cudaError_t err = cudaMemsetAsync(p.nx_count, 0, 2 * sizeof(uint32_t), stream);
   if (err != cudaSuccess) return err;
   pregen_count_kernel<<<(p.n + 127) / 128, 128, 0, stream>>>(p, reset ? 1 : 0);
