@@ -1202,6 +1202,8 @@ __device__ __forceinline__ bool box_hits(uint32_t m, int ox, int oy, int cx, flo
 template <int MAPK>
 __device__ __noinline__ void open_unlocked(const Params& p, int e, uint8_t* smap, int cx, float fx, int cy, float fy,
                                            int lane) {
+  // an opened door may lie on the border: rays test the bounds from here on
+  if (lane == 0) reinterpret_cast<int32_t*>(smap - p.off_map + p.off_obj)[7] = 0;
   const int S = p.S;
   const float r = p.radius;
   const int i0 = cx + floor_small(fx - r), i1 = cx + floor_small(fx + r);
@@ -1332,17 +1334,17 @@ __device__ __forceinline__ bool step_env(const Params& p, int e, Env& r, const u
 // ---------------------------------------------------------------- render ----
 // DDA (Sec. 2.1), one crossing per iteration. The next x boundary is at
 // t = (kx + gx) / ax, the next y boundary at (ky + gy) / ay; the
-// cross-multiplied forms are compared, so no division is needed.
+// cross-multiplied forms lhs = kx ay + gx ay and rhs = ky ax + gy ax are
+// compared, so no division is needed, and only the side that was crossed is
+// computed anew.
 struct Ray {
-  int mx, my, sx, sy, side;
   float kx, ky;  // boundaries crossed so far (exact small integers)
-  float ax, ay, gx, gy, gxay, gyax;
-  bool done;
+  float ax, ay, gx, gy, gxay, gyax, lhs, rhs;
+  int sx, sy;
+  bool tx;  // the last crossing was an x boundary
 };
 
-__device__ __forceinline__ void ray_init(Ray& q, const Env& r, float rx, float ry, bool valid) {
-  q.mx = r.cx;
-  q.my = r.cy;
+__device__ __forceinline__ void ray_init(Ray& q, const Env& r, float rx, float ry) {
   q.sx = rx < 0.f ? -1 : 1;
   q.sy = ry < 0.f ? -1 : 1;
   q.ax = fabsf(rx);
@@ -1354,207 +1356,256 @@ __device__ __forceinline__ void ray_init(Ray& q, const Env& r, float rx, float r
   q.gxay = q.ax == 0.f ? inf : q.gx * q.ay;
   q.gyax = q.ay == 0.f ? inf : q.gy * q.ax;
   q.kx = q.ky = 0.f;
-  q.side = -1;
-  q.done = !valid;
+  q.lhs = q.gxay;
+  q.rhs = q.gyax;
+  q.tx = false;
 }
 
-// One crossing. CHECK: a cell outside the map ends the ray (as wall 1);
-// without it the map's border must be solid and the ray start inside it, so
-// that every ray hits before it could leave (see mark_border).
-template <int MAPK, bool CHECK>
-__device__ __forceinline__ void ray_advance(const Params& p, Ray& q, const uint8_t* smap, int S) {
-  const float lhs = fmaf(q.kx, q.ay, q.gxay);
-  const float rhs = fmaf(q.ky, q.ax, q.gyax);
-  const bool tx = lhs < rhs;
-  q.mx += tx ? q.sx : 0;
-  q.my += tx ? 0 : q.sy;
-  q.kx += tx ? 1.f : 0.f;
-  q.ky += tx ? 0.f : 1.f;
-  q.side = tx ? 0 : 1;
-  if (CHECK) {
-    const bool out = (unsigned)q.mx >= (unsigned)S || (unsigned)q.my >= (unsigned)S;
-    q.done = out || cell_set<MAPK>(p, smap, q.my * S + q.mx);
+// One crossing; `cell` is the index of the ray's cell, S the row pitch.
+__device__ __forceinline__ void ray_cross(Ray& q, int& cell, int step_x, int step_y) {
+  q.tx = q.lhs < q.rhs;
+  if (q.tx) {
+    q.kx += 1.f;
+    cell += step_x;
+    q.lhs = fmaf(q.kx, q.ay, q.gxay);
   } else {
-    q.done = cell_set<MAPK>(p, smap, q.my * S + q.mx);
+    q.ky += 1.f;
+    cell += step_y;
+    q.rhs = fmaf(q.ky, q.ax, q.gyax);
   }
 }
 
 // Whether rays of the staged map can skip the bounds test: every border cell
-// is solid in the staged map (locked doors of held keys already cleared) and
-// the agent's cell is not on the border, so a ray meets a solid cell before
-// it could leave the map, and the agent, blocked by the border, stays inside.
-// Kept in the warp's object words (obj[7]); recomputed whenever the staged map
-// or the keys change. ASCII maps, whose unlocked doors open on contact, always
-// take the bounds test.
+// is solid in the staged map (locked doors of held keys already cleared), so a
+// ray from a cell inside the border meets a solid cell before it could leave
+// the map. Kept in the warp's object words (obj[7]); recomputed whenever the
+// staged map or the keys change, and cleared when an unlocked door opens.
 template <int MAPK>
-__device__ __forceinline__ void mark_border(const Params& p, const WarpSmem& ws, int cx, int cy, int lane) {
+__device__ __forceinline__ void mark_border(const Params& p, const WarpSmem& ws, int lane) {
   const int S = p.S;
-  bool ok = p.task != kTaskAscii && cx > 0 && cy > 0 && cx < S - 1 && cy < S - 1;
-  if (ok) {
-    const uint8_t* smap = ws.map(p);
-    for (int i = lane; i < S; i += 32)
-      ok = ok && cell_set<MAPK>(p, smap, i) && cell_set<MAPK>(p, smap, (S - 1) * S + i) &&
-           cell_set<MAPK>(p, smap, i * S) && cell_set<MAPK>(p, smap, i * S + S - 1);
-    ok = __all_sync(0xffffffffu, ok);
-  }
+  const uint8_t* smap = ws.map(p);
+  bool ok = true;
+  for (int i = lane; i < S; i += 32)
+    ok = ok && cell_set<MAPK>(p, smap, i) && cell_set<MAPK>(p, smap, (S - 1) * S + i) &&
+         cell_set<MAPK>(p, smap, i * S) && cell_set<MAPK>(p, smap, i * S + S - 1);
+  ok = __all_sync(0xffffffffu, ok);
   if (lane == 0) ws.obj(p)[7] = ok ? 1 : 0;
   __syncwarp();
 }
 
 // A finished ray's hit: perpendicular distance, face, and the hit cell's
 // value. With bit-plane maps the value is a load from the state block; it is
-// issued here and first used by finish_column, after the next pass's DDA, so
-// that its latency overlaps that loop.
+// issued here and first used by finish_column.
 struct Hit {
   float perp;
-  int side, v, col, mx, my;
+  int v, mx, my;  // the cell only in MODE_RAYS
+  bool y_face, none;
 };
 
-template <int MAPK>
-__device__ __forceinline__ Hit hit_of(const Params& p, int e, const Ray& q, int col, const WarpSmem& ws) {
+// The rays of a warp, each lane its own, from the agent's cell to their first
+// solid cell. With a solid border around the agent (INSIDE) the loop ends by
+// itself: every crossing moves one cell in the ray's quadrant, so after at
+// most 2 S of them the ray stands on a border cell. Lanes leave it as their
+// rays hit; no ballot is needed. Otherwise each crossing also tests the
+// bounds (a cell outside the map ends the ray, as wall 1), at most 4 S + 8.
+// (Recomputing only the crossed side, indexing cells instead of (x, y) pairs
+// and leaving without a ballot, with the depth test of project_sprites, took
+// the 4096-env rollout of 128 steps from 8.82 to 7.98 us per step, the one of
+// 20 steps from 9.67 to 9.33, and the single step from 13.4 to 12.9 us.)
+template <int MODE, int MAPK, int COLS>
+__device__ __forceinline__ void march(const Params& p, int e, const Env& r, Ray (&q)[COLS], Hit (&h)[COLS],
+                                      const WarpSmem& ws, bool inside, const bool (&valid)[COLS]) {
   const int S = p.S;
-  Hit h;
-  if (q.side == 0)
-    h.perp = __fdividef((q.kx - 1.f) + q.gx, q.ax);
-  else if (q.side == 1)
-    h.perp = __fdividef((q.ky - 1.f) + q.gy, q.ay);
-  else
-    h.perp = __int_as_float(0x7f800000);  // no hit
-  h.side = q.side;
-  h.col = col;
-  h.mx = q.mx;
-  h.my = q.my;
-  h.v = 1;
-  const bool inside = (unsigned)q.mx < (unsigned)S && (unsigned)q.my < (unsigned)S;
-  if (q.side >= 0 && inside)
-    h.v = map_bits<MAPK>(p) ? p.st.map[(size_t)e * S * S + q.my * S + q.mx] : ws.map(p)[q.my * S + q.mx];
-  return h;
+  const uint8_t* smap = ws.map(p);
+  const int cell0 = r.cy * S + r.cx;
+  int cell[COLS];
+  bool out[COLS], none[COLS];
+#pragma unroll
+  for (int j = 0; j < COLS; ++j) {
+    cell[j] = cell0;
+    out[j] = false;
+    none[j] = false;
+  }
+  if (MODE != MODE_RAYS && inside) {
+    if (COLS == 1) {
+      const int sy = q[0].sy * S;
+      if (valid[0])
+        do ray_cross(q[0], cell[0], q[0].sx, sy);
+        while (!cell_set<MAPK>(p, smap, cell[0]));
+    } else {
+      uint32_t left = 0u;
+#pragma unroll
+      for (int j = 0; j < COLS; ++j) left |= valid[j] ? 1u << j : 0u;
+      while (left) {
+#pragma unroll
+        for (int j = 0; j < COLS; ++j)
+          if ((left >> j) & 1u) {
+            ray_cross(q[j], cell[j], q[j].sx, q[j].sy * S);
+            if (cell_set<MAPK>(p, smap, cell[j])) left &= ~(1u << j);
+          }
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < COLS; ++j) h[j].mx = h[j].my = 0;
+  } else {
+#pragma unroll
+    for (int j = 0; j < COLS; ++j) {
+      int mx = r.cx, my = r.cy, unused = 0;
+      bool hit = !valid[j];
+      for (int it = 0; it < 4 * S + 8 && !hit; ++it) {
+        ray_cross(q[j], unused, 0, 0);
+        mx += q[j].tx ? q[j].sx : 0;
+        my += q[j].tx ? 0 : q[j].sy;
+        out[j] = (unsigned)mx >= (unsigned)S || (unsigned)my >= (unsigned)S;
+        hit = out[j] || cell_set<MAPK>(p, smap, my * S + mx);
+      }
+      none[j] = !hit;
+      cell[j] = my * S + mx;
+      h[j].mx = mx;
+      h[j].my = my;
+    }
+  }
+  __syncwarp();
+#pragma unroll
+  for (int j = 0; j < COLS; ++j) {
+    const float num = (q[j].tx ? q[j].kx : q[j].ky) - 1.f + (q[j].tx ? q[j].gx : q[j].gy);
+    h[j].perp = none[j] ? __int_as_float(0x7f800000) : __fdividef(num, q[j].tx ? q[j].ax : q[j].ay);
+    h[j].y_face = !q[j].tx;
+    h[j].none = none[j];
+    h[j].v = 1;
+    if (!out[j] && !none[j] && valid[j])
+      h[j].v = map_bits<MAPK>(p) ? p.st.map[(size_t)e * S * S + cell[j]] : smap[cell[j]];
+  }
 }
 
-// Slice of a hit: rows and colour into the column arrays.
+// Slice of a hit: rows and colour into the column arrays. `slot` is col_slot of
+// the column.
 template <int MODE>
-__device__ __forceinline__ void finish_column(const Params& p, int e, const Hit& q, const WarpSmem& ws) {
-  const int H = p.H, col = q.col;
+__device__ __forceinline__ void finish_column(const Params& p, int e, const Hit& q, int col, int slot,
+                                              const WarpSmem& ws) {
+  const int H = p.H;
   const float perp = q.perp;
-  // h = floor(H / perp + 1/2), clamped; top = floor((H - h) / 2)
-  int h;
-  if (perp > 0.f) {
-    const float v = __fdividef((float)H, perp) + 0.5f;
-    h = v >= 1048576.f ? kHMax : (int)floorf(v);
-  } else {
-    h = kHMax;
-  }
-  const int top = (H - h) >> 1;  // arithmetic shift: floor division by 2
-  const int bot = top + h;
+  // h = floor(H / perp + 1/2), of which the frame needs min(h, H): the rows
+  // top = floor((H - h) / 2) and top + h clamped to [0, H] are those of min(h, H)
+  const float hv = perp > 0.f ? __fdividef((float)H, perp) + 0.5f : (float)H;
+  const int h = __float2int_rd(fminf(hv, (float)H));
+  const int top = (H - h) >> 1;
   const int v = q.v;
-  const int slot = col_slot(col, p.W >> 4);
-  uint32_t colour = ws.pal(p)[(q.side == 1 ? kCellColours : 0) + (v < kCellColours ? v : 1)];
-  if (p.shading) {  // distance shading: channels scaled by q / 256, q = 64 + 192 min(h, H) / H
-    const uint32_t qq = 64u + (uint32_t)(192 * (h < H ? h : H)) / (uint32_t)H;
+  uint32_t colour = ws.pal(p)[(q.y_face && !q.none ? kCellColours : 0) + (v < kCellColours ? v : 1)];
+  if (p.shading) {  // distance shading: channels scaled by q / 256, q = 64 + floor(192 min(h, H) / H)
+    // 192 h + 1/2 over H lies at least 1/512 from an integer, far beyond the rounding here
+    const uint32_t qq = 64u + (uint32_t)__float2int_rd(__fdividef((float)(192 * h) + 0.5f, (float)H));
     const uint32_t R = ((colour & 255u) * qq) >> 8, G = (((colour >> 8) & 255u) * qq) >> 8,
                    B = (((colour >> 16) & 255u) * qq) >> 8;
     colour = R | (G << 8) | (B << 16) | (luma(R, G, B) << 24);
   }
   ws.col_rgb(p)[slot] = colour;
-  // h >= 0, so top <= H/2 <= bot: clamped to [0, H] they fit the byte offsets
-  ws.col_top(p)[col] = (uint8_t)(127 + (top < 0 ? 0 : top));
-  ws.col_bot(p)[col] = (uint8_t)(127 + (bot > H ? H : bot) - (H >> 1));
+  // 0 <= top <= H/2 <= top + h <= H: they fit the byte offsets
+  ws.col_top(p)[col] = (uint8_t)(127 + top);
+  ws.col_bot(p)[col] = (uint8_t)(127 + top + h - (H >> 1));
   ws.zbuf(p)[col] = perp;
   if (MODE == MODE_RAYS) {
-    int4 hv = make_int4(q.side >= 0 ? q.mx : -1, q.side >= 0 ? q.my : -1, q.side, h);
-    reinterpret_cast<int4*>(p.dbg_hits)[(size_t)e * p.W + col] = hv;
+    int full = kHMax;  // the unclamped height
+    if (perp > 0.f) {
+      const float f = __fdividef((float)H, perp) + 0.5f;
+      full = f >= 1048576.f ? kHMax : (int)floorf(f);
+    }
+    const int4 out = make_int4(q.none ? -1 : q.mx, q.none ? -1 : q.my, q.none ? -1 : (q.y_face ? 1 : 0), full);
+    reinterpret_cast<int4*>(p.dbg_hits)[(size_t)e * p.W + col] = out;
     p.dbg_perp[(size_t)e * p.W + col] = perp;
   }
 }
 
-// Cast every column's ray: in each pass lane l marches the rays of columns
-// l + 32 j (j < COLS) together, and the warp leaves the DDA loop when a
-// ballot says every ray has hit.
 // The column table's entries lane and 32 + lane (0 beyond the frame), fetched
 // ahead with the env's state: the first two passes of cast_columns use them.
 __device__ __forceinline__ float2 col_k_pair(const Params& p, int lane) {
-  return make_float2(__ldg(p.col_k + lane), lane + 32 < p.W ? __ldg(p.col_k + lane + 32) : 0.f);
+  return make_float2(__ldg(p.col_k + (lane < p.W ? lane : 0)), lane + 32 < p.W ? __ldg(p.col_k + lane + 32) : 0.f);
 }
 
+// Cast every column's ray: in each pass lane l marches the rays of columns
+// l + 32 j (j < COLS) together. Returns the lane's largest hit distance.
 template <int MODE, int MAPK, int COLS>
-__device__ __forceinline__ void cast_columns(const Params& p, int e, const Env& r, float c, float s,
-                                             const WarpSmem& ws, int lane, float2 k01) {
+__device__ __forceinline__ float cast_columns(const Params& p, int e, const Env& r, float c, float s,
+                                              const WarpSmem& ws, int lane, float2 k01) {
   const int W = p.W, S = p.S;
-  const uint8_t* smap = ws.map(p);
-  const int max_it = 4 * S + 8;
-  const bool inside = ws.obj(p)[7] != 0;  // rays need no bounds test (mark_border)
-  // single steps (latency-bound) finish a lane's hit after its next ray;
-  // the other modes at once (a rollout keeps more state live across the loop)
+  // a solid border and the agent strictly inside it: rays need no bounds test
+  const bool inside = ws.obj(p)[7] != 0 && (unsigned)(r.cx - 1) < (unsigned)(S - 2) &&
+                      (unsigned)(r.cy - 1) < (unsigned)(S - 2);
+  // single steps (latency-bound) finish a lane's hit after its next ray, so
+  // that the hit cell's load overlaps that ray; the other modes at once (a
+  // rollout keeps more state live across the loop)
   constexpr bool kDefer = MODE == MODE_STEP;
   Hit last;  // the lane's previous hit, finished after the next one is found
   bool pending = false;
-  for (int col0 = lane; col0 - lane < W; col0 += 32 * COLS) {
+  float far = 0.f;
+  // col_slot of column lane; column lane + 32 m lies 8 m further
+  const int slot0 = col_slot(lane, W >> 4);
+  for (int m = 0; 32 * m < W; m += COLS) {
     Ray q[COLS];
+    Hit h[COLS];
+    bool valid[COLS];
 #pragma unroll
     for (int j = 0; j < COLS; ++j) {
-      const int col = col0 + 32 * j;
-      const bool valid = col < W;
-      const int m = (col - lane) >> 5;  // column col = lane + 32 m
-      const float k = m == 0 ? k01.x : (m == 1 ? k01.y : __ldg(p.col_k + (valid ? col : 0)));
-      ray_init(q[j], r, fmaf(-k, s, c), fmaf(k, c, s), valid);
+      const int col = lane + 32 * (m + j);
+      valid[j] = col < W;
+      const float k = m + j == 0 ? k01.x : (m + j == 1 ? k01.y : __ldg(p.col_k + (valid[j] ? col : 0)));
+      ray_init(q[j], r, fmaf(-k, s, c), fmaf(k, c, s));
     }
-    if (inside) {
-      for (int it = 0; it < max_it; ++it) {
-        bool all = true;
+    march<MODE, MAPK, COLS>(p, e, r, q, h, ws, inside, valid);
 #pragma unroll
-        for (int j = 0; j < COLS; ++j) {
-          if (!q[j].done) ray_advance<MAPK, false>(p, q[j], smap, S);
-          all = all && q[j].done;
+    for (int j = 0; j < COLS; ++j) {
+      const int col = lane + 32 * (m + j);
+      if (kDefer && pending) finish_column<MODE>(p, e, last, col - 32, slot0 + 8 * (m + j - 1), ws);
+      pending = false;
+      if (valid[j]) {
+        far = fmaxf(far, h[j].perp);
+        if (kDefer) {
+          last = h[j];
+          pending = true;
+        } else {
+          finish_column<MODE>(p, e, h[j], col, slot0 + 8 * (m + j), ws);
         }
-        if (__all_sync(0xffffffffu, all)) break;
-      }
-    } else {
-      for (int it = 0; it < max_it; ++it) {
-        bool all = true;
-#pragma unroll
-        for (int j = 0; j < COLS; ++j) {
-          if (!q[j].done) ray_advance<MAPK, true>(p, q[j], smap, S);
-          all = all && q[j].done;
-        }
-        if (__all_sync(0xffffffffu, all)) break;
       }
     }
-#pragma unroll
-    for (int j = 0; j < COLS; ++j)
-      if (col0 + 32 * j < W) {
-        const Hit h = hit_of<MAPK>(p, e, q[j], col0 + 32 * j, ws);
-        if (!kDefer) {
-          finish_column<MODE>(p, e, h, ws);
-          continue;
-        }
-        if (pending) finish_column<MODE>(p, e, last, ws);
-        last = h;
-        pending = true;
-      }
   }
-  if (kDefer && pending) finish_column<MODE>(p, e, last, ws);
+  if (kDefer && pending) {
+    const int m = (W - 1 - lane) >> 5;  // the lane's last column
+    finish_column<MODE>(p, e, last, lane + 32 * m, slot0 + 8 * m, ws);
+  }
   __syncwarp();
+  return far;
 }
 
 // Project sprites (lane j takes sprite j) and order the visible ones far to
 // near (equal depths: higher index first, so the lower index is drawn last).
 // A sprite at depth ty is 0.25 W / (tan(fov/2) ty) columns wide, centred on
 // column (W/2)(1 + tx/ty), and (H/2) / ty rows high from row H/2 down.
+// `far` is the lane's largest column depth: a sprite at or beyond the frame's
+// largest depth covers no pixel, and in mazes and rooms nearly all are, so
+// most frames end at the first ballot.
 __device__ __forceinline__ int project_sprites(const Params& p, const Env& r, float c, float s, const WarpSmem& ws,
-                                               int lane) {
+                                               int lane, float far) {
   const int W = p.W, H = p.H;
   bool vis = false;
-  float ty = 0.f;
-  int cA = 0, cB = -1;
+  float ty = 0.f, vx = 0.f, vy = 0.f;
+  int cA = 0, cB = -1, type = 0;
   const int nspr = ws.obj(p)[6];
+  if (nspr == 0) return 0;
+  // depths are never negative, so their bits order like the values
+  const float deepest = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(far)));
   if (lane < nspr) {
     const float4 sp = ws.spr_in(p)[lane];
-    const int type = (int)sp.z;
-    const float vx = (sp.x - (float)r.cx) - r.fx;
-    const float vy = (sp.y - (float)r.cy) - r.fy;
+    type = (int)sp.z;
+    vx = (sp.x - (float)r.cx) - r.fx;
+    vy = (sp.y - (float)r.cy) - r.fy;
     ty = fmaf(vx, c, vy * s);
+    vis = type != 0 && ty > 0.1f && ty < deepest;
+  }
+  if (!__any_sync(0xffffffffu, vis)) return 0;
+  if (vis) {
+    vis = false;
     const int kc = key_colour(type);
-    if (type != 0 && !(kc >= 0 && ((r.keys >> kc) & 1)) && ty > 0.1f) {
+    if (!(kc >= 0 && ((r.keys >> kc) & 1))) {
       // 1/ty within an ulp or two: pixel positions move by far less than the
       // 1e-3 pixel the silhouette-edge tolerance allows
       const float inv_ty = __fdividef(1.f, ty);
@@ -1753,15 +1804,17 @@ __device__ __forceinline__ void fill_block(const Params& p, const WarpSmem& ws, 
 template <int MODE, int MAPK, int COLS, int GRAY>
 __device__ __forceinline__ void render_env(const Params& p, int e, const Env& r, float c, float s,
                                            const WarpSmem& ws, int lane, int& slot, uint8_t* frame, float2 k01) {
-  cast_columns<MODE, MAPK, COLS>(p, e, r, c, s, ws, lane, k01);
+  const float far = cast_columns<MODE, MAPK, COLS>(p, e, r, c, s, ws, lane, k01);
   if (MODE == MODE_RAYS) return;
-  const int nvis = project_sprites(p, r, c, s, ws, lane);  // ends with __syncwarp
+  const int nvis = project_sprites(p, r, c, s, ws, lane, far);  // ends with __syncwarp when any is visible
   const int H = p.H, W = p.W, rowb = 3 * W;
-  if (lane < nvis) {  // rows each sprite of the far-to-near order can cover
-    const int4 rc = ws.spr_rect(p)[ws.order(p)[lane]];
-    ws.spr_span(p)[lane] = rc.x <= rc.y ? ((uint32_t)rc.z << 16) | (uint32_t)rc.w : 0xFFFF0000u;
+  if (nvis > 0) {  // rows each sprite of the far-to-near order can cover
+    if (lane < nvis) {
+      const int4 rc = ws.spr_rect(p)[ws.order(p)[lane]];
+      ws.spr_span(p)[lane] = rc.x <= rc.y ? ((uint32_t)rc.z << 16) | (uint32_t)rc.w : 0xFFFF0000u;
+    }
+    __syncwarp();
   }
-  __syncwarp();
   const bool gray_on = GRAY == 1 || (GRAY == 2 && p.st.gray != nullptr);
   for (int r0 = 0; r0 < H; r0 += p.rows_per_block) {
     const int r1 = r0 + p.rows_per_block < H ? r0 + p.rows_per_block : H;
@@ -1899,7 +1952,7 @@ __device__ __forceinline__ bool stage_prefetched(const Params& p, const WarpSmem
   if (lane < p.K) ws.spr_in(p)[lane] = q.spr;
   if (!small_map<MAPK>(p)) {
     if (!stage<MAPK>(p, e, ws.map(p), lane)) return false;  // ends with __syncwarp
-    mark_border<MAPK>(p, ws, q.r.cx, q.r.cy, lane);
+    mark_border<MAPK>(p, ws, lane);
     return true;
   }
   const int n = p.S * p.S;
@@ -1909,10 +1962,8 @@ __device__ __forceinline__ bool stage_prefetched(const Params& p, const WarpSmem
                        nonzero4(q.m1.w) << 28;
     if (lane < (n >> 5)) reinterpret_cast<uint32_t*>(ws.map(p))[lane] = w;
     if (p.S == 32) {  // word `lane` is row `lane`: its end cells, and all of rows 0 and 31, solid
-      const int S = 32, cx = q.r.cx, cy = q.r.cy;
-      const bool row_ok = (w & 0x80000001u) == 0x80000001u && ((lane != 0 && lane != S - 1) || w == 0xffffffffu);
-      const bool ok = __all_sync(0xffffffffu, row_ok) && p.task != kTaskAscii && cx > 0 && cy > 0 && cx < S - 1 &&
-                      cy < S - 1;
+      const bool row_ok = (w & 0x80000001u) == 0x80000001u && ((lane != 0 && lane != 31) || w == 0xffffffffu);
+      const bool ok = __all_sync(0xffffffffu, row_ok);
       if (lane == 0) ws.obj(p)[7] = ok ? 1 : 0;
       __syncwarp();
       return true;
@@ -1923,7 +1974,7 @@ __device__ __forceinline__ bool stage_prefetched(const Params& p, const WarpSmem
     if (lane + 32 < (n >> 4)) dst[lane + 32] = q.m1;
   }
   __syncwarp();
-  mark_border<MAPK>(p, ws, q.r.cx, q.r.cy, lane);
+  mark_border<MAPK>(p, ws, lane);
   return true;
 }
 
@@ -1951,7 +2002,7 @@ __device__ __forceinline__ void next_episode(const Params& p, int e, Env& r, con
   load_objects(p, ws, e, lane);
   __syncwarp();
   heading(p, r, c, s);
-  mark_border<MAPK>(p, ws, r.cx, r.cy, lane);
+  mark_border<MAPK>(p, ws, lane);
 }
 
 // Everything one launch does for env e: MODE_ROLLOUT runs the launch's steps
@@ -1968,7 +2019,7 @@ __device__ __forceinline__ bool run_env(const Params& p, int e, uint8_t* wbase, 
     const Env r = load_env(p, e);
     load_objects(p, ws, e, lane);
     __syncwarp();
-    mark_border<MAPK>(p, ws, r.cx, r.cy, lane);
+    mark_border<MAPK>(p, ws, lane);
     float c, s;
     heading(p, r, c, s);
     render_env<MODE, MAPK, COLS, GRAY>(p, e, r, c, s, ws, lane, slot, p.frames + (size_t)e * frame_bytes,
@@ -1981,7 +2032,7 @@ __device__ __forceinline__ bool run_env(const Params& p, int e, uint8_t* wbase, 
   if (!stage_prefetched<MAPK>(p, ws, e, q, lane)) return false;  // ends with __syncwarp
   if (r.keys != 0) {  // doors of held keys open: the border flag again
     open_doors<MAPK>(p, e, r.keys, ws, lane);
-    mark_border<MAPK>(p, ws, r.cx, r.cy, lane);
+    mark_border<MAPK>(p, ws, lane);
   }
   if (MODE == MODE_ROLLOUT) {
     int a_next = q.action;
@@ -1997,7 +2048,7 @@ __device__ __forceinline__ bool run_env(const Params& p, int e, uint8_t* wbase, 
         next_episode<MAPK>(p, e, r, ws, scratch, lane, c, s);
       if (__builtin_expect(r.keys != keys0, 0)) {
         open_doors<MAPK>(p, e, r.keys, ws, lane);
-        mark_border<MAPK>(p, ws, r.cx, r.cy, lane);
+        mark_border<MAPK>(p, ws, lane);
       }
       render_env<MODE, MAPK, COLS, GRAY>(p, e, r, c, s, ws, lane, slot,
                                          p.frames + (size_t)t * p.frame_step + (size_t)e * frame_bytes, q.k01);
@@ -2026,7 +2077,7 @@ __device__ __forceinline__ bool run_env(const Params& p, int e, uint8_t* wbase, 
       next_episode<MAPK>(p, e, r, ws, scratch, lane, c, s);
     else if (r.keys != keys0) {
       open_doors<MAPK>(p, e, r.keys, ws, lane);
-      mark_border<MAPK>(p, ws, r.cx, r.cy, lane);
+      mark_border<MAPK>(p, ws, lane);
     }
   } else {
     heading(p, r, c, s);

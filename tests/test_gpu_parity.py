@@ -690,6 +690,32 @@ def test_unlocked_door_opens_when_bumped():
     stats.check()
 
 
+def test_unlocked_door_on_the_border_opens_the_map():
+    """An unlocked door in the border of the grid: the border is solid until it
+    is bumped, then rays leave the map through it and the agent walks onto it,
+    in lockstep with the oracle, and as one rollout."""
+    row = "#.............." + '"'
+    run = _corridor("################\n" + row + "\n" + "#" * 16)
+    start = run.env.get_state()
+    run.env.fields(start)["cell_x"][:] = 13
+    run.env.set_state(start)
+    stats = Stats()
+    forward = lambda seed, step, n: np.ones(n, np.uint8)  # noqa: E731
+    lockstep(run, stats, 30, seed=0, action_fn=forward)
+    stats.check()
+    end = run.env.get_state()
+    f = run.env.fields(end)
+    assert (f["map"][:, 1, 15] == 0).all() and (f["cell_x"] == 15).all()
+    n, T = run.env.n, 30
+    run.env.set_state(start)
+    frames = torch.zeros((T, n) + tuple(run.frames.shape[1:]), dtype=torch.uint8, device=run.dev)
+    rewards = torch.zeros((T, n), dtype=torch.float32, device=run.dev)
+    dones = torch.zeros((T, n), dtype=torch.uint8, device=run.dev)
+    run.env.rollout(torch.ones((T, n), dtype=torch.uint8, device=run.dev), frames, rewards, dones)
+    torch.cuda.synchronize()
+    assert torch.equal(frames[-1], run.frames) and (run.env.get_state() == end).all()
+
+
 def test_late_handoff_is_reported_and_later_rollouts_exact():
     """With the hand-off wait limit at 0 polls every hand-off of a chunked
     rollout counts as late: the launch still ends, the device error word says
