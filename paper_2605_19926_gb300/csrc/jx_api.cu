@@ -279,7 +279,7 @@ namespace {
 
 // jx_create / jx_env_bytes / jx_create_in. Everything that does not need
 // device memory is decided first (layout, tables, launch shape); then the
-// env's one device block (state | aux | maze scratch) is allocated, or placed
+// env's one device block (state | aux | bit planes | maze scratch) is allocated, or placed
 // in the caller's memory `ext`. With `bytes_only` the block size is returned
 // in *bytes and nothing is kept.
 jx_status create_impl(const jx_config* cfg, int device, void* ext, size_t ext_bytes, bool bytes_only, size_t* bytes,
@@ -347,6 +347,8 @@ jx_status create_impl(const jx_config* cfg, int device, void* ext, size_t ext_by
   // blocks beat double buffering at the same shared memory. The map is held
   // as a bit plane when that buys fewer row blocks per frame (the smaller map
   // leaves room for more rows), and always at side 128 (2 KB instead of 16 KB).
+  p.pitch_shift = jx::plane_pitch_shift(c.map_side);
+  p.plane_words = jx::plane_words(c.map_side);
   p.gray = c.gray_stack != 0;
   p.shading = c.shading != 0;
   p.out_stride = c.n_envs;
@@ -401,8 +403,10 @@ jx_status create_impl(const jx_config* cfg, int device, void* ext, size_t ext_by
   p.gen_scratch_stride = jx::gen_scratch_bytes(c.task, c.map_side);
   const size_t scratch_bytes = p.gen_scratch_stride * (size_t)env->grid * jx::kWarpsPerBlock;
 
-  // the device block: state | aux | scratch
-  const size_t off_aux = align256(env->state_bytes), off_scratch = off_aux + aux_bytes;
+  // the device block: state | aux | bit planes of the maps | scratch
+  const size_t plane_bytes = 4 * (size_t)p.plane_words * c.n_envs;
+  const size_t off_aux = align256(env->state_bytes), off_plane = off_aux + aux_bytes;
+  const size_t off_scratch = off_plane + align256(plane_bytes);
   const size_t total = off_scratch + align256(scratch_bytes);
   if (bytes) *bytes = total;
   if (bytes_only) {
@@ -437,10 +441,12 @@ jx_status create_impl(const jx_config* cfg, int device, void* ext, size_t ext_by
   env->state = env->mem;
   env->aux = env->mem + off_aux;
   env->scratch = scratch_bytes ? env->mem + off_scratch : nullptr;
-  if ((err = cudaMemset(env->state, 0, env->state_bytes)) != cudaSuccess) {
+  if ((err = cudaMemset(env->state, 0, env->state_bytes)) != cudaSuccess ||
+      (err = cudaMemset(env->mem + off_plane, 0, plane_bytes)) != cudaSuccess) {
     jx_destroy(env);
     return cuda_fail(err, "cudaMemset of the state");
   }
+  p.plane = reinterpret_cast<uint32_t*>(env->mem + off_plane);
   {
     // per-env constant tables, computed in double and rounded once
     std::string host(aux_bytes, '\0');
@@ -950,6 +956,7 @@ jx_status jx_set_state(jx_env* env, const void* h_buf, size_t bytes) {
   DeviceGuard g(env->device);
   cudaError_t err = cudaDeviceSynchronize();
   if (err == cudaSuccess) err = cudaMemcpy(env->state, blob.data(), bytes, cudaMemcpyHostToDevice);
+  if (err == cudaSuccess) err = jx::plane_launch(env->base, 0);
   if (err == cudaSuccess) err = cudaDeviceSynchronize();
   return err == cudaSuccess ? JX_OK : cuda_fail(err, "set_state");
 }

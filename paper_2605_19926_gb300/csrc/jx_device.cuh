@@ -381,20 +381,32 @@ __device__ __forceinline__ uint32_t nonzero4(uint32_t x) {
   return (m * 0x10204080u) >> 28;  // gathers bits 0, 8, 16, 24 into bits 28..31
 }
 
-// The map as a bit plane: bit i of word i / 32 is set iff cell i is nonzero
-// (S * S is a multiple of 32; rows run on across word boundaries).
-// The bytes are read from `src` (16-byte aligned; the state block's map when null).
-__device__ __forceinline__ void stage_map_bits(const Params& p, int e, uint8_t* smap, int lane,
-                                               const uint8_t* src = nullptr) {
-  const int words = (p.S * p.S) >> 5;
-  const uint4* g = reinterpret_cast<const uint4*>(src ? src : p.st.map + (size_t)e * p.S * p.S);
-  uint32_t* w = reinterpret_cast<uint32_t*>(smap);
-  for (int i = lane; i < words; i += 32) {
-    const uint4 a = g[2 * i], b = g[2 * i + 1];
-    w[i] = nonzero4(a.x) | nonzero4(a.y) << 4 | nonzero4(a.z) << 8 | nonzero4(a.w) << 12 | nonzero4(b.x) << 16 |
+// The map as a bit plane: bit x & 31 of word y * pitch / 32 + x / 32 is set iff
+// cell (x, y) is nonzero; rows are padded to a pitch of 32, 64 or 128 cells
+// (the bits beyond S are unused). Every env keeps its plane in device memory
+// beside the state (Params::plane), written with the map, so that a launch
+// stages 1 bit a cell: a step of 16,384 rooms of sides 16 to 128 read 90 MB of
+// map bytes before and packed them (157 us; 141 with the planes), and an 8-step
+// rollout of 16,384 envs of side 128 took 1.73 ms (1.64 with the planes).
+__device__ __forceinline__ uint32_t* plane_of(const Params& p, int e) {
+  return p.plane + (size_t)e * p.plane_words;
+}
+
+// Plane word i (of a row's pitch / 32) from the map bytes at src.
+__device__ __forceinline__ uint32_t plane_word(const Params& p, const uint8_t* src, int i) {
+  const int S = p.S, sh = p.pitch_shift - 5;  // words per row: 1 << sh
+  const int y = i >> sh, x = (i & ((1 << sh) - 1)) << 5;
+  if (y >= S) return 0u;  // padding of the last 16 bytes
+  const uint8_t* q = src + y * S + x;
+  if ((S & 31) == 0) {  // 16-byte aligned rows
+    const uint4 a = reinterpret_cast<const uint4*>(q)[0], b = reinterpret_cast<const uint4*>(q)[1];
+    return nonzero4(a.x) | nonzero4(a.y) << 4 | nonzero4(a.z) << 8 | nonzero4(a.w) << 12 | nonzero4(b.x) << 16 |
            nonzero4(b.y) << 20 | nonzero4(b.z) << 24 | nonzero4(b.w) << 28;
   }
-  __syncwarp();
+  uint32_t w = 0;
+  const int n = S - x < 32 ? S - x : 32;
+  for (int k = 0; k < n; ++k) w |= (q[k] != 0 ? 1u : 0u) << k;
+  return w;
 }
 
 template <int MAPK>
@@ -402,18 +414,42 @@ __device__ __forceinline__ bool map_bits(const Params& p) {
   return MAPK == MAP_BITS || (MAPK == MAP_RUNTIME && p.map_bits != 0);
 }
 
-// cell i of the staged map blocks movement and rays (in bit mode the door's
-// bit is cleared while the key is held, see open_door)
+// Cells from one row of the staged map to the next.
+template <int MAPK>
+__device__ __forceinline__ int map_pitch(const Params& p) {
+  return map_bits<MAPK>(p) ? 1 << p.pitch_shift : p.S;
+}
+
+// cell i (y * pitch + x) of the staged map blocks movement and rays (in bit
+// mode the door's bit is cleared while the key is held, see open_doors)
 template <int MAPK>
 __device__ __forceinline__ bool cell_set(const Params& p, const uint8_t* smap, int i) {
   if (map_bits<MAPK>(p)) return (reinterpret_cast<const uint32_t*>(smap)[i >> 5] >> (i & 31)) & 1u;
   return smap[i] != 0;
 }
 
+// A new map's plane from its bytes at src: into device memory, and with
+// bit-plane maps into the warp's shared memory too.
+template <int MAPK>
+__device__ __forceinline__ void write_plane(const Params& p, int e, const uint8_t* src, uint8_t* smap, int lane) {
+  uint32_t* g = plane_of(p, e);
+  uint32_t* w = reinterpret_cast<uint32_t*>(smap);
+  for (int i = lane; i < p.plane_words; i += 32) {
+    const uint32_t v = plane_word(p, src, i);
+    g[i] = v;
+    if (map_bits<MAPK>(p)) w[i] = v;
+  }
+  __syncwarp();
+}
+
 template <int MAPK>
 __device__ __forceinline__ bool stage(const Params& p, int e, uint8_t* smap, int lane) {
   if (map_bits<MAPK>(p)) {
-    stage_map_bits(p, e, smap, lane);
+    const uint4* g = reinterpret_cast<const uint4*>(plane_of(p, e));
+    uint4* w = reinterpret_cast<uint4*>(smap);
+#pragma unroll 4
+    for (int i = lane; i < (p.plane_words >> 2); i += 32) w[i] = g[i];
+    __syncwarp();
     return true;
   }
   return stage_map(p, e, smap, lane);
@@ -1062,7 +1098,7 @@ __device__ __noinline__ void take_next(const Params& p, int e, uint32_t ep, uint
     st.spr_type[i] = nx.spr_type[i];
   }
   __syncwarp();
-  if (map_bits<MAPK>(p)) stage_map_bits(p, e, ws.map(p), lane, p.nx.map + (size_t)e * n);
+  write_plane<MAPK>(p, e, p.nx.map + (size_t)e * n, ws.map(p), lane);
 }
 
 // ASCII maps (Table 2): each episode copies the parsed map; the spawn is
@@ -1153,14 +1189,14 @@ __device__ __forceinline__ void generate(const Params& p, int e, uint32_t ep, ui
   } else {
     gen_maze(p, e, ep, smap, work_in_ring ? ws.ring() : scratch, lane);
   }
-  if (bits) stage_map_bits(p, e, ws.map(p), lane, map_in_ring ? smap : nullptr);
+  write_plane<MAPK>(p, e, smap, ws.map(p), lane);
 }
 
 // ------------------------------------------------------------------ step ----
 template <int MAPK>
 __device__ __forceinline__ bool solid(const Params& p, const uint8_t* smap, int S, int x, int y, int keys) {
   if (x < 0 || y < 0 || x >= S || y >= S) return true;
-  if (map_bits<MAPK>(p)) return cell_set<MAPK>(p, smap, y * S + x);
+  if (map_bits<MAPK>(p)) return cell_set<MAPK>(p, smap, (y << p.pitch_shift) + x);
   int v = smap[y * S + x];
   return v != 0 && !(is_locked(v) && ((keys >> (v - kLocked)) & 1));
 }
@@ -1216,8 +1252,10 @@ __device__ __noinline__ void open_unlocked(const Params& p, int e, uint8_t* smap
       if (!is_unlocked(map_bits<MAPK>(p) ? g[c] : smap[c])) continue;
       if (lane == 0) {
         g[c] = 0;
+        const int b = (j << p.pitch_shift) + i;
+        plane_of(p, e)[b >> 5] &= ~(1u << (b & 31));
         if (map_bits<MAPK>(p))
-          reinterpret_cast<uint32_t*>(smap)[c >> 5] &= ~(1u << (c & 31));
+          reinterpret_cast<uint32_t*>(smap)[b >> 5] &= ~(1u << (b & 31));
         else
           smap[c] = 0;
       }
@@ -1382,12 +1420,12 @@ __device__ __forceinline__ void ray_cross(Ray& q, int& cell, int step_x, int ste
 // staged map or the keys change, and cleared when an unlocked door opens.
 template <int MAPK>
 __device__ __forceinline__ void mark_border(const Params& p, const WarpSmem& ws, int lane) {
-  const int S = p.S;
+  const int S = p.S, pitch = map_pitch<MAPK>(p);
   const uint8_t* smap = ws.map(p);
   bool ok = true;
   for (int i = lane; i < S; i += 32)
-    ok = ok && cell_set<MAPK>(p, smap, i) && cell_set<MAPK>(p, smap, (S - 1) * S + i) &&
-         cell_set<MAPK>(p, smap, i * S) && cell_set<MAPK>(p, smap, i * S + S - 1);
+    ok = ok && cell_set<MAPK>(p, smap, i) && cell_set<MAPK>(p, smap, (S - 1) * pitch + i) &&
+         cell_set<MAPK>(p, smap, i * pitch) && cell_set<MAPK>(p, smap, i * pitch + S - 1);
   ok = __all_sync(0xffffffffu, ok);
   if (lane == 0) ws.obj(p)[7] = ok ? 1 : 0;
   __syncwarp();
@@ -1415,9 +1453,9 @@ struct Hit {
 template <int MODE, int MAPK, int COLS>
 __device__ __forceinline__ void march(const Params& p, int e, const Env& r, Ray (&q)[COLS], Hit (&h)[COLS],
                                       const WarpSmem& ws, bool inside, const bool (&valid)[COLS]) {
-  const int S = p.S;
+  const int S = p.S, pitch = map_pitch<MAPK>(p);
   const uint8_t* smap = ws.map(p);
-  const int cell0 = r.cy * S + r.cx;
+  const int cell0 = r.cy * pitch + r.cx;
   int cell[COLS];
   bool out[COLS], none[COLS];
 #pragma unroll
@@ -1428,7 +1466,7 @@ __device__ __forceinline__ void march(const Params& p, int e, const Env& r, Ray 
   }
   if (MODE != MODE_RAYS && inside) {
     if (COLS == 1) {
-      const int sy = q[0].sy * S;
+      const int sy = q[0].sy * pitch;
       if (valid[0])
         do ray_cross(q[0], cell[0], q[0].sx, sy);
         while (!cell_set<MAPK>(p, smap, cell[0]));
@@ -1440,7 +1478,7 @@ __device__ __forceinline__ void march(const Params& p, int e, const Env& r, Ray 
 #pragma unroll
         for (int j = 0; j < COLS; ++j)
           if ((left >> j) & 1u) {
-            ray_cross(q[j], cell[j], q[j].sx, q[j].sy * S);
+            ray_cross(q[j], cell[j], q[j].sx, q[j].sy * pitch);
             if (cell_set<MAPK>(p, smap, cell[j])) left &= ~(1u << j);
           }
       }
@@ -1457,10 +1495,10 @@ __device__ __forceinline__ void march(const Params& p, int e, const Env& r, Ray 
         mx += q[j].tx ? q[j].sx : 0;
         my += q[j].tx ? 0 : q[j].sy;
         out[j] = (unsigned)mx >= (unsigned)S || (unsigned)my >= (unsigned)S;
-        hit = out[j] || cell_set<MAPK>(p, smap, my * S + mx);
+        hit = out[j] || cell_set<MAPK>(p, smap, my * pitch + mx);
       }
       none[j] = !hit;
-      cell[j] = my * S + mx;
+      cell[j] = my * pitch + mx;
       h[j].mx = mx;
       h[j].my = my;
     }
@@ -1474,7 +1512,9 @@ __device__ __forceinline__ void march(const Params& p, int e, const Env& r, Ray 
     h[j].none = none[j];
     h[j].v = 1;
     if (!out[j] && !none[j] && valid[j])
-      h[j].v = map_bits<MAPK>(p) ? p.st.map[(size_t)e * S * S + cell[j]] : smap[cell[j]];
+      h[j].v = map_bits<MAPK>(p)  // the byte map has no row padding
+                   ? p.st.map[(size_t)e * S * S + cell[j] - (cell[j] >> p.pitch_shift) * (pitch - S)]
+                   : smap[cell[j]];
   }
 }
 
@@ -1862,17 +1902,20 @@ __device__ __noinline__ void open_doors(const Params& p, int e, int keys, const 
     for (int i = lane; i < n; i += 32) {
       const int v = map_bits<MAPK>(p) ? g[i] : smap[i];
       if (!(is_locked(v) && ((keys >> (v - kLocked)) & 1))) continue;
-      if (map_bits<MAPK>(p))
-        atomicAnd(reinterpret_cast<uint32_t*>(smap) + (i >> 5), ~(1u << (i & 31)));
-      else
+      if (map_bits<MAPK>(p)) {
+        const int b = ((i / S) << p.pitch_shift) + i % S;
+        atomicAnd(reinterpret_cast<uint32_t*>(smap) + (b >> 5), ~(1u << (b & 31)));
+      } else {
         smap[i] = 0;
+      }
     }
   } else if (keys & 1) {
     const int2 door = *reinterpret_cast<const int2*>(ws.obj(p) + 4);
     if (lane == 0 && door.x >= 0 && door.y >= 0 && door.x < S && door.y < S) {
       const int i = door.y * S + door.x;
       if (map_bits<MAPK>(p)) {
-        if (g[i] == kDoor) reinterpret_cast<uint32_t*>(smap)[i >> 5] &= ~(1u << (i & 31));
+        const int b = (door.y << p.pitch_shift) + door.x;
+        if (g[i] == kDoor) reinterpret_cast<uint32_t*>(smap)[b >> 5] &= ~(1u << (b & 31));
       } else if (smap[i] == kDoor) {
         smap[i] = 0;
       }
@@ -1884,8 +1927,8 @@ __device__ __noinline__ void open_doors(const Params& p, int e, int keys, const 
 // What a launch reads of env e before its first step, fetched in one round of
 // independent loads so that their latencies overlap: the scalar state, the
 // key / goal / door cells and sprite count (lanes 0..6), the sprite slots
-// (lane j: slot j), the map when it holds at most 1 KB (two 16-byte chunks a
-// lane), the first action, the column table's first two entries of the lane,
+// (lane j: slot j), the map when it is a plane of at most 32 words (one a lane)
+// or holds at most 1 KB (two 16-byte chunks a lane), the first action, the column table's first two entries of the lane,
 // and for the single step the turn table's entries lane, 32 + lane and
 // 64 + lane (tables of at most 96 turns).
 struct Prefetch {
@@ -1900,6 +1943,7 @@ struct Prefetch {
 
 template <int MAPK>
 __device__ __forceinline__ bool small_map(const Params& p) {
+  if (map_bits<MAPK>(p)) return p.plane_words <= 32;  // a word a lane
   const int n = p.S * p.S;
   return n <= 1024 && (n & 31) == 0;
 }
@@ -1919,11 +1963,8 @@ __device__ __forceinline__ Prefetch prefetch(const Params& p, int e, int t0, int
   if (small_map<MAPK>(p)) {
     const int n = p.S * p.S;
     const uint4* g = reinterpret_cast<const uint4*>(st.map + (size_t)e * n);
-    if (map_bits<MAPK>(p)) {  // word `lane` of the bit plane: cells 32 lane .. 32 lane + 31
-      if (lane < (n >> 5)) {
-        q.m0 = g[2 * lane];
-        q.m1 = g[2 * lane + 1];
-      }
+    if (map_bits<MAPK>(p)) {  // word `lane` of the bit plane
+      if (lane < p.plane_words) q.m0.x = plane_of(p, e)[lane];
     } else {
       if (lane < (n >> 4)) q.m0 = g[lane];
       if (lane + 32 < (n >> 4)) q.m1 = g[lane + 32];
@@ -1957,10 +1998,8 @@ __device__ __forceinline__ bool stage_prefetched(const Params& p, const WarpSmem
   }
   const int n = p.S * p.S;
   if (map_bits<MAPK>(p)) {
-    const uint32_t w = nonzero4(q.m0.x) | nonzero4(q.m0.y) << 4 | nonzero4(q.m0.z) << 8 | nonzero4(q.m0.w) << 12 |
-                       nonzero4(q.m1.x) << 16 | nonzero4(q.m1.y) << 20 | nonzero4(q.m1.z) << 24 |
-                       nonzero4(q.m1.w) << 28;
-    if (lane < (n >> 5)) reinterpret_cast<uint32_t*>(ws.map(p))[lane] = w;
+    const uint32_t w = q.m0.x;
+    if (lane < p.plane_words) reinterpret_cast<uint32_t*>(ws.map(p))[lane] = w;
     if (p.S == 32) {  // word `lane` is row `lane`: its end cells, and all of rows 0 and 31, solid
       const bool row_ok = (w & 0x80000001u) == 0x80000001u && ((lane != 0 && lane != 31) || w == 0xffffffffu);
       const bool ok = __all_sync(0xffffffffu, row_ok);

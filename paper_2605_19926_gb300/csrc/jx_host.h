@@ -19,7 +19,7 @@ struct jx_env {
   int grid_handoff = 0;  // blocks of a rollout launch in hand-off chunks (see rollout_chunk)
   int smem_block = 0;
   jx::Params base{};
-  // one device block: state | aux | scratch (owned, or in the caller's memory)
+  // one device block: state | aux | bit planes | scratch (owned, or in the caller's memory)
   uint8_t* mem = nullptr;
   size_t mem_bytes = 0;
   bool owns_mem = true;

@@ -70,6 +70,8 @@ struct State {
 
 struct Params {
   State st;
+  uint32_t* plane;  // [n][plane_words] the maps as bit planes, rows padded to a pitch of 1 << pitch_shift cells
+  int32_t plane_words, pitch_shift;
   uint32_t* err;          // device error word
   const float2* turn_cs;  // [turns_per_rev] (cos, sin) of turn * 2 pi / turns_per_rev
   const float* col_k;     // [W] (2 (c + 1/2) / W - 1) * tan(fov / 2)
@@ -125,7 +127,7 @@ struct Params {
   int32_t rows_per_block;  // rows per staged frame block
   int32_t staging;         // staging buffers per warp (1: each block waits for the last one's copy-out)
   int32_t frame_block_bytes;
-  int32_t map_smem_bytes;  // S * S rounded up to 16
+  int32_t map_smem_bytes;  // of the staged map, rounded up to 16
   // per-warp shared memory layout (byte offsets from the warp's base; set by layout_warp_smem)
   int32_t off_gray, off_pal, off_map, off_col_rgb, off_col_top, off_col_bot, off_zbuf, off_spr_in, off_spr_a, off_spr_rect,
       off_spr_ty, off_spr_rgb, off_spr_kind, off_order, off_spr_span, off_obj, warp_bytes;
@@ -150,6 +152,11 @@ void layout_warp_smem(Params& p);
 // Dynamic shared memory bytes of one block.
 int block_smem_bytes(const Params& p);
 size_t gen_scratch_bytes(int task, int S);
+// Bit planes of maps of side S: log2 of the row pitch in cells, words per map (a multiple of 4).
+inline int plane_pitch_shift(int S) { return S <= 32 ? 5 : (S <= 64 ? 6 : 7); }
+inline int plane_words(int S) { return ((S << (plane_pitch_shift(S) - 5)) + 3) & ~3; }
+// Rebuild every env's bit plane from the state's map bytes (after the state was replaced).
+cudaError_t plane_launch(const Params& p, cudaStream_t stream);
 // Lane-parallel pre-generation: for maze tasks of side >= kPregenMinSide (a
 // multiple of 4), one lane per env advances the build of the env's next
 // episode (reset: episode 0) into p.nx by its share of the launches left

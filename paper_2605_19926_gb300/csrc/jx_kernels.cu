@@ -115,6 +115,16 @@ __global__ void __launch_bounds__(kThreads, kMinBlocksPerSm / kWarpsPerBlock)
   if (lane == 0) bulk_wait_read_all();
 }
 
+// One plane word a thread.
+__global__ void __launch_bounds__(256) plane_kernel(const __grid_constant__ Params p) {
+  const int64_t items = (int64_t)p.n * p.plane_words;
+  for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < items;
+       idx += (int64_t)gridDim.x * blockDim.x) {
+    const int e = (int)(idx / p.plane_words), i = (int)(idx % p.plane_words);
+    p.plane[idx] = plane_word(p, p.st.map + (size_t)e * p.S * p.S, i);
+  }
+}
+
 // Whether env e needs a pre-built episode, and which: episode 0 at a reset,
 // else the one after its current episode (with a horizon, which bounds when it
 // starts), unless the next-episode block holds it already.
@@ -271,7 +281,7 @@ void layout_warp_smem(Params& p) {
     q += align16(bytes);
     return at;
   };
-  p.map_smem_bytes = align16(p.map_bits ? (p.S * p.S + 7) / 8 : p.S * p.S);
+  p.map_smem_bytes = p.map_bits ? 4 * p.plane_words : align16(p.S * p.S);
   p.off_gray = take(p.staging * p.gray_block_bytes);
   p.off_pal = take(4 * kPaletteWords);
   p.off_map = take(p.map_smem_bytes);
@@ -289,6 +299,12 @@ void layout_warp_smem(Params& p) {
   p.off_spr_span = take(4 * K);
   p.off_obj = take(4 * 8);
   p.warp_bytes = align16(q);
+}
+
+cudaError_t plane_launch(const Params& p, cudaStream_t stream) {
+  const int64_t blocks = ((int64_t)p.n * p.plane_words + 255) / 256;
+  plane_kernel<<<(unsigned)(blocks < 65536 ? blocks : 65536), 256, 0, stream>>>(p);
+  return cudaGetLastError();
 }
 
 int block_smem_bytes(const Params& p) { return p.warp_bytes * kWarpsPerBlock; }

@@ -171,6 +171,26 @@ def test_graph_replay_matches_steps():
     graph.close()
 
 
+@pytest.mark.parametrize("side", [8, 24, 40, 72, 104])
+def test_bit_planes_with_padded_rows(side):
+    """Bit planes hold rows of 32, 64 or 128 cells: sides that do not fill them,
+    in lockstep with the oracle, from a reset and from a state set by the host."""
+    cfgs = [inputs.rooms(n_envs=6, map_side=side, wall_prob=0.2, seed=91, max_sprites=3),
+            inputs.maze_keydoor(n_envs=5, map_side=side, seed=92, horizon=9)]
+    run = BatchRun(cfgs, tiling(2, 1, 8, 16))
+    stats = Stats()
+    batch_check_reset(run, stats)
+    batch_lockstep(run, stats, 12, seed=93, action_fn=forward_biased_actions)
+    for env in run.envs:
+        blob = env.get_state()
+        m = env.fields(blob)["map"]
+        m[:, 1:-1, 1:-1] = m[:, 1:-1, 1:-1].transpose(0, 2, 1).copy()
+        env.fields(blob)["map"][np.arange(env.n), env.fields(blob)["cell_y"], env.fields(blob)["cell_x"]] = 0
+        env.set_state(blob)
+    batch_lockstep(run, stats, 6, seed=94, first_step=12)
+    stats.check()
+
+
 @pytest.mark.parametrize("mode", [0, 1])
 def test_autotune_keeps_fastest_and_resets(mode):
     cfgs = mixed()
