@@ -50,9 +50,9 @@ MIN_RING = 4  # rollout buffer slots at least: 4 x 50 MB frames > L2
 GRAPH_MIN_STEPS = 128  # the per-step graph leg launches at least this many steps (at most 16 x ring)
 SUBMIT_SLACK_CYCLES = 2_000_000  # device-side wait (~1 ms) queued before a timed region's first event
 KERNEL_SOURCES = ["paper_2605_19926_gb300/csrc/jx_device.cuh", "paper_2605_19926_gb300/csrc/jx_kernels.cu",
-                  "paper_2605_19926_gb300/csrc/jx_internal.h"]
+                  "paper_2605_19926_gb300/csrc/jx_rollout.cu", "paper_2605_19926_gb300/csrc/jx_internal.h"]
 BATCH_KERNEL_SOURCES = ["paper_2605_19926_gb300/csrc/jx_device.cuh", "paper_2605_19926_gb300/csrc/jx_batch_kernels.cu",
-                        "paper_2605_19926_gb300/csrc/jx_internal.h"]
+                        "paper_2605_19926_gb300/csrc/jx_rollout.cu", "paper_2605_19926_gb300/csrc/jx_internal.h"]
 # the batched-kernel tiling the large-scale record beside the headline pins
 # (the autotuner's choice on that workload: 2 warps per block, 1 ray per lane,
 # bit planes from side 128, 16-row blocks, one staging buffer)
@@ -542,7 +542,7 @@ def large_record(g: Gpu, n_envs: int, slots: int, steps: int, tiling_text: str, 
     del frames, rewards, dones, acts
     if g.rank != 0:
         return None
-    gray = H * W  # one plane per env-step (all four at an episode start)
+    gray = H * W * min(T, 4) / T  # a launch leaves the planes of its last four frames
     bpes = algorithmic_bytes_per_env_step(cfg) + gray
     peak, peak_src = measured_peak()
     # launches whose steps end episodes (the horizon), against the others

@@ -157,9 +157,10 @@ jx_status jx_create(const jx_config* cfg, int device, jx_env** out);
  * 16 keys, or no floor. */
 jx_status jx_create_ascii(const jx_config* cfg, const char* ascii, int device, jx_env** out);
 
-/* Device bytes jx_create allocates for cfg on `device`: one block holding
- * the state, the per-env tables and the maze work space. Validates cfg like
- * jx_create. */
+/* Device bytes of an env of cfg on `device`: one block holding the state, the
+ * per-env tables, the maps' bit planes and the maze work space (jx_create also
+ * allocates the camera records of its rollouts, at most 24 bytes per env for
+ * 128 steps). Validates cfg like jx_create. */
 jx_status jx_env_bytes(const jx_config* cfg, int device, size_t* bytes);
 
 /* jx_create with the env's device block placed in caller memory d_mem
@@ -204,15 +205,22 @@ jx_status jx_step(jx_env* env, void* stream, const uint8_t* d_actions, uint8_t* 
  * sequence of jx_step calls.
  *  d_actions [steps][N] uint8; d_frames [steps][N][H][W][3] uint8;
  *  d_rewards [steps][N] float32; d_dones [steps][N] uint8.
- * Each env's pose stays in registers and its map in shared memory across the
- * steps. Rollouts of 64 steps or more (envs without a grayscale stack) are cut
- * into chunks of 12 steps that the launch's warps take in turn: a warp that
- * finishes a chunk takes the next free one, of any env, and the chunk after
- * it starts once its env's previous chunk has stored the state (a hand-off
- * through device memory that a late partner cannot stall for more than a
- * bounded wait; bit 2 of the device error word records one that ran out).
+ * Rollouts of 4 steps or more (of envs that jx_create made, except the ASCII
+ * task) run in two passes: a walk steps every agent up to the step that ends
+ * its episode, one lane per env, and leaves a camera record per env and step;
+ * a draw renders the records' frames in any order. The env kernel, launched
+ * last, then runs the envs whose episode ends in the rollout from that step
+ * on. Other rollouts run in the env kernel alone. In the env kernel each env's
+ * pose stays in registers and its map in shared memory across its steps. For
+ * 64 steps or more (envs without a grayscale stack) they are cut into chunks
+ * of 12 steps that the launch's warps take in turn: a warp that finishes a
+ * chunk takes the next free one, of any env, and the chunk after it starts
+ * once its env's previous chunk has stored the state (a hand-off through
+ * device memory that a late partner cannot stall for more than a bounded wait;
+ * bit 2 of the device error word records one that ran out).
  * Asynchronous on `stream`; allocates nothing. steps >= 1. Launches of one
- * env must be ordered on one stream (they share its hand-off words). */
+ * env must be ordered on one stream (they share its hand-off words and camera
+ * records). */
 jx_status jx_rollout(jx_env* env, void* stream, const uint8_t* d_actions, int32_t steps, uint8_t* d_frames,
                      float* d_rewards, uint8_t* d_dones);
 
@@ -331,15 +339,17 @@ jx_status jx_sync_status(jx_env* env, void* stream);
  * (at least 3 x 28 per SM), jx_reset, jx_step and jx_rollout each also launch the three kernels that build episodes ahead (a
  * count, the walls of builds that start, then the build's share of the launch,
  * after a 4-byte cudaMemsetAsync on the same stream; all capturable in a CUDA
- * graph). */
+ * graph). A jx_rollout in two passes (see there) counts its walk and draw
+ * launches and the env kernel's, per 128 steps. */
 jx_status jx_launch_count(const jx_env* env, uint64_t* count);
 
 /* Launch shape of the fused step kernel: grid blocks, threads per block,
  * dynamic shared memory bytes per block. */
 jx_status jx_launch_shape(const jx_env* env, int32_t* grid, int32_t* block, int32_t* smem_bytes);
 
-/* Launch shape of a jx_rollout of `steps` steps: as jx_launch_shape, plus the
- * steps per hand-off chunk (0: every warp runs whole envs). For an env routed
+/* Launch shape of the env kernel in a jx_rollout of `steps` steps (see
+ * jx_rollout): as jx_launch_shape, plus the steps per hand-off chunk (0: every
+ * warp runs whole envs). For an env routed
  * through the batched kernel (jx_autotune), the batch's shape and chunk 0.
  * JX_EINVAL for steps < 1. */
 jx_status jx_rollout_shape(const jx_env* env, int32_t steps, int32_t* grid, int32_t* block, int32_t* smem_bytes,

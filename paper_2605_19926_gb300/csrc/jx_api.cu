@@ -169,15 +169,9 @@ int rollout_chunk(const jx_env* env, int steps) {
   return chunk < steps ? chunk : steps;
 }
 
-jx_status run(jx_env* env, const jx::Params& p, int mode, void* stream) {
-  DeviceGuard g(env->device);
-  if (g.err != cudaSuccess) return cuda_fail(g.err, "cudaSetDevice");
-  cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (jx::pregen_runs(p) && (mode == jx::MODE_STEP || mode == jx::MODE_ROLLOUT || mode == jx::MODE_RESET)) {
-    cudaError_t err = jx::pregen_launch(p, mode == jx::MODE_ROLLOUT ? p.steps : 1, mode == jx::MODE_RESET, s);
-    if (err != cudaSuccess) return cuda_fail(err, "pre-generation launch");
-    env->launches.fetch_add(jx::kPregenKernels, std::memory_order_relaxed);
-  }
+// One launch of the env kernel (MODE_ROLLOUT: in hand-off chunks, of all steps
+// or of what the walk and the draw left).
+jx_status launch_env(jx_env* env, const jx::Params& p, int mode, cudaStream_t s) {
   cudaError_t err = jx::launch(p, mode, mode == jx::MODE_ROLLOUT && p.chunk > 0 ? env->grid_handoff : env->grid, s);
   if (err != cudaSuccess) {
     // a failed rollout launch may leave the hand-off words set (the kernel
@@ -187,6 +181,54 @@ jx_status run(jx_env* env, const jx::Params& p, int mode, void* stream) {
   }
   env->launches.fetch_add(1, std::memory_order_relaxed);
   return JX_OK;
+}
+
+// A rollout of p.steps steps: walk, draw and the env kernel for what they left,
+// in segments that the camera records hold; short ones, and envs without
+// records, in the env kernel alone.
+jx_status run_rollout(jx_env* env, jx::Params p, cudaStream_t s) {
+  const int steps = p.steps;
+  if (!p.stop || steps < jx::kRolloutMinSteps) {
+    p.stop = nullptr;
+    p.chunk = rollout_chunk(env, steps);
+    return launch_env(env, p, jx::MODE_ROLLOUT, s);
+  }
+  const int seg = jx::rollout_segment(env->cfg.n_envs);
+  for (int t = 0; t < steps; t += seg) {
+    const size_t n = (size_t)t * p.out_stride;
+    jx::Params w = p;
+    w.steps = steps - t < seg ? steps - t : seg;
+    w.chunk = rollout_chunk(env, w.steps);
+    w.actions = p.actions + n;
+    w.rewards = p.rewards + n;
+    w.dones = p.dones + n;
+    w.frames = p.frames + (size_t)t * p.frame_step;
+    jx::Params q = env->draw;
+    q.steps = w.steps;
+    q.actions = w.actions;
+    q.frames = w.frames;
+    q.rewards = w.rewards;
+    q.dones = w.dones;
+    int launches = 0;
+    cudaError_t err = jx::rollout_launch(q, env->draw_slots, s, &launches);
+    env->launches.fetch_add(launches, std::memory_order_relaxed);
+    if (err != cudaSuccess) return cuda_fail(err, "rollout launch");
+    if (jx_status st = launch_env(env, w, jx::MODE_ROLLOUT, s)) return st;
+  }
+  return JX_OK;
+}
+
+jx_status run(jx_env* env, const jx::Params& p, int mode, void* stream) {
+  DeviceGuard g(env->device);
+  if (g.err != cudaSuccess) return cuda_fail(g.err, "cudaSetDevice");
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  if (jx::pregen_runs(p) && (mode == jx::MODE_STEP || mode == jx::MODE_ROLLOUT || mode == jx::MODE_RESET)) {
+    cudaError_t err = jx::pregen_launch(p, mode == jx::MODE_ROLLOUT ? p.steps : 1, mode == jx::MODE_RESET, s);
+    if (err != cudaSuccess) return cuda_fail(err, "pre-generation launch");
+    env->launches.fetch_add(jx::kPregenKernels, std::memory_order_relaxed);
+  }
+  if (mode == jx::MODE_ROLLOUT) return run_rollout(env, p, s);
+  return launch_env(env, p, mode, s);
 }
 
 }  // namespace
@@ -408,6 +450,7 @@ jx_status create_impl(const jx_config* cfg, int device, void* ext, size_t ext_by
   const size_t off_aux = align256(env->state_bytes), off_plane = off_aux + aux_bytes;
   const size_t off_scratch = off_plane + align256(plane_bytes);
   const size_t total = off_scratch + align256(scratch_bytes);
+  const bool two_pass = !ext && jx::rollout_wanted(c.task);  // camera records after the block
   if (bytes) *bytes = total;
   if (bytes_only) {
     delete env;
@@ -421,7 +464,17 @@ jx_status create_impl(const jx_config* cfg, int device, void* ext, size_t ext_by
     env->mem = static_cast<uint8_t*>(ext);
     env->owns_mem = false;
   } else {
-    if ((err = cudaMalloc(&env->mem, total)) != cudaSuccess) {
+    // without memory for the camera records, rollouts run in the env kernel alone
+    const size_t cam_bytes = two_pass ? jx::rollout_bytes(c.n_envs) : 0;
+    bool cam = cam_bytes > 0;
+    err = cudaMalloc(&env->mem, total + cam_bytes);
+    if (err != cudaSuccess && cam) {
+      (void)cudaGetLastError();
+      cam = false;
+      err = cudaMalloc(&env->mem, total);
+    }
+    if (err == cudaSuccess && cam) jx::rollout_place(p, env->mem + total);
+    if (err != cudaSuccess) {
       env->mem = nullptr;
       delete env;
       return fail(JX_ENOMEM, "cudaMalloc of %zu env bytes failed: %s", total, cudaGetErrorString(err));
@@ -543,6 +596,16 @@ jx_status create_impl(const jx_config* cfg, int device, void* ext, size_t ext_by
       env->nx_mem = nullptr;
       (void)cudaGetLastError();
     }
+  }
+  if (p.stop) {
+    env->draw = p;
+    jx::rollout_layout(env->draw, prop.sharedMemPerMultiprocessor, prop.reservedSharedMemPerBlock);
+    int b = 0;
+    if ((err = jx::rollout_prepare(env->draw, &b)) != cudaSuccess) {
+      jx_destroy(env);
+      return cuda_fail(err, "occupancy query");
+    }
+    env->draw_slots = (b > 0 ? b : 1) * jx::kWarpsPerBlock * env->num_sms;
   }
   // the memset and the table copy are done before the handle is returned
   if ((err = cudaStreamSynchronize(0)) != cudaSuccess) {
@@ -673,7 +736,6 @@ jx_status jx_rollout(jx_env* env, void* stream, const uint8_t* d_actions, int32_
   p.rewards = d_rewards;
   p.dones = d_dones;
   p.steps = steps;
-  p.chunk = rollout_chunk(env, steps);
   return run(env, p, jx::MODE_ROLLOUT, stream);
 }
 
@@ -807,7 +869,6 @@ jx_status jx_autotune(jx_env* env, void* stream, int32_t mode, int32_t steps, in
         p.actions = base;
         p.frames = frames;
         p.steps = steps;
-        p.chunk = rollout_chunk(env, steps);  // the launch jx_rollout makes
         return run(env, p, jx::MODE_ROLLOUT, s);
       }
       for (size_t k = 0; k < T; ++k) {

@@ -24,6 +24,9 @@ struct jx_batch {
   std::vector<int> order;  // launch order of the groups (indices into envs): largest frames first
   jx_tiling tiling{};
   jx::BatchParams bp{};  // groups in launch order; per-call pointers unset
+  jx::BatchParams draw{};  // the same with the draw pass's layouts (rollouts in two passes)
+  int draw_slots = 0;
+  int segment = 0;  // steps the camera records of every group hold (0: the batched kernel runs rollouts alone)
   int block_smem = 0;
   int grid[5] = {};  // per mode
   uint32_t* queue = nullptr;
@@ -119,6 +122,29 @@ jx_status apply_tiling(jx_batch* b, const jx_tiling& t) {
   return JX_OK;
 }
 
+// The parameters of rollouts in two passes: each group's own layout, the
+// batch's array layout. They do not depend on the tiling.
+jx_status prepare_draw(jx_batch* b) {
+  jx::BatchParams& bq = b->draw;
+  bq.n_groups = (int32_t)b->order.size();
+  for (int i = 0; i < bq.n_groups; ++i) {
+    const jx_env* env = b->envs[b->order[i]];
+    bq.g[i] = env->base.stop ? env->draw : env->base;
+    bq.g[i].out_stride = (int32_t)b->n_total;
+    bq.g[i].frame_step = (size_t)b->frame_total;
+    if (!env->base.stop) continue;
+    bq.warp_bytes = std::max(bq.warp_bytes, env->draw.warp_bytes);
+    const int seg = jx::rollout_segment(env->cfg.n_envs);
+    b->segment = b->segment == 0 ? seg : std::min(b->segment, seg);
+  }
+  if (b->segment == 0) return JX_OK;
+  int blocks = 0;
+  cudaError_t err = jx::batch_rollout_prepare(bq, &blocks);
+  if (err != cudaSuccess) return cuda_fail(err, "occupancy query");
+  b->draw_slots = std::max(1, blocks) * jx::kWarpsPerBlock * b->num_sms;
+  return JX_OK;
+}
+
 jx_status check_batch(const jx_batch* b) {
   if (!b) return fail(JX_EINVAL, "batch is NULL");
   return JX_OK;
@@ -139,12 +165,40 @@ jx_status batch_run(jx_batch* b, int mode, cudaStream_t stream, const uint8_t* a
   }
   DeviceGuard dg(b->device);
   if (dg.err != cudaSuccess) return cuda_fail(dg.err, "cudaSetDevice");
+  // a rollout: the walk and the draw of the steps in segments, then what they
+  // left in the batched kernel
+  if (mode == jx::MODE_ROLLOUT && b->segment > 0 && steps > b->segment) {
+    const size_t N = (size_t)b->n_total, F = (size_t)b->frame_total;
+    for (int32_t t = 0; t < steps; t += b->segment)
+      if (jx_status st = batch_run(b, mode, stream, actions + t * N, frames + t * F, rewards + t * N, dones + t * N,
+                                   std::min(b->segment, steps - t), count))
+        return st;
+    return JX_OK;
+  }
   if (mode == jx::MODE_STEP || mode == jx::MODE_ROLLOUT || mode == jx::MODE_RESET) {
     for (int i = 0; i < bp.n_groups; ++i) {  // groups whose next episodes are built ahead
       if (!jx::pregen_runs(bp.g[i])) continue;
       cudaError_t err = jx::pregen_launch(bp.g[i], mode == jx::MODE_ROLLOUT ? steps : 1, mode == jx::MODE_RESET, stream);
       if (err != cudaSuccess) return cuda_fail(err, "pre-generation launch");
       if (count) b->launches.fetch_add(jx::kPregenKernels, std::memory_order_relaxed);
+    }
+  }
+  if (mode == jx::MODE_ROLLOUT) {
+    if (b->segment > 0 && steps >= jx::kRolloutMinSteps) {
+      jx::BatchParams bq = b->draw;
+      for (int i = 0; i < bp.n_groups; ++i) {
+        bq.g[i].actions = bp.g[i].actions;
+        bq.g[i].frames = bp.g[i].frames;
+        bq.g[i].rewards = bp.g[i].rewards;
+        bq.g[i].dones = bp.g[i].dones;
+        bq.g[i].steps = steps;
+      }
+      int launches = 0;
+      cudaError_t err = jx::batch_rollout_launch(bq, steps, b->draw_slots, stream, &launches);
+      if (count) b->launches.fetch_add(launches, std::memory_order_relaxed);
+      if (err != cudaSuccess) return cuda_fail(err, "batched rollout launch");
+    } else {
+      for (int i = 0; i < bp.n_groups; ++i) bp.g[i].stop = nullptr;
     }
   }
   cudaError_t err = jx::batch_launch(bp, mode, b->tiling.cols_per_lane, b->tiling.warps_per_block, b->grid[mode],
@@ -270,6 +324,10 @@ jx_status jx_batch_create(jx_env* const* groups, int32_t n_groups, const jx_tili
     return cuda_fail(err, "cudaMemset of the work queues");
   }
   if (jx_status st = apply_tiling(b, t)) {
+    jx_batch_destroy(b);
+    return st;
+  }
+  if (jx_status st = prepare_draw(b)) {
     jx_batch_destroy(b);
     return st;
   }

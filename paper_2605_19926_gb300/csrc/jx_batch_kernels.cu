@@ -19,6 +19,17 @@ __global__ void __launch_bounds__(kBatchMaxThreads, kBatchMinBlocks)
   const int wpb = blockDim.x >> 5;
   uint8_t* const wbase = smem_raw + warp * bp.warp_bytes;
   init_warp_header(wbase, lane);
+  if (MODE == MODE_ROLLOUT) {  // after the walk and the draw: only the envs they left
+    uint32_t left = 0u;
+    for (int g = 0; g < bp.n_groups; ++g) {
+      const Params& p = bp.g[g];
+      if (p.stop == nullptr)
+        left = 1u;
+      else
+        for (int i = lane; i < (p.n + 31) >> 5; i += 32) left |= p.ended[i];
+    }
+    if (!__any_sync(0xffffffffu, left != 0u)) return;  // the whole grid
+  }
   const int gw = blockIdx.x * wpb + warp;
   int slot = 0;
   bool fresh = true;  // nothing of an earlier group is pending in the ring
@@ -43,10 +54,13 @@ __global__ void __launch_bounds__(kBatchMaxThreads, kBatchMinBlocks)
       uint32_t next = 0;
       if (lane == 0) next = atomicAdd(bp.queue + g, 1u);
       const int e = (int)ticket;
-      if (SPEC == 1)
-        lost = !run_env<MODE, MAP_BITS, COLS, 0>(p, e, wbase, scratch, lane, slot, 0, p.steps);
+      const int first = MODE == MODE_ROLLOUT && p.stop != nullptr ? p.stop[e] : 0;
+      if (MODE == MODE_ROLLOUT && first >= p.steps)
+        ;  // all of its steps are drawn
+      else if (SPEC == 1)
+        lost = !run_env<MODE, MAP_BITS, COLS, 0>(p, e, wbase, scratch, lane, slot, first, p.steps);
       else
-        lost = !run_env<MODE, MAP_RUNTIME, COLS, 2>(p, e, wbase, scratch, lane, slot, 0, p.steps);
+        lost = !run_env<MODE, MAP_RUNTIME, COLS, 2>(p, e, wbase, scratch, lane, slot, first, p.steps);
       if (lost) break;  // the counters are still cleared below: every warp reaches the end
       ticket = __shfl_sync(0xffffffffu, next, 0);
     }

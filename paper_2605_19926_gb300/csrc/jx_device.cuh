@@ -1263,19 +1263,14 @@ __device__ __noinline__ void open_unlocked(const Params& p, int e, uint8_t* smap
   __syncwarp();
 }
 
-// keep the position split as an integer cell plus a fraction in [0, 1)
+// keep the position split as an integer cell plus a fraction in [0, 1), for f in
+// [-1, 2); a tiny negative fraction that rounds up to 1 becomes 0 in its cell
 __device__ __forceinline__ void renormalise(int& c, float& f) {
-  if (f < 0.f) {
-    f += 1.f;
-    c -= 1;
-    if (f >= 1.f) {  // a tiny negative fraction rounded up to 1
-      f = 0.f;
-      c += 1;
-    }
-  } else if (f >= 1.f) {
-    f -= 1.f;
-    c += 1;
-  }
+  const int d = f >= 1.f ? 1 : (f < 0.f ? -1 : 0);
+  const float g = f >= 1.f ? f - 1.f : (f < 0.f ? f + 1.f : f);
+  const bool up = g >= 1.f;
+  f = up ? 0.f : g;
+  c += up ? 0 : d;
 }
 
 // An action outside 0..6 is recorded in the error word and taken as a no-op;
@@ -1290,6 +1285,44 @@ __device__ __forceinline__ int turn_for(const Params& p, Env& r, int a, int lane
   return a;
 }
 
+// The displacement of action a under heading (c, s). Products and sums here and
+// in try_move are rounded one by one, so that every kernel that steps an agent
+// gets the same bits.
+__device__ __forceinline__ float2 move_delta(int a, float ms, float c, float s) {
+  float dx = 0.f, dy = 0.f;
+  if (a == 1) {
+    dx = __fmul_rn(ms, c);
+    dy = __fmul_rn(ms, s);
+  } else if (a == 2) {
+    dx = -__fmul_rn(ms, c);
+    dy = -__fmul_rn(ms, s);
+  } else if (a == 3) {
+    dx = __fmul_rn(ms, s);
+    dy = -__fmul_rn(ms, c);
+  } else if (a == 4) {
+    dx = -__fmul_rn(ms, s);
+    dy = __fmul_rn(ms, c);
+  }
+  return make_float2(dx, dy);
+}
+
+// One axis of a move by d: taken unless the moved box overlaps a solid cell of
+// mask m (solid3x3 around (ox, oy)). Returns false when it was rejected.
+__device__ __forceinline__ bool try_move_x(Env& r, uint32_t m, int ox, int oy, float d, float rad) {
+  const float nf = __fadd_rn(r.fx, d);
+  if (box_hits(m, ox, oy, r.cx, nf, r.cy, r.fy, rad)) return false;
+  r.fx = nf;
+  renormalise(r.cx, r.fx);
+  return true;
+}
+__device__ __forceinline__ bool try_move_y(Env& r, uint32_t m, int ox, int oy, float d, float rad) {
+  const float nf = __fadd_rn(r.fy, d);
+  if (box_hits(m, ox, oy, r.cx, r.fx, r.cy, nf, rad)) return false;
+  r.fy = nf;
+  renormalise(r.cy, r.fy);
+  return true;
+}
+
 // One step of env e under action a (already checked by turn_for, with the
 // heading (c, s) of the turned agent); the reward and done flag go to output
 // slot `out`. Returns true when the episode ended (the caller regenerates).
@@ -1298,41 +1331,18 @@ template <int MAPK>
 __device__ __forceinline__ bool step_env(const Params& p, int e, Env& r, const uint8_t* smap, const int32_t* obj,
                                          const float4* spr_in, int lane, float c, float s, int a, size_t out,
                                          bool write_state) {
-  const float ms = p.move;
-  float dx = 0.f, dy = 0.f;
-  if (a == 1) {
-    dx = ms * c;
-    dy = ms * s;
-  } else if (a == 2) {
-    dx = -(ms * c);
-    dy = -(ms * s);
-  } else if (a == 3) {
-    dx = ms * s;
-    dy = -(ms * c);
-  } else if (a == 4) {
-    dx = -(ms * s);
-    dy = ms * c;
-  }
+  const float2 d = move_delta(a, p.move, c, s);
   const float rad = p.radius;
   const bool doors = p.task == kTaskAscii;  // maps with unlocked doors
   // both axis tests read the solidity of the cells around the start cell
   const int ox = r.cx, oy = r.cy;
   uint32_t m = solid3x3<MAPK>(p, smap, ox, oy, r.keys, lane);
-  float nfx = r.fx + dx;
-  if (!box_hits(m, ox, oy, r.cx, nfx, r.cy, r.fy, rad)) {
-    r.fx = nfx;
-    renormalise(r.cx, r.fx);
-  } else if (__builtin_expect(doors, 0)) {
-    open_unlocked<MAPK>(p, e, const_cast<uint8_t*>(smap), r.cx, nfx, r.cy, r.fy, lane);
+  if (!try_move_x(r, m, ox, oy, d.x, rad) && __builtin_expect(doors, 0)) {
+    open_unlocked<MAPK>(p, e, const_cast<uint8_t*>(smap), r.cx, __fadd_rn(r.fx, d.x), r.cy, r.fy, lane);
     m = solid3x3<MAPK>(p, smap, ox, oy, r.keys, lane);  // opened doors are floor now
   }
-  float nfy = r.fy + dy;
-  if (!box_hits(m, ox, oy, r.cx, r.fx, r.cy, nfy, rad)) {
-    r.fy = nfy;
-    renormalise(r.cy, r.fy);
-  } else if (__builtin_expect(doors, 0)) {
-    open_unlocked<MAPK>(p, e, const_cast<uint8_t*>(smap), r.cx, r.fx, r.cy, nfy, lane);
-  }
+  if (!try_move_y(r, m, ox, oy, d.y, rad) && __builtin_expect(doors, 0))
+    open_unlocked<MAPK>(p, e, const_cast<uint8_t*>(smap), r.cx, r.fx, r.cy, __fadd_rn(r.fy, d.y), lane);
   // key and goal events from the sprite table (lane j looks at slot j): a key
   // of a colour not held yet on the agent's cell is picked up; a goal there
   // is reached
@@ -1841,9 +1851,12 @@ __device__ __forceinline__ void fill_block(const Params& p, const WarpSmem& ws, 
 #undef JX_QUAD_WORDS
 
 // GRAY: 0 no grayscale stack, 1 a stack, 2 as p.st.gray says (batched kernel).
+// gray_now: this frame's plane is wanted (false only where a later frame of
+// the same launch overwrites it).
 template <int MODE, int MAPK, int COLS, int GRAY>
 __device__ __forceinline__ void render_env(const Params& p, int e, const Env& r, float c, float s,
-                                           const WarpSmem& ws, int lane, int& slot, uint8_t* frame, float2 k01) {
+                                           const WarpSmem& ws, int lane, int& slot, uint8_t* frame, float2 k01,
+                                           bool gray_now = true) {
   const float far = cast_columns<MODE, MAPK, COLS>(p, e, r, c, s, ws, lane, k01);
   if (MODE == MODE_RAYS) return;
   const int nvis = project_sprites(p, r, c, s, ws, lane, far);  // ends with __syncwarp when any is visible
@@ -1855,7 +1868,7 @@ __device__ __forceinline__ void render_env(const Params& p, int e, const Env& r,
     }
     __syncwarp();
   }
-  const bool gray_on = GRAY == 1 || (GRAY == 2 && p.st.gray != nullptr);
+  const bool gray_on = gray_now && (GRAY == 1 || (GRAY == 2 && p.st.gray != nullptr));
   for (int r0 = 0; r0 < H; r0 += p.rows_per_block) {
     const int r1 = r0 + p.rows_per_block < H ? r0 + p.rows_per_block : H;
     uint8_t* buf = ws.ring() + slot * p.frame_block_bytes;

@@ -19,7 +19,10 @@ struct jx_env {
   int grid_handoff = 0;  // blocks of a rollout launch in hand-off chunks (see rollout_chunk)
   int smem_block = 0;
   jx::Params base{};
-  // one device block: state | aux | bit planes | scratch (owned, or in the caller's memory)
+  jx::Params draw{};   // base with the draw pass's shared-memory layout (rollouts in two passes)
+  int draw_slots = 0;  // warps of the draw pass resident at once
+  // one device block: state | aux | bit planes | scratch (owned, or in the
+  // caller's memory), and in owned memory the camera records of rollouts
   uint8_t* mem = nullptr;
   size_t mem_bytes = 0;
   bool owns_mem = true;

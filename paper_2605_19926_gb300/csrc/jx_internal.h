@@ -113,6 +113,15 @@ struct Params {
   uint32_t* work;
   int32_t chunk;
   int32_t handoff_polls;  // polls of a hand-off wait before it counts as late (jx_debug_handoff_limit)
+  // Rollouts in two passes (see jx_rollout.cu), or all null: the walk's camera
+  // records [steps][n] (cell, fractions and heading cosine; heading sine and
+  // keys | (t mod 4) << 8), the first step of the launch it left to the env
+  // kernel ([n], `steps`: none), and one word per 32 envs of the envs it left any.
+  uint4* cam_a;
+  uint2* cam_b;
+  int32_t* stop;
+  uint32_t* ended;
+  int32_t step_bits;  // in the two passes, where map_bits is 1: the env kernel's map_bits
   int32_t out_stride;  // envs per step in the action / reward / done arrays (n, or a batch's total)
   size_t frame_step;   // bytes per step in the frame array (n frames, or a batch's total)
   int32_t map_bits;    // the map is staged as a bit plane (see MapKind)
@@ -181,6 +190,39 @@ inline bool pregen_runs(const Params& p) { return p.nx_ep != nullptr && p.nx_lan
 cudaError_t kernel_blocks_per_sm(const Params& p, int mode, int* blocks);
 // Launch the fused kernel for `mode`.
 cudaError_t launch(const Params& p, int mode, int grid, cudaStream_t stream);
+
+// Rollouts in two passes (jx_rollout.cu). Camera records are kept for at most
+// rollout_segment(n) steps: longer rollouts run in segments of that many.
+constexpr int kRolloutMinSteps = 4;  // shorter rollouts run in the env kernel alone
+int rollout_segment(int n);
+bool rollout_wanted(int task);  // whether envs of a task roll out in two passes
+size_t rollout_bytes(int n);    // camera records, stop steps and end words of n envs
+void rollout_place(Params& p, uint8_t* mem);  // the pointers into rollout_bytes(p.n) bytes at mem
+// Base parameters to those of the two passes, rows chosen as for the env kernel.
+void rollout_layout(Params& q, size_t smem_per_sm, size_t reserved);
+// Kernel attributes, and the resident blocks per SM.
+cudaError_t rollout_prepare(const Params& q, int* blocks);
+// The walk and the draw of q.steps steps with room for `slots` warps at once;
+// adds the kernels launched to *launches.
+cudaError_t rollout_launch(const Params& q, int slots, cudaStream_t stream, int* launches);
+
+// One launch of the two passes: steps walk_t0 .. walk_t1 - 1 are walked by the
+// first walk_blocks blocks, steps t0 .. t1 - 1 drawn by the others, in
+// n_chunks chunks of `chunk` steps, n_pairs of two, and single steps.
+struct DrawPart {
+  int32_t walk_blocks, walk_t0, walk_t1;
+  int32_t t0, t1, chunk, n_chunks, n_pairs;
+};
+// The same over the groups of a batch: the first block of each group's walk
+// and draw (a group's own walk_blocks is unused).
+struct BatchDrawPart {
+  DrawPart g[kMaxGroups];
+  int32_t first_walk[kMaxGroups], first_draw[kMaxGroups];
+  int32_t walk_blocks;
+};
+static_assert(sizeof(BatchParams) + sizeof(BatchDrawPart) <= 32764, "kernel parameters");
+cudaError_t batch_rollout_prepare(const BatchParams& bq, int* blocks);
+cudaError_t batch_rollout_launch(const BatchParams& bq, int steps, int slots, cudaStream_t stream, int* launches);
 
 // The batched kernel: blocks of `warps` warps, `cols` rays marched together per lane;
 // spec 1 (every group with bit-plane maps and no grayscale stack) selects a

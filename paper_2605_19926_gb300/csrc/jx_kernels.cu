@@ -88,6 +88,11 @@ __global__ void __launch_bounds__(kThreads, kMinBlocksPerSm / kWarpsPerBlock)
   uint8_t* scratch = p.gen_scratch ? p.gen_scratch + (size_t)gw * p.gen_scratch_stride : nullptr;
   int slot = 0;
   if (MODE == MODE_ROLLOUT && p.chunk > 0) {
+    if (p.stop != nullptr) {  // after the walk and the draw: only the envs they left
+      uint32_t left = 0u;
+      for (int i = lane; i < (p.n + 31) >> 5; i += 32) left |= p.ended[i];
+      if (!__any_sync(0xffffffffu, left != 0u)) return;  // the whole grid
+    }
     const uint32_t nch = (uint32_t)((p.steps + p.chunk - 1) / p.chunk);
     const uint32_t items = (uint32_t)p.n * nch;  // below 2^31 (the host caps it)
     bool lost = false;
@@ -95,8 +100,17 @@ __global__ void __launch_bounds__(kThreads, kMinBlocksPerSm / kWarpsPerBlock)
       const uint32_t next = take_item(p, lane);  // its latency overlaps this item
       const int e = (int)(item % (uint32_t)p.n);
       const uint32_t k = item / (uint32_t)p.n;
-      if (k > 0 && !await_chunk(p, e, k) && lane == 0) atomicOr(p.err, 4u);
-      const int t0 = (int)k * p.chunk, t1 = t0 + p.chunk < p.steps ? t0 + p.chunk : p.steps;
+      int t0 = (int)k * p.chunk;
+      const int t1 = t0 + p.chunk < p.steps ? t0 + p.chunk : p.steps;
+      const int first = p.stop != nullptr ? p.stop[e] : 0;  // the env's first step in this kernel
+      if (first >= t1) {
+        item = next;
+        continue;
+      }
+      if (first >= t0)
+        t0 = first;  // its first chunk: nothing to wait for
+      else if (!await_chunk(p, e, k) && lane == 0)
+        atomicOr(p.err, 4u);
       // after a lost map copy the warp only passes its items on (their envs
       // keep their state; the error word says so) and never touches the ring
       if (!lost) lost = !run_env<MODE, MAPK, 1, GRAY>(p, e, wbase, scratch, lane, slot, t0, t1);
@@ -107,9 +121,11 @@ __global__ void __launch_bounds__(kThreads, kMinBlocksPerSm / kWarpsPerBlock)
     finish_items(p, nw, lane);
     return;
   }
-  for (int e = gw; e < p.n; e += nw)
-    if (!run_env<MODE, MAPK, 1, GRAY>(p, e, wbase, scratch, lane, slot, 0, p.steps))
-      break;  // a copy was lost
+  for (int e = gw; e < p.n; e += nw) {
+    const int first = MODE == MODE_ROLLOUT && p.stop != nullptr ? p.stop[e] : 0;
+    if (MODE == MODE_ROLLOUT && first >= p.steps) continue;
+    if (!run_env<MODE, MAPK, 1, GRAY>(p, e, wbase, scratch, lane, slot, first, p.steps)) break;  // a copy was lost
+  }
   if (!kEarlyRelease) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   // shared memory stays allocated until the bulk stores have read it
   if (lane == 0) bulk_wait_read_all();

@@ -716,6 +716,56 @@ def test_unlocked_door_on_the_border_opens_the_map():
     assert torch.equal(frames[-1], run.frames) and (run.env.get_state() == end).all()
 
 
+def _two_pass_cases():
+    m, r = inputs.maze_keydoor, inputs.rooms
+    return [
+        (m(n_envs=1, map_side=32, seed=41, horizon=500), 4),  # the shortest, one env
+        (m(n_envs=33, map_side=32, seed=42, horizon=7), 9),  # ragged warps, every env ends twice
+        (m(n_envs=31, map_side=6, seed=43, horizon=40), 130),  # two segments; keys, goals
+        (dict(r(n_envs=65, map_side=9, seed=44, max_sprites=3, frame_h=21, frame_w=16), turns_per_rev=7), 17),
+        (dict(r(n_envs=5, map_side=45, seed=45, frame_h=3, frame_w=256), radius=0.0, move_step=0.5, horizon=30), 64),
+        (dict(r(n_envs=7, map_side=3, wall_prob=0.0, seed=46, max_sprites=16), turns_per_rev=1, radius=0.49), 6),
+        (dict(r(n_envs=40, map_side=100, seed=47, max_sprites=16, frame_h=64, frame_w=48), shading=1), 12),
+        (dict(m(n_envs=3, map_side=64, seed=48, horizon=11), gray_stack=1), 5),  # planes of one launch and the one before
+        (dict(m(n_envs=1200, map_side=16, seed=49, horizon=100), gray_stack=1), 40),  # parts
+    ]
+
+
+@pytest.mark.parametrize("case", range(9))
+def test_two_pass_rollout_equals_single_steps(case):
+    """Rollouts of 4 or more steps walk first and draw afterwards: three of them
+    in a row (the second from a state set by the host, holding keys beside maps
+    with further locked doors) equal the sequence of steps, state included."""
+    cfg, T = _two_pass_cases()[case]
+    N, H, W = cfg["n_envs"], cfg["frame_h"], cfg["frame_w"]
+    a, b = Run(cfg), Run(cfg)
+    a.reset()
+    b.reset()
+    frames = torch.zeros((T, N, H, W, 3), dtype=torch.uint8, device=a.dev)
+    rewards = torch.zeros((T, N), dtype=torch.float32, device=a.dev)
+    dones = torch.zeros((T, N), dtype=torch.uint8, device=a.dev)
+    for rep in range(3):
+        if rep == 1:
+            for run in (a, b):
+                blob = run.env.get_state()
+                f = run.env.fields(blob)
+                f["flags"][:] = np.arange(N) % 8
+                f["map"][:, 1::3, 1::4] = 16 + np.arange(N)[:, None, None] % 3
+                f["map"][np.arange(N), f["cell_y"], f["cell_x"]] = 0
+                run.env.set_state(blob)
+        acts = torch.from_numpy(np.stack([forward_biased_actions(50 + rep, s, N) for s in range(T)])).to(a.dev)
+        b.env.rollout(acts, frames, rewards, dones)
+        for t in range(T):
+            a.actions.copy_(acts[t])
+            a.env.step(a.actions, a.frames, a.rewards, a.dones)
+            assert torch.equal(a.frames, frames[t]), (rep, t)
+            assert torch.equal(a.rewards, rewards[t]) and torch.equal(a.dones, dones[t]), (rep, t)
+        torch.cuda.synchronize()
+        assert (a.env.get_state() == b.env.get_state()).all(), rep
+    a.env.sync_status()
+    b.env.sync_status()
+
+
 def test_late_handoff_is_reported_and_later_rollouts_exact():
     """With the hand-off wait limit at 0 polls every hand-off of a chunked
     rollout counts as late: the launch still ends, the device error word says
