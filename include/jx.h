@@ -331,7 +331,8 @@ jx_status jx_set_state(jx_env* env, const void* h_buf, size_t bytes);
  * JX_EDEVICE when a kernel recorded bad data since the last call (bit 0: an
  * action outside 0..6, taken as a no-op; bit 1: a bulk map copy completed
  * late or was lost, see jx_debug_wait_limit; bit 2: a rollout hand-off
- * between warps ran out of its bounded wait, see jx_rollout). */
+ * between warps ran out of its bounded wait, see jx_rollout; bit 3: an episode
+ * found no free maze work space in a bounded search and was not built). */
 jx_status jx_sync_status(jx_env* env, void* stream);
 
 /* Number of kernel launches this env has issued since creation. For maze
@@ -415,8 +416,8 @@ jx_status jx_batch_group(const jx_batch* batch, int32_t group, int64_t* env_offs
 /* Change / read the tiling. Results do not depend on it, only speed does. */
 jx_status jx_batch_set_tiling(jx_batch* batch, const jx_tiling* tiling);
 jx_status jx_batch_get_tiling(const jx_batch* batch, jx_tiling* tiling);
-/* Launch shape of the batched step kernel: grid, threads per block, dynamic
- * shared memory per block. */
+/* Launch shape of the batched step kernel: grid (a block per warps_per_block
+ * envs of a group), threads per block, dynamic shared memory per block. */
 jx_status jx_batch_launch_shape(const jx_batch* batch, int32_t* grid, int32_t* block, int32_t* smem_bytes);
 /* Number of batched kernel launches issued since creation (graph replays
  * count their steps; autotuning trials do not count). */

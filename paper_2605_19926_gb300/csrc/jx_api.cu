@@ -1034,7 +1034,7 @@ jx_status jx_sync_status(jx_env* env, void* stream) {
     cudaMemset(env->base.err, 0, 4);
     return fail(JX_EDEVICE, "device error word 0x%x (1: action outside 0..6; 2: a bulk map copy completed late, or "
                             "was lost and its warp left that env and its later envs unstepped; 4: a rollout hand-off between "
-                            "warps ran out of its bounded wait)", word);
+                            "warps ran out of its bounded wait; 8: no maze work space was free)", word);
   }
   return JX_OK;
 }

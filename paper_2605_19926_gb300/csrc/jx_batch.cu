@@ -87,7 +87,7 @@ jx_status apply_tiling(jx_batch* b, const jx_tiling& t) {
   if ((size_t)smem > b->optin)
     return fail(JX_EINVAL, "tiling needs %d bytes of shared memory per block (limit %zu)", smem, b->optin);
   int grid[5] = {};
-  int max_grid = 0;
+  int64_t max_resident = 0;  // blocks
   for (int mode : kModes) {
     int bps = 0;
     cudaError_t err = jx::batch_blocks_per_sm(mode, t.cols_per_lane, jx::batch_spec(bp), t.warps_per_block, smem, &bps);
@@ -96,9 +96,17 @@ jx_status apply_tiling(jx_batch* b, const jx_tiling& t) {
     const int64_t need = (b->n_total + t.warps_per_block - 1) / t.warps_per_block;
     const int64_t cap = (int64_t)bps * b->num_sms;
     grid[mode] = (int)std::min(need, cap);
-    max_grid = std::max(max_grid, grid[mode]);
+    if (mode == jx::MODE_STEP) {  // not persistent: a block per warps_per_block envs of a group
+      int64_t blocks = 0;
+      for (int i = 0; i < bp.n_groups; ++i) blocks += (bp.g[i].n + t.warps_per_block - 1) / t.warps_per_block;
+      grid[mode] = (int)blocks;
+    }
+    max_resident = std::max(max_resident, cap);
   }
-  const size_t scratch_need = stride * (size_t)max_grid * t.warps_per_block;
+  // the work space of each resident warp, then the bits of the spaces in use
+  const size_t warps = (size_t)max_resident * t.warps_per_block;
+  const size_t slots_off = jx::host::align256(stride * warps);
+  const size_t scratch_need = stride > 0 ? slots_off + jx::gen_slot_bytes((int64_t)warps) : 0;
   if (scratch_need > b->scratch_bytes) {
     uint8_t* fresh = nullptr;
     cudaError_t err = cudaMalloc(&fresh, scratch_need);
@@ -110,9 +118,18 @@ jx_status apply_tiling(jx_batch* b, const jx_tiling& t) {
     b->scratch = fresh;
     b->scratch_bytes = scratch_need;
   }
+  uint32_t* slots = stride > 0 ? reinterpret_cast<uint32_t*>(b->scratch + slots_off) : nullptr;
+  if (slots) {
+    cudaError_t err = cudaDeviceSynchronize();  // steps in flight hold spaces of the former layout
+    if (err == cudaSuccess) err = cudaMemset(slots, 0, jx::gen_slot_bytes((int64_t)warps));
+    if (err == cudaSuccess) err = cudaDeviceSynchronize();
+    if (err != cudaSuccess) return cuda_fail(err, "clearing the maze work spaces");
+  }
   for (int i = 0; i < bp.n_groups; ++i) {
     bp.g[i].gen_scratch = stride > 0 ? b->scratch : nullptr;
     bp.g[i].gen_scratch_stride = stride;
+    bp.g[i].gen_slots = slots;
+    bp.g[i].n_gen_slots = (int32_t)warps;
   }
   bp.queue = b->queue;
   b->bp = bp;

@@ -1156,6 +1156,33 @@ __device__ __forceinline__ void gen_ascii(const Params& p, int e, uint32_t ep, u
   __syncwarp();
 }
 
+// A free work space of Params::gen_slots, or -1 after a bounded search (there
+// are as many as resident warps, so one is always free). Every lane gets it.
+__device__ __forceinline__ int take_gen_slot(const Params& p, int lane) {
+  int slot = -1;
+  if (lane == 0) {
+    const int words = (p.n_gen_slots + 31) >> 5;
+    int w = (int)((blockIdx.x * 37u) % (unsigned)words);
+    for (int it = 0; it < 1 << 20 && slot < 0; ++it, w = w + 1 == words ? 0 : w + 1) {
+      const uint32_t valid = p.n_gen_slots - 32 * w >= 32 ? 0xFFFFFFFFu : (1u << (p.n_gen_slots - 32 * w)) - 1u;
+      uint32_t open = ~*reinterpret_cast<volatile uint32_t*>(p.gen_slots + w) & valid;
+      while (open && slot < 0) {
+        const uint32_t bit = open & (0u - open);
+        const uint32_t old = atomicOr(p.gen_slots + w, bit);
+        if (!(old & bit)) slot = 32 * w + __ffs(bit) - 1;
+        open = ~old & valid & ~bit;
+      }
+    }
+    __threadfence();
+  }
+  return __shfl_sync(0xffffffffu, slot, 0);
+}
+__device__ __forceinline__ void give_gen_slot(const Params& p, int slot, int lane) {
+  __threadfence();
+  __syncwarp();
+  if (lane == 0) atomicAnd(p.gen_slots + (slot >> 5), ~(1u << (slot & 31)));
+}
+
 // The maze work space lives in the warp's frame staging ring when it fits
 // (32 x 32 mazes need 2.3 KB), else in the global per-warp slot. Inlined
 // behind unlikely branches: a call would make every value live across it
@@ -1170,7 +1197,7 @@ __device__ __forceinline__ void generate(const Params& p, int e, uint32_t ep, ui
     take_next<MAPK>(p, e, ep, wbase, lane);
     return;
   }
-  const WarpSmem ws{wbase, fill_lane(p, lane)};
+  const WarpSmem ws{wbase, FillLane{}};
   const bool bits = map_bits<MAPK>(p);
   const bool maze = p.task != 0 && p.task != kTaskAscii;
   const size_t ring = (size_t)p.staging * p.frame_block_bytes;
@@ -1181,6 +1208,15 @@ __device__ __forceinline__ void generate(const Params& p, int e, uint32_t ep, ui
     if (lane == 0) bulk_wait_read_all();  // the ring's pending frame stores have read it
     __syncwarp();
   }
+  int gen_slot = -1;
+  if (maze && !work_in_ring && scratch == nullptr) {
+    gen_slot = take_gen_slot(p, lane);
+    if (gen_slot < 0) {  // never: see take_gen_slot
+      if (lane == 0) atomicOr(p.err, 8u);
+      return;
+    }
+    scratch = p.gen_scratch + (size_t)gen_slot * p.gen_scratch_stride;
+  }
   uint8_t* smap = !bits ? ws.map(p) : (map_in_ring ? ws.ring() + align16((int)work_bytes) : p.st.map + (size_t)e * p.S * p.S);
   if (p.task == 0) {
     gen_rooms(p, e, ep, smap, lane);
@@ -1190,6 +1226,7 @@ __device__ __forceinline__ void generate(const Params& p, int e, uint32_t ep, ui
     gen_maze(p, e, ep, smap, work_in_ring ? ws.ring() : scratch, lane);
   }
   write_plane<MAPK>(p, e, smap, ws.map(p), lane);
+  if (gen_slot >= 0) give_gen_slot(p, gen_slot, lane);
 }
 
 // ------------------------------------------------------------------ step ----

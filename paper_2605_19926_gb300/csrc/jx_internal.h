@@ -77,6 +77,11 @@ struct Params {
   const float* col_k;     // [W] (2 (c + 1/2) / W - 1) * tan(fov / 2)
   uint8_t* gen_scratch;   // [warps][gen_scratch_stride], maze generation work space
   size_t gen_scratch_stride;
+  // Batched steps (blocks handed out in order, no warp index to tell work
+  // spaces apart): one bit per slot of gen_scratch, taken and given back by
+  // the warps that build a maze; there are as many slots as resident warps.
+  uint32_t* gen_slots;
+  int32_t n_gen_slots;
   // The next episode of each env, built ahead by the lane-parallel
   // pre-generation kernel (mazes of side >= kPregenMinSide), or all null:
   // the state fields generation writes, the episode number they hold
@@ -154,6 +159,7 @@ struct BatchParams {
   uint32_t* queue;       // [kMaxGroups + 1] next env per group, warps finished; zero between launches
   int32_t n_groups;
   int32_t warp_bytes;  // per-warp shared memory: the largest group's layout
+  int32_t first_block[kMaxGroups];  // steps: the first block of each group
 };
 
 // Fill in the per-warp shared memory layout of p (needs W, K, S, map_bits, frame_block_bytes).
@@ -229,6 +235,9 @@ cudaError_t batch_rollout_launch(const BatchParams& bq, int steps, int slots, cu
 // specialised instance, 0 the general one (batch_spec gives it for a launch).
 int batch_spec(const BatchParams& bp);
 cudaError_t batch_blocks_per_sm(int mode, int cols, int spec, int warps, int smem_bytes, int* blocks);
-cudaError_t batch_launch(const BatchParams& bp, int mode, int cols, int warps, int grid, cudaStream_t stream);
+// `grid` resident blocks; MODE_STEP launches one block per `warps` envs of a
+// group instead (and fills in bp.first_block).
+cudaError_t batch_launch(BatchParams& bp, int mode, int cols, int warps, int grid, cudaStream_t stream);
+inline size_t gen_slot_bytes(int64_t warps) { return 4 * (size_t)((warps + 31) / 32); }  // Params::gen_slots
 
 }  // namespace jx

@@ -116,7 +116,8 @@ struct Slot {
   cudaStream_t stream = nullptr;
   cudaEvent_t done = nullptr;
   uint32_t* queue = nullptr;    // work-queue counters of the batched kernel
-  uint8_t* scratch = nullptr;   // maze work space, one slot per warp
+  uint8_t* scratch = nullptr;   // maze work space, one slot per warp, then the bits of those in use
+  uint32_t* gen_slots = nullptr;
   uint8_t* h_actions = nullptr;  // pinned staging of the launch's actions
   uint8_t* d_actions = nullptr;
   bool busy = false;
@@ -198,6 +199,8 @@ jx_status dispatch(jx_server* sv, Slot& sl, std::vector<Session*>& chosen) {
     p.actions = sl.d_actions + off;
     p.gen_scratch = sv->scratch_stride ? sl.scratch : nullptr;
     p.gen_scratch_stride = sv->scratch_stride;
+    p.gen_slots = sl.gen_slots;
+    p.n_gen_slots = sv->max_warps;
     bp.g[i] = p;
     warp_bytes = std::max(warp_bytes, p.warp_bytes);
     off += (r.actions.size() + 15) & ~(size_t)15;
@@ -360,7 +363,7 @@ jx_status jx_server_create(int device, uint64_t budget_bytes, int32_t max_sessio
   sv->tiling = t;
   sv->max_map_side = max_map_side;
   sv->scratch_stride = jx::gen_scratch_bytes(JX_TASK_MAZE_KEYDOOR, max_map_side & ~1);
-  sv->max_warps = jx::kMinBlocksPerSm * sv->num_sms;
+  sv->max_warps = 32 * sv->num_sms;  // at least the resident warps of a step
   sv->max_launch_envs = 1 << 20;
   sv->budget = (size_t)budget_bytes;
   sv->max_sessions = max_sessions;
@@ -381,16 +384,19 @@ jx_status jx_server_create(int device, uint64_t budget_bytes, int32_t max_sessio
   sv->slots.resize(max_inflight);
   for (Slot& sl : sv->slots) {
     const size_t qbytes = sizeof(uint32_t) * (jx::kMaxGroups + 1);
-    const size_t scratch = sv->scratch_stride * (size_t)sv->max_warps;
+    const size_t slots_off = jx::host::align256(sv->scratch_stride * (size_t)sv->max_warps);
+    const size_t scratch = sv->scratch_stride ? slots_off + jx::gen_slot_bytes(sv->max_warps) : 0;
     if ((err = cudaStreamCreateWithFlags(&sl.stream, cudaStreamNonBlocking)) != cudaSuccess ||
         (err = cudaEventCreateWithFlags(&sl.done, cudaEventDisableTiming)) != cudaSuccess ||
         (err = cudaMalloc(&sl.queue, qbytes)) != cudaSuccess ||
         (err = cudaMemset(sl.queue, 0, qbytes)) != cudaSuccess ||
-        (scratch && (err = cudaMalloc(&sl.scratch, scratch)) != cudaSuccess) ||
+        (scratch && ((err = cudaMalloc(&sl.scratch, scratch)) != cudaSuccess ||
+                     (err = cudaMemset(sl.scratch + slots_off, 0, scratch - slots_off)) != cudaSuccess)) ||
         (err = cudaMalloc(&sl.d_actions, (size_t)sv->max_launch_envs + 16 * jx::kMaxGroups)) != cudaSuccess ||
         (err = cudaHostAlloc(&sl.h_actions, (size_t)sv->max_launch_envs + 16 * jx::kMaxGroups,
                              cudaHostAllocDefault)) != cudaSuccess)
       return bail(fail(JX_ENOMEM, "launch slot allocation failed: %s", cudaGetErrorString(err)));
+    if (scratch) sl.gen_slots = reinterpret_cast<uint32_t*>(sl.scratch + slots_off);
   }
   if ((err = cudaDeviceSynchronize()) != cudaSuccess) return bail(cuda_fail(err, "server create"));
   try {
