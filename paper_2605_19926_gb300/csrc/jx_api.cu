@@ -494,8 +494,7 @@ jx_status create_impl(const jx_config* cfg, int device, void* ext, size_t ext_by
   env->state = env->mem;
   env->aux = env->mem + off_aux;
   env->scratch = scratch_bytes ? env->mem + off_scratch : nullptr;
-  if ((err = cudaMemset(env->state, 0, env->state_bytes)) != cudaSuccess ||
-      (err = cudaMemset(env->mem + off_plane, 0, plane_bytes)) != cudaSuccess) {
+  if ((err = cudaMemset(env->mem, 0, off_plane + plane_bytes)) != cudaSuccess) {  // the tables follow below
     jx_destroy(env);
     return cuda_fail(err, "cudaMemset of the state");
   }
@@ -600,12 +599,11 @@ jx_status create_impl(const jx_config* cfg, int device, void* ext, size_t ext_by
   if (p.stop) {
     env->draw = p;
     jx::rollout_layout(env->draw, prop.sharedMemPerMultiprocessor, prop.reservedSharedMemPerBlock);
-    int b = 0;
-    if ((err = jx::rollout_prepare(env->draw, &b)) != cudaSuccess) {
+    if ((err = jx::rollout_prepare(env->draw)) != cudaSuccess) {
       jx_destroy(env);
-      return cuda_fail(err, "occupancy query");
+      return cuda_fail(err, "kernel attributes");
     }
-    env->draw_slots = (b > 0 ? b : 1) * jx::kWarpsPerBlock * env->num_sms;
+    env->draw_slots = jx::kMinBlocksPerSm * env->num_sms;
   }
   // the memset and the table copy are done before the handle is returned
   if ((err = cudaStreamSynchronize(0)) != cudaSuccess) {

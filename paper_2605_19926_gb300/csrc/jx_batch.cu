@@ -155,10 +155,9 @@ jx_status prepare_draw(jx_batch* b) {
     b->segment = b->segment == 0 ? seg : std::min(b->segment, seg);
   }
   if (b->segment == 0) return JX_OK;
-  int blocks = 0;
-  cudaError_t err = jx::batch_rollout_prepare(bq, &blocks);
-  if (err != cudaSuccess) return cuda_fail(err, "occupancy query");
-  b->draw_slots = std::max(1, blocks) * jx::kWarpsPerBlock * b->num_sms;
+  cudaError_t err = jx::batch_rollout_prepare(bq);
+  if (err != cudaSuccess) return cuda_fail(err, "kernel attributes");
+  b->draw_slots = jx::kMinBlocksPerSm * b->num_sms;
   return JX_OK;
 }
 

@@ -20,7 +20,7 @@ struct jx_env {
   int smem_block = 0;
   jx::Params base{};
   jx::Params draw{};   // base with the draw pass's shared-memory layout (rollouts in two passes)
-  int draw_slots = 0;  // warps of the draw pass resident at once
+  int draw_slots = 0;  // warps of the draw pass resident at once, about
   // one device block: state | aux | bit planes | scratch (owned, or in the
   // caller's memory), and in owned memory the camera records of rollouts
   uint8_t* mem = nullptr;

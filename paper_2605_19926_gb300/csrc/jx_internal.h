@@ -206,8 +206,7 @@ size_t rollout_bytes(int n);    // camera records, stop steps and end words of n
 void rollout_place(Params& p, uint8_t* mem);  // the pointers into rollout_bytes(p.n) bytes at mem
 // Base parameters to those of the two passes, rows chosen as for the env kernel.
 void rollout_layout(Params& q, size_t smem_per_sm, size_t reserved);
-// Kernel attributes, and the resident blocks per SM.
-cudaError_t rollout_prepare(const Params& q, int* blocks);
+cudaError_t rollout_prepare(const Params& q);  // kernel attributes
 // The walk and the draw of q.steps steps with room for `slots` warps at once;
 // adds the kernels launched to *launches.
 cudaError_t rollout_launch(const Params& q, int slots, cudaStream_t stream, int* launches);
@@ -227,7 +226,7 @@ struct BatchDrawPart {
   int32_t walk_blocks;
 };
 static_assert(sizeof(BatchParams) + sizeof(BatchDrawPart) <= 32764, "kernel parameters");
-cudaError_t batch_rollout_prepare(const BatchParams& bq, int* blocks);
+cudaError_t batch_rollout_prepare(const BatchParams& bq);
 cudaError_t batch_rollout_launch(const BatchParams& bq, int steps, int slots, cudaStream_t stream, int* launches);
 
 // The batched kernel: blocks of `warps` warps, `cols` rays marched together per lane;

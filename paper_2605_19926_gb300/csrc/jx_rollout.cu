@@ -490,11 +490,8 @@ void rollout_layout(Params& q, size_t smem_per_sm, size_t reserved) {
   if (q.warp_bytes < walk_warp_bytes(q.K)) q.warp_bytes = walk_warp_bytes(q.K);
 }
 
-cudaError_t rollout_prepare(const Params& q, int* blocks) {
-  auto k = q.gray ? rollout_kernel<1> : rollout_kernel<0>;
-  cudaError_t err = raise_smem_limit(k);
-  if (err == cudaSuccess) err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, k, kThreads, block_smem_bytes(q));
-  return err;
+cudaError_t rollout_prepare(const Params& q) {
+  return raise_smem_limit(q.gray ? rollout_kernel<1> : rollout_kernel<0>);
 }
 
 cudaError_t rollout_launch(const Params& q, int slots, cudaStream_t stream, int* launches) {
@@ -518,14 +515,10 @@ cudaError_t rollout_launch(const Params& q, int slots, cudaStream_t stream, int*
   return cudaSuccess;
 }
 
-cudaError_t batch_rollout_prepare(const BatchParams& bq, int* blocks) {
+cudaError_t batch_rollout_prepare(const BatchParams& bq) {
   bool gray = false;
   for (int g = 0; g < bq.n_groups; ++g) gray = gray || bq.g[g].gray;
-  auto k = gray ? batch_rollout_kernel<2> : batch_rollout_kernel<0>;
-  cudaError_t err = raise_smem_limit(k);
-  if (err == cudaSuccess)
-    err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, k, kThreads, (size_t)bq.warp_bytes * kWarpsPerBlock);
-  return err;
+  return raise_smem_limit(gray ? batch_rollout_kernel<2> : batch_rollout_kernel<0>);
 }
 
 cudaError_t batch_rollout_launch(const BatchParams& bq, int steps, int slots, cudaStream_t stream, int* launches) {
