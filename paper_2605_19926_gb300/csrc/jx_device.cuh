@@ -563,107 +563,198 @@ __device__ __forceinline__ void gen_rooms(const Params& p, int e, uint32_t ep, u
   __syncwarp();
 }
 
-// Work space of one maze generation (n = nodes): the per-carve draws, the
-// DFS stack of node cells, and each node's DFS discovery / finish counters.
-struct MazeScratch {
-  uint32_t* rnd;     // [n] high 32 bits of the per-carve draws
-  uint16_t* stack;   // [n] node cells packed as y << 8 | x
-  uint16_t* disc;    // [n] push counter when the node was discovered
-  uint16_t* fin;     // [n] push counter when the node was finished
-  int32_t* result;   // [4] goal node, its depth, the door's two path nodes (packed cells)
+// Work space of one maze generation of nn x nn nodes. The fast part is in the
+// walk's chain of dependent accesses:
+//   avail  [(nn + 2)^2] bytes, nodes with a border around them: the directions
+//          (bit 0 N, 1 E, 2 S, 3 W) in which an unvisited node lies
+//   stack  [n] the path to the current node, cells packed as y << 8 | x;
+//          afterwards each node's place in the visiting order
+// the slow part is written, or read ahead:
+//   seq    [n] visiting order: node | depth << 16
+//   pick   [n] per carve: the draw's choice among 2, 3 and 4 candidates
+struct MazeWork {
+  uint8_t* avail;
+  uint16_t* stack;
+  uint32_t* seq;
+  uint8_t* pick;
 };
-__host__ __device__ __forceinline__ size_t maze_scratch_bytes(int n) {
-  return (size_t)align16(4 * n) + 3 * (size_t)align16(2 * n) + 16;
+__host__ __device__ __forceinline__ int maze_nodes(int S) { return (S - 2) / 2; }  // per side
+__host__ __device__ __forceinline__ size_t maze_fast_bytes(int nn) {
+  return (size_t)align16((nn + 2) * (nn + 2)) + align16(2 * nn * nn);
 }
-__device__ __forceinline__ MazeScratch maze_scratch(uint8_t* q, int n) {
-  MazeScratch m;
-  m.rnd = (uint32_t*)q;
-  q += align16(4 * n);
-  m.stack = (uint16_t*)q;
-  q += align16(2 * n);
-  m.disc = (uint16_t*)q;
-  q += align16(2 * n);
-  m.fin = (uint16_t*)q;
-  q += align16(2 * n);
-  m.result = (int32_t*)q;
+__host__ __device__ __forceinline__ size_t maze_slow_bytes(int nn) {
+  return (size_t)align16(4 * nn * nn) + align16(nn * nn);
+}
+__device__ __forceinline__ MazeWork maze_work(uint8_t* fast, uint8_t* slow, int nn) {
+  MazeWork m;
+  m.avail = fast;
+  m.stack = (uint16_t*)(fast + align16((nn + 2) * (nn + 2)));
+  m.seq = (uint32_t*)slow;
+  m.pick = slow + align16(4 * nn * nn);
   return m;
 }
 
+// The direction a carve takes: candidate r of the set `open` (bits in N, E, S,
+// W order), r the draw's choice for that many candidates (bit 0: of two, bits
+// 1-2: of three, bits 3-4: of four).
+struct MazePick {
+  uint8_t d[512];
+  constexpr MazePick() : d() {
+    for (int open = 0; open < 16; ++open)
+      for (int pick = 0; pick < 32; ++pick) {
+        int n = 0;
+        for (int b = 0; b < 4; ++b) n += (open >> b) & 1;
+        int r = n == 2 ? (pick & 1) : (n == 3 ? ((pick >> 1) & 3) : (n == 4 ? pick >> 3 : 0));
+        int dir = 0;
+        for (int b = 0; b < 4; ++b)
+          if ((open >> b) & 1) {
+            dir = b;
+            if (r-- == 0) break;
+          }
+        d[open * 32 + pick] = (uint8_t)dir;
+      }
+  }
+};
+__constant__ MazePick c_maze_pick = MazePick();
+
 // Key-door maze: depth-first backtracker over the nodes at odd coordinates,
-// N/E/S/W neighbour order, one draw per carved passage. A node is unvisited
-// while its cell is still a wall. Because the maze is the DFS tree, a node's
-// BFS distance from the spawn is its stack depth when pushed, and the stack at
-// that moment is its path from the spawn: the goal (deepest node, ties to
-// the smallest row-major index) and the two path nodes around the door are
-// recorded during the walk. The nodes reachable without crossing the door are
-// those outside the door's subtree (a discovery / finish interval test).
-__device__ __forceinline__ void gen_maze(const Params& p, int e, uint32_t ep, uint8_t* smap, uint8_t* scratch, int lane) {
+// N/E/S/W neighbour order, one draw per carved passage. Because the maze is
+// the DFS tree, a node's BFS distance from the spawn is its depth, the nodes
+// below a node are a run of the visiting order, and the node at depth j on the
+// path to a node is the last one of depth j visited before it: the goal
+// (deepest, ties to the smallest row-major index), the door's two path nodes
+// and the nodes reachable without crossing the door all come from the visiting
+// order, by the warp together.
+// The walk is a chain of dependent accesses, so it is kept short: all lanes
+// step it together (no divergence), one load says which neighbours are open
+// (the visits keep it up to date, four lanes at a time), one constant says
+// which of them the draw picks, and a dead end is left by looking at 32 nodes
+// of the path at once. (72 instructions a move on one lane, over two moves a
+// node, before; about 60 a node now. Resets of 4096 envs: 32 x 32 mazes 197 ->
+// 97 us, 64 x 64 968 -> 326; of 256 envs 90 -> 46 and 372 -> 138. With the
+// choice in a register table read by shuffles instead of the constant: 117.)
+// FAST_SMEM: the fast part lies in shared memory (an instance of its own, so
+// that the compiler knows the address space).
+template <bool FAST_SMEM>
+__device__ __forceinline__ void gen_maze(const Params& p, int e, uint32_t ep, uint8_t* smap, const MazeWork& m, int lane) {
   const int S = p.S, n_cells = S * S;
-  const int nn = (S - 2) / 2, n = nn * nn;
-  MazeScratch m = maze_scratch(scratch, n);
+  const int nn = maze_nodes(S), n = nn * nn, q = nn + 2;
   const uint64_t kw = stream_key(p.seed, (uint32_t)e, ep, P_WALL);
-  for (int i = lane; i < n_cells; i += 32) smap[i] = (uint8_t)(1 + (draw_at(kw, (uint32_t)i) & 3));
+  for (int i = 4 * lane; i < n_cells; i += 128) {  // S is even: whole words
+    uint32_t w = 0x01010101u;
+#pragma unroll
+    for (int b = 0; b < 4; ++b) w += (uint32_t)(draw_at(kw, (uint32_t)(i + b)) & 3) << (8 * b);
+    *reinterpret_cast<uint32_t*>(smap + i) = w;
+  }
   const uint64_t kd = stream_key(p.seed, (uint32_t)e, ep, P_DFS);
-  for (int j = lane; j < n - 1; j += 32) m.rnd[j] = (uint32_t)(draw_at(kd, (uint32_t)j) >> 32);
+  for (int j = lane; j < n; j += 32) {
+    const uint32_t hi = (uint32_t)(draw_at(kd, (uint32_t)j) >> 32);
+    m.pick[j] = (uint8_t)(hi >> 31 | below32(hi, 3u) << 1 | (hi >> 30) << 3);
+  }
+  for (int i = lane; i < q * q; i += 32) {
+    const int y = i / q, x = i - y * q;
+    const bool node = x >= 1 && x <= nn && y >= 1 && y <= nn;
+    m.avail[i] = node ? (uint8_t)((y > 1 ? 1 : 0) | (x < nn ? 2 : 0) | (y < nn ? 4 : 0) | (x > 1 ? 8 : 0)) : (uint8_t)0;
+  }
   const int start = (int)below(draw_at(stream_key(p.seed, (uint32_t)e, ep, P_SPAWN), 0), (uint32_t)n);
   __syncwarp();
-  if (lane == 0) {
-    int vx = 2 * (start % nn) + 1, vy = 2 * (start / nn) + 1, v = start;
-    smap[vy * S + vx] = 0;
-    int sp = 0, pushes = 0, carved = 0;
-    m.stack[sp++] = (uint16_t)(vy << 8 | vx);
-    m.disc[v] = (uint16_t)pushes++;
-    int best_v = start, best_d = 0, door_a = vy << 8 | vx, door_b = door_a;
-    for (;;) {
-      const int c = vy * S + vx;
-      const uint32_t open = (uint32_t)(vy > 1 && smap[c - 2 * S] != 0) | ((uint32_t)(vx < S - 3 && smap[c + 2] != 0) << 1) |
-                            ((uint32_t)(vy < S - 3 && smap[c + 2 * S] != 0) << 2) |
-                            ((uint32_t)(vx > 1 && smap[c - 2] != 0) << 3);
-      if (open == 0) {
-        m.fin[v] = (uint16_t)pushes;
-        if (--sp == 0) break;
-        const int top = m.stack[sp - 1];
-        vx = top & 0xff;
-        vy = top >> 8;
-        v = (vy >> 1) * nn + (vx >> 1);
-        continue;
-      }
-      // the r-th unvisited neighbour in N, E, S, W order
-      uint32_t bits = open;
-      for (uint32_t r = below32(m.rnd[carved++], (uint32_t)__popc(open)); r > 0; --r) bits &= bits - 1;
-      const int d = __ffs(bits) - 1;
-      const int dx = d == 1 ? 1 : (d == 3 ? -1 : 0), dy = d == 0 ? -1 : (d == 2 ? 1 : 0);
-      smap[c + dy * S + dx] = 0;
-      vx += 2 * dx;
-      vy += 2 * dy;
-      smap[vy * S + vx] = 0;
-      v = (vy >> 1) * nn + (vx >> 1);
-      const int depth = sp;
-      m.stack[sp++] = (uint16_t)(vy << 8 | vx);
-      m.disc[v] = (uint16_t)pushes++;
-      if (depth > best_d || (depth == best_d && v < best_v)) {
-        best_v = v;
-        best_d = depth;
-        const int j = (depth + 1) / 2;  // the door sits on edge ceil(depth / 2) of the path
-        door_a = m.stack[j - 1];
-        door_b = m.stack[j];
-      }
+  // lanes 0..3: the neighbour in direction `lane`, and all its directions but the one back
+  const int my_step = lane == 0 ? -q : (lane == 1 ? 1 : (lane == 2 ? q : -1));
+  const uint32_t my_keep = ~(1u << (lane ^ 2));
+  {
+    int yx = (2 * (start / nn) + 1) << 8 | (2 * (start % nn) + 1);
+    int node = start, a = (start / nn + 1) * q + start % nn + 1, c = (yx >> 8) * S + (yx & 255);
+    int depth = 0;
+    if (lane < 4) m.avail[a + my_step] &= (uint8_t)my_keep;
+    if (lane == 0) {
+      smap[c] = 0;
+      m.stack[0] = (uint16_t)yx;
+      m.seq[0] = (uint32_t)node;
     }
-    m.result[0] = best_v;
-    m.result[1] = best_d;
-    m.result[2] = door_a;
-    m.result[3] = door_b;
+    __syncwarp();
+    uint32_t pick = m.pick[0];
+    uint32_t open = m.avail[a];
+    for (int k = 1; k < n; ++k) {  // the k-th carve
+      if (open == 0) {
+        // a dead end: back to the deepest node of the path with an open side
+        // (the nodes above it are done); there is one until every node is visited
+        int from = depth;
+        for (; from > 0; from -= 32) {
+          const int i = from - 1 - lane;
+          uint32_t yx_i = 0u, open_i = 0u;
+          if (i >= 0) {
+            yx_i = m.stack[i];
+            open_i = m.avail[(((yx_i >> 8) + 1) >> 1) * q + (((yx_i & 255u) + 1) >> 1)];
+          }
+          const uint32_t b = __ballot_sync(0xffffffffu, open_i != 0u);
+          if (b) {
+            const int src = __ffs(b) - 1;
+            depth = from - 1 - src;
+            yx = (int)__shfl_sync(0xffffffffu, yx_i, src);
+            open = __shfl_sync(0xffffffffu, open_i, src);
+            break;
+          }
+        }
+        if (from <= 0) break;
+        const int y = yx >> 8, x = yx & 255;
+        c = y * S + x;
+        a = ((y + 1) >> 1) * q + ((x + 1) >> 1);
+        node = (y >> 1) * nn + (x >> 1);
+      }
+      const int d = c_maze_pick.d[open * 32 + pick];
+      pick = m.pick[k];  // for the next carve
+      const int sgn = ((d + 1) & 2) ? 1 : -1;
+      const bool row = d & 1;
+      const int dc = sgn * (row ? 1 : S);
+      if (lane < 2) smap[c + (lane + 1) * dc] = 0;  // the passage and the node
+      c += 2 * dc;
+      a += sgn * (row ? 1 : q);
+      node += sgn * (row ? 1 : nn);
+      yx += sgn * (row ? 2 : 512);
+      ++depth;
+      open = m.avail[a];
+      if (lane < 4) m.avail[a + my_step] &= (uint8_t)my_keep;
+      if (lane == 0) {
+        m.stack[depth] = (uint16_t)yx;
+        m.seq[k] = (uint32_t)node | (uint32_t)depth << 16;
+      }
+      __syncwarp();
+    }
   }
   __syncwarp();
-  const int goal = m.result[0];
-  const int door_a = m.result[2], door_b = m.result[3];
-  const int dxc = ((door_a & 0xff) + (door_b & 0xff)) >> 1, dyc = ((door_a >> 8) + (door_b >> 8)) >> 1;
+  // the goal: the deepest node, ties to the smallest index (n < 4096)
+  uint32_t top = 0u;
+  for (int k = lane; k < n; k += 32) {
+    const uint32_t v = m.seq[k], key = (v >> 16) << 12 | (4095u - (v & 0xffffu));
+    top = key > top ? key : top;
+  }
+  top = __reduce_max_sync(0xffffffffu, top);
+  const int goal = 4095 - (int)(top & 4095u), goal_d = (int)(top >> 12);
+  // the nodes' places in the visiting order
+  uint16_t* const disc = m.stack;
+  for (int k = lane; k < n; k += 32) disc[m.seq[k] & 0xffffu] = (uint16_t)k;
+  __syncwarp();
+  // the door sits on edge ceil(d / 2) of the path to the goal: between its nodes at depths j - 1 and j
+  const int j = (goal_d + 1) / 2, k_goal = disc[goal];
+  uint32_t ka = 0u, kb = 0u;
+  for (int k = lane; k <= k_goal; k += 32) {
+    const int depth = (int)(m.seq[k] >> 16);
+    if (depth == j) kb = (uint32_t)k;
+    if (depth == j - 1) ka = (uint32_t)k;
+  }
+  ka = __reduce_max_sync(0xffffffffu, ka);
+  kb = __reduce_max_sync(0xffffffffu, kb);
+  // the door's subtree: visits kb .. d1 - 1
+  uint32_t d1_min = (uint32_t)n;
+  for (int k = lane; k < n; k += 32)
+    if (k > (int)kb && (int)(m.seq[k] >> 16) <= j && (uint32_t)k < d1_min) d1_min = (uint32_t)k;
+  const int d0 = (int)kb, d1 = (int)__reduce_min_sync(0xffffffffu, d1_min);
+  const int node_a = (int)(m.seq[ka] & 0xffffu), node_b = (int)(m.seq[kb] & 0xffffu);
+  const int dxc = node_a % nn + node_b % nn + 1, dyc = node_a / nn + node_b / nn + 1;
   if (lane == 0) smap[dyc * S + dxc] = (uint8_t)kDoor;
   // key: uniform over spawn-side nodes except the spawn
-  const int pj = ((door_b >> 8) >> 1) * nn + ((door_b & 0xff) >> 1);
-  const int d0 = m.disc[pj], d1 = m.fin[pj];
   auto side = [&](int v) {
-    int dv = m.disc[v];
+    int dv = disc[v];
     return v != start && !(dv >= d0 && dv < d1);
   };
   const int n_side = n - (d1 - d0) - 1;
@@ -1184,12 +1275,12 @@ __device__ __forceinline__ void give_gen_slot(const Params& p, int slot, int lan
 }
 
 // The maze work space lives in the warp's frame staging ring when it fits
-// (32 x 32 mazes need 2.3 KB), else in the global per-warp slot. Inlined
-// behind unlikely branches: a call would make every value live across it
-// spill in the hot loop. A byte map is generated in shared memory and copied
-// out. In bit mode the byte map is generated in the ring, after the maze work
-// space, when both fit there (the one-lane DFS then never waits on global
-// memory), else in place in the state block; the bit plane is staged from it.
+// (32 x 32 mazes need 2 KB), or its fast part (64 x 64: 3 KB), the rest in the
+// global per-warp slot. Inlined behind unlikely branches: a call would make
+// every value live across it spill in the hot loop. A byte map is generated
+// in shared memory and copied out. In bit mode the byte map is generated in
+// the ring, after the maze work space, when both fit there, else in place in
+// the state block; the bit plane is written from it.
 template <int MAPK>
 __device__ __forceinline__ void generate(const Params& p, int e, uint32_t ep, uint8_t* wbase, uint8_t* scratch,
                                       int lane) {
@@ -1201,10 +1292,12 @@ __device__ __forceinline__ void generate(const Params& p, int e, uint32_t ep, ui
   const bool bits = map_bits<MAPK>(p);
   const bool maze = p.task != 0 && p.task != kTaskAscii;
   const size_t ring = (size_t)p.staging * p.frame_block_bytes;
-  const size_t work_bytes = maze ? maze_scratch_bytes(((p.S - 2) / 2) * ((p.S - 2) / 2)) : 0;
-  const bool work_in_ring = maze && work_bytes <= ring;
+  const int nn = maze_nodes(p.S);
+  const size_t fast_bytes = maze ? maze_fast_bytes(nn) : 0, slow_bytes = maze ? maze_slow_bytes(nn) : 0;
+  const bool fast_in_ring = maze && fast_bytes <= ring, work_in_ring = maze && fast_bytes + slow_bytes <= ring;
+  const size_t work_bytes = work_in_ring ? fast_bytes + slow_bytes : (fast_in_ring ? fast_bytes : 0);
   const bool map_in_ring = bits && (size_t)align16((int)work_bytes) + (size_t)p.S * p.S <= ring;
-  if (work_in_ring || map_in_ring) {
+  if (fast_in_ring || map_in_ring) {
     if (lane == 0) bulk_wait_read_all();  // the ring's pending frame stores have read it
     __syncwarp();
   }
@@ -1222,8 +1315,10 @@ __device__ __forceinline__ void generate(const Params& p, int e, uint32_t ep, ui
     gen_rooms(p, e, ep, smap, lane);
   } else if (p.task == kTaskAscii) {
     gen_ascii(p, e, ep, smap, lane);
+  } else if (fast_in_ring) {
+    gen_maze<true>(p, e, ep, smap, maze_work(ws.ring(), work_in_ring ? ws.ring() + fast_bytes : scratch, nn), lane);
   } else {
-    gen_maze(p, e, ep, smap, work_in_ring ? ws.ring() : scratch, lane);
+    gen_maze<false>(p, e, ep, smap, maze_work(scratch, scratch + fast_bytes, nn), lane);
   }
   write_plane<MAPK>(p, e, smap, ws.map(p), lane);
   if (gen_slot >= 0) give_gen_slot(p, gen_slot, lane);

@@ -362,8 +362,8 @@ cudaError_t pregen_launch(const Params& p, int steps, bool reset, cudaStream_t s
 
 size_t gen_scratch_bytes(int task, int S) {
   if (task != 1 && task != 2) return 0;
-  int nn = (S - 2) / 2;
-  return (maze_scratch_bytes(nn * nn) + 255) & ~(size_t)255;
+  const int nn = maze_nodes(S);
+  return (maze_fast_bytes(nn) + maze_slow_bytes(nn) + 255) & ~(size_t)255;
 }
 
 cudaError_t kernel_blocks_per_sm(const Params& p, int mode, int* blocks) {
