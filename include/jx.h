@@ -205,7 +205,7 @@ jx_status jx_step(jx_env* env, void* stream, const uint8_t* d_actions, uint8_t* 
  * sequence of jx_step calls.
  *  d_actions [steps][N] uint8; d_frames [steps][N][H][W][3] uint8;
  *  d_rewards [steps][N] float32; d_dones [steps][N] uint8.
- * Rollouts of 4 steps or more (of envs that jx_create made, except the ASCII
+ * Rollouts of 2 steps or more (of envs that jx_create made, except the ASCII
  * task) run in two passes: a walk steps every agent up to the step that ends
  * its episode, one lane per env, and leaves a camera record per env and step;
  * a draw renders the records' frames in any order. The env kernel, launched

@@ -184,12 +184,12 @@ jx_status launch_env(jx_env* env, const jx::Params& p, int mode, cudaStream_t s)
 }
 
 // A rollout of p.steps steps: walk, draw and the env kernel for what they left,
-// in segments that the camera records hold; short ones, and envs without
-// records, in the env kernel alone.
+// in segments that the camera records hold; envs without records in the env
+// kernel alone.
 jx_status run_rollout(jx_env* env, jx::Params p, cudaStream_t s) {
   const int steps = p.steps;
-  if (!p.stop || steps < jx::kRolloutMinSteps) {
-    p.stop = nullptr;
+  if (steps < jx::kRolloutMinSteps) return launch_env(env, p, jx::MODE_STEP, s);
+  if (!p.stop) {
     p.chunk = rollout_chunk(env, steps);
     return launch_env(env, p, jx::MODE_ROLLOUT, s);
   }

@@ -199,8 +199,9 @@ jx_status batch_run(jx_batch* b, int mode, cudaStream_t stream, const uint8_t* a
       if (count) b->launches.fetch_add(jx::kPregenKernels, std::memory_order_relaxed);
     }
   }
+  if (mode == jx::MODE_ROLLOUT && steps < jx::kRolloutMinSteps) mode = jx::MODE_STEP;
   if (mode == jx::MODE_ROLLOUT) {
-    if (b->segment > 0 && steps >= jx::kRolloutMinSteps) {
+    if (b->segment > 0) {
       jx::BatchParams bq = b->draw;
       for (int i = 0; i < bp.n_groups; ++i) {
         bq.g[i].actions = bp.g[i].actions;

@@ -719,7 +719,7 @@ def test_unlocked_door_on_the_border_opens_the_map():
 def _two_pass_cases():
     m, r = inputs.maze_keydoor, inputs.rooms
     return [
-        (m(n_envs=1, map_side=32, seed=41, horizon=500), 4),  # the shortest, one env
+        (m(n_envs=1, map_side=32, seed=41, horizon=500), 2),  # the shortest, one env
         (m(n_envs=33, map_side=32, seed=42, horizon=7), 9),  # ragged warps, every env ends twice
         (m(n_envs=31, map_side=6, seed=43, horizon=40), 130),  # two segments; keys, goals
         (dict(r(n_envs=65, map_side=9, seed=44, max_sprites=3, frame_h=21, frame_w=16), turns_per_rev=7), 17),
@@ -733,7 +733,7 @@ def _two_pass_cases():
 
 @pytest.mark.parametrize("case", range(9))
 def test_two_pass_rollout_equals_single_steps(case):
-    """Rollouts of 4 or more steps walk first and draw afterwards: three of them
+    """Rollouts of 2 or more steps walk first and draw afterwards: three of them
     in a row (the second from a state set by the host, holding keys beside maps
     with further locked doors) equal the sequence of steps, state included."""
     cfg, T = _two_pass_cases()[case]
