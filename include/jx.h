@@ -341,11 +341,13 @@ jx_status jx_sync_status(jx_env* env, void* stream);
  * count, the walls of builds that start, then the build's share of the launch,
  * after a 4-byte cudaMemsetAsync on the same stream; all capturable in a CUDA
  * graph). A jx_rollout in two passes (see there) counts its walk and draw
- * launches and the env kernel's, per 128 steps. */
+ * launches and the env kernel's, per 128 steps. Steps of small batches with
+ * large frames count a second launch, which begins the next episodes. */
 jx_status jx_launch_count(const jx_env* env, uint64_t* count);
 
 /* Launch shape of the fused step kernel: grid blocks, threads per block,
- * dynamic shared memory bytes per block. */
+ * dynamic shared memory bytes per block. (Batches that would leave most of the
+ * chip idle step and render with a block of 2 or 4 warps per env.) */
 jx_status jx_launch_shape(const jx_env* env, int32_t* grid, int32_t* block, int32_t* smem_bytes);
 
 /* Launch shape of the env kernel in a jx_rollout of `steps` steps (see

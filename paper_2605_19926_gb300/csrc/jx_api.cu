@@ -172,14 +172,21 @@ int rollout_chunk(const jx_env* env, int steps) {
 // One launch of the env kernel (MODE_ROLLOUT: in hand-off chunks, of all steps
 // or of what the walk and the draw left).
 jx_status launch_env(jx_env* env, const jx::Params& p, int mode, cudaStream_t s) {
-  cudaError_t err = jx::launch(p, mode, mode == jx::MODE_ROLLOUT && p.chunk > 0 ? env->grid_handoff : env->grid, s);
+  int launches = 0;
+  cudaError_t err;
+  if (mode == jx::MODE_ROLLOUT) {
+    err = jx::launch(p, mode, p.chunk > 0 ? env->grid_handoff : env->grid, s);
+    launches = 1;
+  } else {
+    err = jx::host::launch_frame(env, p, mode, s, &launches);
+  }
   if (err != cudaSuccess) {
     // a failed rollout launch may leave the hand-off words set (the kernel
     // zeroes them as it ends): clear them on the same stream
     if (mode == jx::MODE_ROLLOUT && p.chunk > 0) (void)cudaMemsetAsync(p.work, 0, env->work_bytes, s);
     return cuda_fail(err, "kernel launch");
   }
-  env->launches.fetch_add(1, std::memory_order_relaxed);
+  env->launches.fetch_add(launches, std::memory_order_relaxed);
   return JX_OK;
 }
 
@@ -276,6 +283,38 @@ void choose_rows(Params& p, int max_rows, int warps, int blocks, size_t smem_per
   p.frame_block_bytes = rows * rowb;
   p.gray_block_bytes = p.gray ? rows * p.W : 0;
   layout_warp_smem(p);
+}
+
+// A team draws a frame in less time than one warp, but a step whose episodes
+// can end needs the launch that begins the next ones, about 1.5 us. In a graph
+// of steps (us, env kernel / team): key-door mazes with 64 x 64 frames, 64 envs
+// 6.7 / 7.1, 256 7.1 / 7.5; with 128 x 128 frames, 16 envs 11.8 / 7.9, 256 14.6
+// / 9.6, 1024 24.9 / 14.1; 250 ASCII envs, 48 x 80, 8.8 / 8.5. So such steps
+// take a team where a frame has more than 64 x 64 pixels (a grayscale plane
+// counted as a third more); one room env whose episode never ends takes 5.4 /
+// 4.4 us a call. Renders begin nothing: 55 envs, 128 x 128, 18.8 / 6.4 us.
+bool steps_end(const jx_env* env) { return env->cfg.task != JX_TASK_ROOMS || env->cfg.horizon > 0; }
+
+bool takes_team(const jx_env* env, int mode) {
+  if (env->team.staging == 0) return false;
+  if (mode == MODE_RENDER) return true;
+  const int px = env->cfg.frame_h * env->cfg.frame_w * (env->cfg.gray_stack ? 4 : 3);
+  return mode == MODE_STEP && (!steps_end(env) || px > 3 * 64 * 64);
+}
+
+cudaError_t launch_frame(const jx_env* env, const Params& p, int mode, cudaStream_t stream, int* launches) {
+  *launches += 1;
+  if (!takes_team(env, mode)) return launch(p, mode, env->grid, stream);
+  Params q = env->team;
+  q.actions = p.actions;
+  q.frames = p.frames;
+  q.rewards = p.rewards;
+  q.dones = p.dones;
+  q.bulk_wait_rounds = p.bulk_wait_rounds;
+  cudaError_t err = team_launch(q, mode, stream);
+  if (err != cudaSuccess || mode != MODE_STEP || !steps_end(env)) return err;
+  *launches += 1;
+  return launch(p, MODE_BEGIN, env->grid, stream);
 }
 
 }  // namespace host
@@ -604,6 +643,29 @@ jx_status create_impl(const jx_config* cfg, int device, void* ext, size_t ext_by
       return cuda_fail(err, "kernel attributes");
     }
     env->draw_slots = jx::kMinBlocksPerSm * env->num_sms;
+  }
+  {
+    // a team per env while its warps all fit at once; its rows: an equal share
+    // each, or as many as leave room for every block
+    // Byte maps that come by bulk copy keep the env kernel: a lost copy leaves
+    // the done flag alone, which the launch after a team's step reads.
+    int team = p.map_bits || p.S * p.S < 4096 ? jx::kMaxTeam : 1;
+    while (team > 1 && (int64_t)c.n_envs * team > (int64_t)jx::kMinBlocksPerSm * env->num_sms) team /= 2;
+    if (team > 1) {
+      jx::Params q = p;
+      q.staging = team;
+      const size_t per_sm = (c.n_envs + env->num_sms - 1) / env->num_sms;
+      size_t room = prop.sharedMemPerMultiprocessor / per_sm - prop.reservedSharedMemPerBlock;
+      if (room > prop.sharedMemPerBlockOptin) room = prop.sharedMemPerBlockOptin;
+      for (int rows = (c.frame_h + team - 1) / team; rows >= 1; --rows) {
+        q.rows_per_block = rows;
+        q.frame_block_bytes = rows * 3 * W;
+        q.gray_block_bytes = q.gray ? rows * W : 0;
+        jx::layout_warp_smem(q);
+        if ((size_t)jx::team_block_bytes(q) <= room) break;
+      }
+      if ((size_t)jx::team_block_bytes(q) <= room && jx::team_prepare(q) == cudaSuccess) env->team = q;
+    }
   }
   // the memset and the table copy are done before the handle is returned
   if ((err = cudaStreamSynchronize(0)) != cudaSuccess) {
@@ -1068,9 +1130,10 @@ jx_status jx_launch_count(const jx_env* env, uint64_t* count) {
 jx_status jx_launch_shape(const jx_env* env, int32_t* grid, int32_t* block, int32_t* smem_bytes) {
   if (jx_status st = check_env(env)) return st;
   if (env->use_batch) return jx_batch_launch_shape(env->tuned, grid, block, smem_bytes);
-  if (grid) *grid = env->grid;
-  if (block) *block = jx::kThreads;
-  if (smem_bytes) *smem_bytes = env->smem_block;
+  const bool team = jx::host::takes_team(env, jx::MODE_STEP);
+  if (grid) *grid = team ? env->cfg.n_envs : env->grid;
+  if (block) *block = team ? 32 * env->team.staging : jx::kThreads;
+  if (smem_bytes) *smem_bytes = team ? jx::team_block_bytes(env->team) : env->smem_block;
   return JX_OK;
 }
 

@@ -1706,9 +1706,11 @@ __device__ __forceinline__ float2 col_k_pair(const Params& p, int lane) {
 
 // Cast every column's ray: in each pass lane l marches the rays of columns
 // l + 32 j (j < COLS) together. Returns the lane's largest hit distance.
+// Of several warps that share the frame, each takes the passes first, first +
+// every, ... (one column pass of COLS).
 template <int MODE, int MAPK, int COLS>
 __device__ __forceinline__ float cast_columns(const Params& p, int e, const Env& r, float c, float s,
-                                              const WarpSmem& ws, int lane, float2 k01) {
+                                              const WarpSmem& ws, int lane, float2 k01, int first = 0, int every = 1) {
   const int W = p.W, S = p.S;
   // a solid border and the agent strictly inside it: rays need no bounds test
   const bool inside = ws.obj(p)[7] != 0 && (unsigned)(r.cx - 1) < (unsigned)(S - 2) &&
@@ -1722,7 +1724,8 @@ __device__ __forceinline__ float cast_columns(const Params& p, int e, const Env&
   float far = 0.f;
   // col_slot of column lane; column lane + 32 m lies 8 m further
   const int slot0 = col_slot(lane, W >> 4);
-  for (int m = 0; 32 * m < W; m += COLS) {
+  int m_last = 0;
+  for (int m = first * COLS; 32 * m < W; m += every * COLS) {
     Ray q[COLS];
     Hit h[COLS];
     bool valid[COLS];
@@ -1737,12 +1740,13 @@ __device__ __forceinline__ float cast_columns(const Params& p, int e, const Env&
 #pragma unroll
     for (int j = 0; j < COLS; ++j) {
       const int col = lane + 32 * (m + j);
-      if (kDefer && pending) finish_column<MODE>(p, e, last, col - 32, slot0 + 8 * (m + j - 1), ws);
+      if (kDefer && pending) finish_column<MODE>(p, e, last, lane + 32 * m_last, slot0 + 8 * m_last, ws);
       pending = false;
       if (valid[j]) {
         far = fmaxf(far, h[j].perp);
         if (kDefer) {
           last = h[j];
+          m_last = m + j;
           pending = true;
         } else {
           finish_column<MODE>(p, e, h[j], col, slot0 + 8 * (m + j), ws);
@@ -1750,10 +1754,7 @@ __device__ __forceinline__ float cast_columns(const Params& p, int e, const Env&
       }
     }
   }
-  if (kDefer && pending) {
-    const int m = (W - 1 - lane) >> 5;  // the lane's last column
-    finish_column<MODE>(p, e, last, lane + 32 * m, slot0 + 8 * m, ws);
-  }
+  if (kDefer && pending) finish_column<MODE>(p, e, last, lane + 32 * m_last, slot0 + 8 * m_last, ws);
   __syncwarp();
   return far;
 }
@@ -1838,7 +1839,13 @@ __device__ __forceinline__ int project_sprites(const Params& p, const Env& r, fl
     }
   if (vis) ws.order(p)[rank] = lane;
   __syncwarp();
-  return __popc(vmask);
+  const int nvis = __popc(vmask);
+  if (lane < nvis) {  // rows each sprite of that order can cover
+    const int4 rc = ws.spr_rect(p)[ws.order(p)[lane]];
+    ws.spr_span(p)[lane] = rc.x <= rc.y ? ((uint32_t)rc.z << 16) | (uint32_t)rc.w : 0xFFFF0000u;
+  }
+  __syncwarp();
+  return nvis;
 }
 
 // Four pixels of colour c as the three words of their 12 RGB bytes.
@@ -1857,6 +1864,50 @@ __device__ __forceinline__ uint32_t sign_bytes(uint32_t x) {
   return d;
 }
 __device__ __forceinline__ uint32_t select_bytes(uint32_t m, uint32_t a, uint32_t b) { return (m & a) | (~m & b); }
+
+// Draw the sprites over rows [r0, r1) of the frame in `buf`.
+template <bool GRAYF>
+__device__ __forceinline__ void draw_sprites(const Params& p, const WarpSmem& ws, uint8_t* buf, uint8_t* gbuf, int r0,
+                                             int r1, int nvis, int lane) {
+  const int W = p.W, rowb = 3 * W;
+  // sprites, far to near; lanes take columns. For a column, the covered rows
+  // are those whose centre has v in [0, 1) with |2v - 1| below the mask's
+  // half-height at this u (key: 1 - |2u - 1|, disc: sqrt(1 - (2u - 1)^2)).
+  // the sprites whose rows meet this block, far to near
+  const uint32_t span = lane < nvis ? ws.spr_span(p)[lane] : 0xFFFF0000u;
+  uint32_t hits = __ballot_sync(0xffffffffu, (int)(span >> 16) < r1 && (int)(span & 0xffffu) >= r0);
+  while (hits) {
+    const int oi = __ffs(hits) - 1;
+    hits &= hits - 1;
+    const int j = ws.order(p)[oi];
+    const int4 rc = ws.spr_rect(p)[j];
+    const int rA = rc.z < r0 ? r0 : rc.z;
+    const int rB = rc.w > r1 - 1 ? r1 - 1 : rc.w;
+    if (rc.x > rc.y || rA > rB) continue;
+    const float4 a = ws.spr_a(p)[j];  // x0, top, 1/width, 1/height
+    const float ty = ws.spr_ty(p)[j];
+    const uint32_t rgbv = ws.spr_rgb(p)[j];
+    const int kind = ws.spr_kind(p)[j];
+    for (int col = rc.x + lane; col <= rc.y; col += 32) {
+      const float u = ((float)col + 0.5f - a.x) * a.z;
+      if (!(u >= 0.f && u < 1.f && ty < ws.zbuf(p)[col])) continue;
+      const float au = fabsf(fmaf(2.f, u, -1.f));
+      const float half = kind == 1 ? 1.f - au : (kind == 2 ? 2.f : sqrtf(fmaxf(0.f, fmaf(-au, au, 1.f))));
+      uint8_t* px = buf + col * 3;
+      for (int row = rA; row <= rB; ++row) {
+        const float v = ((float)row + 0.5f - a.y) * a.w;
+        if (v >= 0.f && v < 1.f && fabsf(fmaf(2.f, v, -1.f)) < half) {
+          uint8_t* q = px + (row - r0) * rowb;
+          q[0] = (uint8_t)(rgbv & 255);
+          q[1] = (uint8_t)((rgbv >> 8) & 255);
+          q[2] = (uint8_t)((rgbv >> 16) & 255);
+          if (GRAYF) gbuf[(row - r0) * W + col] = (uint8_t)(rgbv >> 24);
+        }
+      }
+    }
+    __syncwarp();
+  }
+}
 
 // Fill rows [r0, r1) of the frame into `buf` (row-major RGB), then draw the
 // sprites over them.
@@ -1941,46 +1992,33 @@ __device__ __forceinline__ void fill_block(const Params& p, const WarpSmem& ws, 
     }
   }
   __syncwarp();
-  if (nvis == 0) return;  // warp-uniform
-  // sprites, far to near; lanes take columns. For a column, the covered rows
-  // are those whose centre has v in [0, 1) with |2v - 1| below the mask's
-  // half-height at this u (key: 1 - |2u - 1|, disc: sqrt(1 - (2u - 1)^2)).
-  // the sprites whose rows meet this block, far to near
-  const uint32_t span = lane < nvis ? ws.spr_span(p)[lane] : 0xFFFF0000u;
-  uint32_t hits = __ballot_sync(0xffffffffu, (int)(span >> 16) < r1 && (int)(span & 0xffffu) >= r0);
-  while (hits) {
-    const int oi = __ffs(hits) - 1;
-    hits &= hits - 1;
-    const int j = ws.order(p)[oi];
-    const int4 rc = ws.spr_rect(p)[j];
-    const int rA = rc.z < r0 ? r0 : rc.z;
-    const int rB = rc.w > r1 - 1 ? r1 - 1 : rc.w;
-    if (rc.x > rc.y || rA > rB) continue;
-    const float4 a = ws.spr_a(p)[j];  // x0, top, 1/width, 1/height
-    const float ty = ws.spr_ty(p)[j];
-    const uint32_t rgbv = ws.spr_rgb(p)[j];
-    const int kind = ws.spr_kind(p)[j];
-    for (int col = rc.x + lane; col <= rc.y; col += 32) {
-      const float u = ((float)col + 0.5f - a.x) * a.z;
-      if (!(u >= 0.f && u < 1.f && ty < ws.zbuf(p)[col])) continue;
-      const float au = fabsf(fmaf(2.f, u, -1.f));
-      const float half = kind == 1 ? 1.f - au : (kind == 2 ? 2.f : sqrtf(fmaxf(0.f, fmaf(-au, au, 1.f))));
-      uint8_t* px = buf + col * 3;
-      for (int row = rA; row <= rB; ++row) {
-        const float v = ((float)row + 0.5f - a.y) * a.w;
-        if (v >= 0.f && v < 1.f && fabsf(fmaf(2.f, v, -1.f)) < half) {
-          uint8_t* q = px + (row - r0) * rowb;
-          q[0] = (uint8_t)(rgbv & 255);
-          q[1] = (uint8_t)((rgbv >> 8) & 255);
-          q[2] = (uint8_t)((rgbv >> 16) & 255);
-          if (GRAYF) gbuf[(row - r0) * W + col] = (uint8_t)(rgbv >> 24);
-        }
-      }
-    }
-    __syncwarp();
-  }
+  if (nvis > 0) draw_sprites<GRAYF>(p, ws, buf, gbuf, r0, r1, nvis, lane);  // warp-uniform
 }
 #undef JX_QUAD_WORDS
+
+// Rows [r0, r1) of env e's frame (and of its grayscale plane of episode step t)
+// on their way out of the warp's staging buffers, as one bulk group.
+__device__ __forceinline__ void copy_out(const Params& p, int e, int t, uint8_t* frame, const uint8_t* buf,
+                                         const uint8_t* gbuf, int r0, int r1, bool gray_on, int lane) {
+  const int H = p.H, W = p.W, rowb = 3 * W;
+  fence_proxy_async_smem();
+  __syncwarp();
+  if (lane == 0) {
+    bulk_copy(frame + (size_t)r0 * rowb, buf, (uint32_t)((r1 - r0) * rowb));
+    if (gray_on) {
+      // grayscale stack: plane t mod 4, or all four planes for an episode's first frame
+      const size_t plane = (size_t)H * W;
+      uint8_t* g0 = p.st.gray + (size_t)e * 4 * plane + (size_t)r0 * W;
+      const uint32_t gbytes = (uint32_t)((r1 - r0) * W);
+      if (t == 0) {
+        for (int k = 0; k < 4; ++k) bulk_copy(g0 + k * plane, gbuf, gbytes);
+      } else {
+        bulk_copy(g0 + (size_t)(t & 3) * plane, gbuf, gbytes);
+      }
+    }
+    bulk_commit();
+  }
+}
 
 // GRAY: 0 no grayscale stack, 1 a stack, 2 as p.st.gray says (batched kernel).
 // gray_now: this frame's plane is wanted (false only where a later frame of
@@ -1992,14 +2030,7 @@ __device__ __forceinline__ void render_env(const Params& p, int e, const Env& r,
   const float far = cast_columns<MODE, MAPK, COLS>(p, e, r, c, s, ws, lane, k01);
   if (MODE == MODE_RAYS) return;
   const int nvis = project_sprites(p, r, c, s, ws, lane, far);  // ends with __syncwarp when any is visible
-  const int H = p.H, W = p.W, rowb = 3 * W;
-  if (nvis > 0) {  // rows each sprite of the far-to-near order can cover
-    if (lane < nvis) {
-      const int4 rc = ws.spr_rect(p)[ws.order(p)[lane]];
-      ws.spr_span(p)[lane] = rc.x <= rc.y ? ((uint32_t)rc.z << 16) | (uint32_t)rc.w : 0xFFFF0000u;
-    }
-    __syncwarp();
-  }
+  const int H = p.H;
   const bool gray_on = gray_now && (GRAY == 1 || (GRAY == 2 && p.st.gray != nullptr));
   for (int r0 = 0; r0 < H; r0 += p.rows_per_block) {
     const int r1 = r0 + p.rows_per_block < H ? r0 + p.rows_per_block : H;
@@ -2011,23 +2042,7 @@ __device__ __forceinline__ void render_env(const Params& p, int e, const Env& r,
       fill_block<true>(p, ws, buf, gbuf, r0, r1, nvis, lane);
     else
       fill_block<false>(p, ws, buf, gbuf, r0, r1, nvis, lane);
-    fence_proxy_async_smem();
-    __syncwarp();
-    if (lane == 0) {
-      bulk_copy(frame + (size_t)r0 * rowb, buf, (uint32_t)((r1 - r0) * rowb));
-      if (gray_on) {
-        // grayscale stack: plane t mod 4, or all four planes for an episode's first frame
-        const size_t plane = (size_t)H * W;
-        uint8_t* g0 = p.st.gray + (size_t)e * 4 * plane + (size_t)r0 * W;
-        const uint32_t gbytes = (uint32_t)((r1 - r0) * W);
-        if (r.t == 0) {
-          for (int k = 0; k < 4; ++k) bulk_copy(g0 + k * plane, gbuf, gbytes);
-        } else {
-          bulk_copy(g0 + (size_t)(r.t & 3) * plane, gbuf, gbytes);
-        }
-      }
-      bulk_commit();
-    }
+    copy_out(p, e, r.t, frame, buf, gbuf, r0, r1, gray_on, lane);
     slot = slot + 1 == p.staging ? 0 : slot + 1;
   }
 }
@@ -2189,6 +2204,106 @@ __device__ __forceinline__ void next_episode(const Params& p, int e, Env& r, con
   mark_border<MAPK>(p, ws, lane);
 }
 
+// One frame by the warps of a block together (MODE_STEP, MODE_RENDER): one
+// env's step and frame are a chain of some 5 us on one warp at 64 x 64 and 25
+// at 96 x 96 with a grayscale plane; small batches leave most of the chip idle
+// meanwhile. Warp 0 steps the agent, the warps share out the columns' rays
+// (a pass of 32 columns each), then the rows (each warp its own staging
+// buffer; p.staging is their number), while warp 0 looks for visible sprites.
+// There is no generator here: an env whose episode ended is left, with its
+// reward and done flag stored, to the env kernel launched next (MODE_BEGIN).
+struct TeamShared {
+  int32_t cx, cy, t, keys;
+  float fx, fy, c, s;
+  int32_t nvis, skip;
+  float far[kMaxTeam];
+};
+
+template <int MODE, int MAPK, int GRAY>
+__device__ __forceinline__ void run_team(const Params& p, int e, uint8_t* base, TeamShared& sh, int warp, int warps,
+                                         int lane) {
+  const WarpSmem ws{base, fill_lane(p, lane)};
+  Env r;
+  float c = 0.f, s = 0.f;
+  if (warp == 0) {
+    const Prefetch q = prefetch<MODE, MAPK>(p, e, 0, lane);
+    r = q.r;
+    bool ok = stage_prefetched<MAPK>(p, ws, e, q, lane);
+    if (ok) {
+      const int keys0 = r.keys;
+      if (MODE == MODE_STEP) {
+        if (r.keys != 0) open_doors<MAPK>(p, e, r.keys, ws, lane);  // for the move
+        const int a = turn_for(p, r, q.action, lane);
+        heading_from(r, turn_entry(p, q, r.turn), c, s);
+        ok = !step_env<MAPK>(p, e, r, ws.map(p), ws.obj(p), ws.spr_in(p), lane, c, s, a, (size_t)e, true);
+      } else {
+        heading(p, r, c, s);
+      }
+      if (ok && r.keys != 0) {  // doors of held keys open: the border flag again
+        if (MODE != MODE_STEP || r.keys != keys0) open_doors<MAPK>(p, e, r.keys, ws, lane);
+        mark_border<MAPK>(p, ws, lane);
+      }
+    }
+    if (lane == 0) {
+      sh.cx = r.cx;
+      sh.cy = r.cy;
+      sh.t = r.t;
+      sh.keys = r.keys;
+      sh.fx = r.fx;
+      sh.fy = r.fy;
+      sh.c = c;
+      sh.s = s;
+      sh.skip = ok ? 0 : 1;
+    }
+  }
+  const float2 k01 = col_k_pair(p, lane);
+  __syncthreads();
+  if (sh.skip) return;  // the whole block: the episode ended, or the map's copy was lost
+  if (warp != 0) {
+    r.cx = sh.cx;
+    r.cy = sh.cy;
+    r.t = sh.t;
+    r.keys = sh.keys;
+    r.fx = sh.fx;
+    r.fy = sh.fy;
+    c = sh.c;
+    s = sh.s;
+  }
+  const float far = cast_columns<MODE_RENDER, MAPK, 1>(p, e, r, c, s, ws, lane, k01, warp, warps);
+  const float warp_far = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(far)));
+  if (lane == 0) sh.far[warp] = warp_far;
+  __syncthreads();
+  const int H = p.H, W = p.W;
+  uint8_t* const frame = p.frames + (size_t)e * 3 * H * W;
+  uint8_t* const buf = ws.ring() + warp * p.frame_block_bytes;
+  uint8_t* const gbuf = GRAY ? ws.gray_ring(p) + warp * p.gray_block_bytes : nullptr;
+  if (warp == 0) {
+    float all = 0.f;
+    for (int w = 0; w < warps; ++w) all = fmaxf(all, sh.far[w]);
+    const int nvis = project_sprites(p, r, c, s, ws, lane, all);
+    if (lane == 0) sh.nvis = nvis;
+  }
+  bool first = true;
+  for (int r0 = warp * p.rows_per_block; first || r0 < H; r0 += warps * p.rows_per_block) {
+    const int r1 = r0 + p.rows_per_block < H ? r0 + p.rows_per_block : H;
+    if (r0 < H) {
+      if (!first) {
+        if (lane == 0) bulk_wait_read_all();
+        __syncwarp();
+      }
+      fill_block<GRAY == 1>(p, ws, buf, gbuf, r0, r1, 0, lane);
+    }
+    if (first) __syncthreads();  // every warp once: the sprites are known
+    first = false;
+    if (r0 >= H) break;
+    const int nvis = sh.nvis;
+    if (nvis > 0) draw_sprites<GRAY == 1>(p, ws, buf, gbuf, r0, r1, nvis, lane);
+    copy_out(p, e, r.t, frame, buf, gbuf, r0, r1, GRAY == 1, lane);
+  }
+  // shared memory stays allocated until the bulk stores have read it
+  if (lane == 0) bulk_wait_read_all();
+}
+
 // Everything one launch does for env e: MODE_ROLLOUT runs the launch's steps
 // t0 .. t1 - 1 with the env's scalar state in registers and its map in shared
 // memory (the state is loaded before step t0 and stored after step t1 - 1).
@@ -2198,8 +2313,13 @@ __device__ __forceinline__ bool run_env(const Params& p, int e, uint8_t* wbase, 
                                         int& slot, int t0 = 0, int t1 = 0) {
   const WarpSmem ws{wbase, fill_lane(p, lane)};
   const size_t frame_bytes = (size_t)3 * p.H * p.W;
-  if (MODE == MODE_RESET) {
-    generate<MAPK>(p, e, 0u, wbase, scratch, lane);
+  if (MODE == MODE_RESET || MODE == MODE_BEGIN) {
+    uint32_t ep = 0u;
+    if (MODE == MODE_BEGIN) {
+      if (p.dones[e] == 0) return true;
+      ep = p.st.episode[e] + 1;
+    }
+    generate<MAPK>(p, e, ep, wbase, scratch, lane);
     const Env r = load_env(p, e);
     load_objects(p, ws, e, lane);
     __syncwarp();

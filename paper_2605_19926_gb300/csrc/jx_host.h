@@ -20,6 +20,7 @@ struct jx_env {
   int smem_block = 0;
   jx::Params base{};
   jx::Params draw{};   // base with the draw pass's shared-memory layout (rollouts in two passes)
+  jx::Params team{};   // base with a team's layout (small batches: steps and renders), staging 0: none
   int draw_slots = 0;  // warps of the draw pass resident at once, about
   // one device block: state | aux | bit planes | scratch (owned, or in the
   // caller's memory), and in owned memory the camera records of rollouts
@@ -95,6 +96,12 @@ inline size_t frame_bytes(const jx_config& c) { return (size_t)3 * c.frame_h * c
 // layout fit in `smem_per_sm` bytes, each block of `warps` warps also taking
 // `reserved` bytes. Sets rows_per_block, frame_block_bytes and the layout.
 void choose_rows(Params& p, int max_rows, int warps, int blocks, size_t smem_per_sm, size_t reserved);
+
+// The launch of a step, render, reset or ray query over p (env's parameters
+// with the call's pointers): a team per env for small batches, else the env
+// kernel. Adds the kernels launched to *launches.
+bool takes_team(const jx_env* env, int mode);
+cudaError_t launch_frame(const jx_env* env, const Params& p, int mode, cudaStream_t stream, int* launches);
 
 // jx_env_bytes / jx_create_in, for the ASCII task too (ascii: the map text, or null).
 jx_status env_bytes(const jx_config* cfg, const char* ascii, int device, size_t* bytes);

@@ -22,7 +22,9 @@ constexpr int kHandoffPolls = 1 << 22;  // default polls (about 0.25 us apart) b
 constexpr int kHandoffMinSteps = 64;    // rollouts of at least this many steps run in hand-off chunks
 constexpr int kHandoffChunk = 12;       // steps per hand-off chunk
 
-enum Mode { MODE_STEP = 0, MODE_RESET = 1, MODE_RENDER = 2, MODE_RAYS = 3, MODE_ROLLOUT = 4 };
+// MODE_BEGIN starts the next episode of the envs whose done flag is set (after a
+// team's step) and draws its first frame.
+enum Mode { MODE_STEP = 0, MODE_RESET = 1, MODE_RENDER = 2, MODE_RAYS = 3, MODE_ROLLOUT = 4, MODE_BEGIN = 5 };
 
 // How a warp holds its env's map in shared memory: one byte per cell, or one
 // bit per cell (wall or closed door) with the wall type read from the state
@@ -191,6 +193,14 @@ cudaError_t pregen_launch(const Params& p, int steps, bool reset, cudaStream_t s
 // stack, took 33.9 us with a memset and three kernels that returned at once,
 // 28.6 us without them).
 inline bool pregen_runs(const Params& p) { return p.nx_ep != nullptr && p.nx_lanes > 0 && p.n >= p.nx_min; }
+
+// Teams: blocks of up to kMaxTeam warps that share one env's step and frame, for
+// batches too small to fill the chip with a warp per env. rows_per_block,
+// staging and the layout are the team's; MODE_STEP and MODE_RENDER.
+constexpr int kMaxTeam = 4;
+int team_block_bytes(const Params& q);  // dynamic shared memory of a team's block
+cudaError_t team_prepare(const Params& q);  // kernel attributes
+cudaError_t team_launch(const Params& q, int mode, cudaStream_t stream);  // q.staging warps a block, one env
 
 // Configure (attributes) and query occupancy of the kernel for `mode`.
 cudaError_t kernel_blocks_per_sm(const Params& p, int mode, int* blocks);

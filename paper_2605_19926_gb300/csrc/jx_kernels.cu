@@ -75,7 +75,7 @@ template <int MODE, int MAPK, int GRAY>
 __global__ void __launch_bounds__(kThreads, kMinBlocksPerSm / kWarpsPerBlock)
     env_kernel(const __grid_constant__ Params p) {
   extern __shared__ __align__(128) uint8_t smem_raw[];
-  constexpr bool kEarlyRelease = MODE == MODE_STEP || MODE == MODE_RENDER || MODE == MODE_RAYS;
+  constexpr bool kEarlyRelease = MODE == MODE_STEP || MODE == MODE_RENDER || MODE == MODE_RAYS || MODE == MODE_BEGIN;
   if (kEarlyRelease) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   uint8_t* const wbase = smem_raw + warp * p.warp_bytes;
@@ -139,6 +139,28 @@ __global__ void __launch_bounds__(256) plane_kernel(const __grid_constant__ Para
     const int e = (int)(idx / p.plane_words), i = (int)(idx % p.plane_words);
     p.plane[idx] = plane_word(p, p.st.map + (size_t)e * p.S * p.S, i);
   }
+}
+
+// One env per block of p.staging warps (see run_team).
+template <int MODE, int MAPK, int GRAY>
+__global__ void __launch_bounds__(32 * kMaxTeam, kMinBlocksPerSm / kMaxTeam)
+    team_kernel(const __grid_constant__ Params p) {
+  extern __shared__ __align__(128) uint8_t smem_raw[];
+  TeamShared& sh = *reinterpret_cast<TeamShared*>(smem_raw + p.warp_bytes);
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (warp == 0) {
+    write_palette(p, WarpSmem{smem_raw, FillLane{}}, lane);
+    if (!p.map_bits && p.S * p.S >= 4096) init_warp_header(smem_raw, lane);
+  }
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  run_team<MODE, MAPK, GRAY>(p, (int)blockIdx.x, smem_raw, sh, warp, (int)(blockDim.x >> 5), lane);
+}
+
+template <int MODE>
+auto team_kernel_of(const Params& p) {
+  if (p.map_bits) return p.gray ? team_kernel<MODE, MAP_BITS, 1> : team_kernel<MODE, MAP_BITS, 0>;
+  return p.gray ? team_kernel<MODE, MAP_BYTES, 1> : team_kernel<MODE, MAP_BYTES, 0>;
 }
 
 // Whether env e needs a pre-built episode, and which: episode 0 at a reset,
@@ -366,12 +388,35 @@ size_t gen_scratch_bytes(int task, int S) {
   return (maze_fast_bytes(nn) + maze_slow_bytes(nn) + 255) & ~(size_t)255;
 }
 
+int team_block_bytes(const Params& q) { return q.warp_bytes + align16((int)sizeof(TeamShared)); }
+
+cudaError_t team_prepare(const Params& q) {
+  cudaError_t err = raise_smem_limit(team_kernel_of<MODE_STEP>(q));
+  if (err == cudaSuccess) err = raise_smem_limit(team_kernel_of<MODE_RENDER>(q));
+  return err == cudaSuccess ? raise_smem_limit(env_kernel_of<MODE_BEGIN>(q)) : err;
+}
+
+cudaError_t team_launch(const Params& q, int mode, cudaStream_t stream) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)q.n);
+  cfg.blockDim = dim3((unsigned)(32 * q.staging));
+  cfg.dynamicSmemBytes = (size_t)team_block_bytes(q);
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, mode == MODE_STEP ? team_kernel_of<MODE_STEP>(q) : team_kernel_of<MODE_RENDER>(q), q);
+}
+
 cudaError_t kernel_blocks_per_sm(const Params& p, int mode, int* blocks) {
   switch (mode) {
     case MODE_STEP: return blocks_per_sm_mode<MODE_STEP>(p, blocks);
     case MODE_RESET: return blocks_per_sm_mode<MODE_RESET>(p, blocks);
     case MODE_RENDER: return blocks_per_sm_mode<MODE_RENDER>(p, blocks);
     case MODE_ROLLOUT: return blocks_per_sm_mode<MODE_ROLLOUT>(p, blocks);
+    case MODE_BEGIN: return blocks_per_sm_mode<MODE_BEGIN>(p, blocks);
     default: return blocks_per_sm_mode<MODE_RAYS>(p, blocks);
   }
 }
@@ -382,6 +427,7 @@ cudaError_t launch(const Params& p, int mode, int grid, cudaStream_t stream) {
     case MODE_RESET: return launch_mode<MODE_RESET>(p, grid, stream);
     case MODE_RENDER: return launch_mode<MODE_RENDER>(p, grid, stream);
     case MODE_ROLLOUT: return launch_mode<MODE_ROLLOUT>(p, grid, stream);
+    case MODE_BEGIN: return launch_mode<MODE_BEGIN>(p, grid, stream);
     default: return launch_mode<MODE_RAYS>(p, grid, stream);
   }
 }

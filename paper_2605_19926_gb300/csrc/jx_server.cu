@@ -198,7 +198,8 @@ jx_status issue(jx_server* sv, Slot& sl, const std::vector<Session*>& chosen) {
   if (chosen.size() == 1) {
     jx::Params p = chosen[0]->env->base;
     step_params(sl, chosen[0], 0, p);
-    err = jx::launch(p, jx::MODE_STEP, chosen[0]->env->grid, sl.stream);
+    int launches = 0;
+    err = jx::host::launch_frame(chosen[0]->env, p, jx::MODE_STEP, sl.stream, &launches);
   } else {
     jx::BatchParams bp{};
     for (size_t i = 0; i < chosen.size(); ++i) {

@@ -171,6 +171,48 @@ def test_graph_replay_matches_steps():
     graph.close()
 
 
+TEAM_CASES = [
+    inputs.rooms(n_envs=3, map_side=16, seed=61, max_sprites=5, frame_h=1, frame_w=256),  # fewer rows than warps
+    inputs.rooms(n_envs=2, map_side=9, seed=62, frame_h=3, frame_w=16),
+    dict(inputs.maze_keydoor(n_envs=5, map_side=32, seed=63, horizon=6, frame_h=17, frame_w=256), gray_stack=1),
+    dict(inputs.rooms(n_envs=600, map_side=24, seed=64, max_sprites=8, frame_h=70, frame_w=80), horizon=5),
+    dict(inputs.maze_rooms(n_envs=1500, map_side=64, seed=65, horizon=4, max_sprites=16, frame_h=66, frame_w=64,
+                           gray_stack=1)),  # two warps an env
+    inputs.ascii_env("coloured-rooms", n_envs=40, map_side=24, seed=66, horizon=30, frame_h=100, frame_w=48),
+]
+
+
+@pytest.mark.parametrize("cfg", TEAM_CASES)
+def test_teams_equal_one_warp_per_env(cfg):
+    """Small batches with large frames (or endless episodes) step and render with
+    a block of warps per env: frames, rewards, dones and state equal those of
+    the batched kernel, a warp per env, across episode ends."""
+    team, ref = Run(cfg), Run(cfg)
+    ref.env.tiling = tiling(1, 1, 0, 16)
+    assert team.env.launch_shape().grid == cfg["n_envs"] and team.env.launch_shape().block in (64, 128)
+    team.reset()
+    ref.reset()
+    n_done = 0
+    for s in range(12):
+        act = forward_biased_actions(67, s, cfg["n_envs"])
+        fa, ra, da = team.step(act)
+        fb, rb, db = ref.step(act)
+        assert (fa == fb).all() and (ra == rb).all() and (da == db).all(), s
+        n_done += int(da.sum())
+    assert (team.env.get_state() == ref.env.get_state()).all()
+    assert n_done > 0 or cfg["horizon"] in (0, 30)
+    blob = team.env.get_state()
+    team.env.fields(blob)["flags"][:] = np.arange(cfg["n_envs"]) % 8  # keys held: their doors are open
+    frames = []
+    for run in (team, ref):
+        run.env.set_state(blob)
+        run.env.render(run.frames)
+        torch.cuda.synchronize()
+        frames.append(run.frames.clone())
+        run.env.sync_status()
+    assert torch.equal(*frames)
+
+
 @pytest.mark.parametrize("side", [8, 24, 40, 72, 104])
 def test_bit_planes_with_padded_rows(side):
     """Bit planes hold rows of 32, 64 or 128 cells: sides that do not fill them,
