@@ -171,11 +171,11 @@ int rollout_chunk(const jx_env* env, int steps) {
 
 // One launch of the env kernel (MODE_ROLLOUT: in hand-off chunks, of all steps
 // or of what the walk and the draw left).
-jx_status launch_env(jx_env* env, const jx::Params& p, int mode, cudaStream_t s) {
+jx_status launch_env(jx_env* env, const jx::Params& p, int mode, cudaStream_t s, bool joined = false) {
   int launches = 0;
   cudaError_t err;
   if (mode == jx::MODE_ROLLOUT) {
-    err = jx::launch(p, mode, p.chunk > 0 ? env->grid_handoff : env->grid, s);
+    err = jx::launch(p, mode, p.chunk > 0 ? env->grid_handoff : env->grid, joined, s);
     launches = 1;
   } else {
     err = jx::host::launch_frame(env, p, mode, s, &launches);
@@ -187,6 +187,30 @@ jx_status launch_env(jx_env* env, const jx::Params& p, int mode, cudaStream_t s)
     return cuda_fail(err, "kernel launch");
   }
   env->launches.fetch_add(launches, std::memory_order_relaxed);
+  return JX_OK;
+}
+
+// Whether the next episodes of a rollout of p.steps steps are built beside its
+// draw. (16,384 envs of 128 x 128 cells and pixels, 8 steps: 1312 us a
+// launch before the walk, 1234 beside the draw.)
+bool pregen_beside_draw(const jx_env* env, const jx::Params& p) {
+  return env->side && p.stop && p.steps >= jx::kRolloutMinSteps && jx::pregen_runs(p);
+}
+
+// The pre-generation of a rollout of `steps` steps on the env's side stream,
+// after the launches on s so far (its walk); env->join is recorded behind it.
+jx_status pregen_beside(jx_env* env, const jx::Params& p, int steps, cudaStream_t s) {
+  cudaError_t err = cudaEventRecord(env->fork, s);
+  if (err == cudaSuccess) err = cudaStreamWaitEvent(env->side, env->fork, 0);
+  if (err != cudaSuccess) return cuda_fail(err, "pre-generation stream");
+  cudaError_t built = jx::pregen_launch(p, steps, false, true, env->side);
+  err = cudaEventRecord(env->join, env->side);  // also behind a failed launch: s waits for what was launched
+  if (built != cudaSuccess) {
+    (void)cudaStreamWaitEvent(s, env->join, 0);
+    return cuda_fail(built, "pre-generation launch");
+  }
+  if (err != cudaSuccess) return cuda_fail(err, "pre-generation stream");
+  env->launches.fetch_add(jx::kPregenKernels, std::memory_order_relaxed);
   return JX_OK;
 }
 
@@ -216,11 +240,24 @@ jx_status run_rollout(jx_env* env, jx::Params p, cudaStream_t s) {
     q.frames = w.frames;
     q.rewards = w.rewards;
     q.dones = w.dones;
-    int launches = 0;
-    cudaError_t err = jx::rollout_launch(q, env->draw_slots, s, &launches);
-    env->launches.fetch_add(launches, std::memory_order_relaxed);
+    // next episodes are built beside the draw of the first segment: the walk
+    // does not read them, the draw leaves most of the chip's issue slots idle
+    const bool beside = t == 0 && pregen_beside_draw(env, p);
+    const jx::RolloutParts parts = jx::rollout_parts(q);
+    jx_status st = JX_OK;
+    cudaError_t err = cudaSuccess;
+    for (int i = 0; i <= parts.n && err == cudaSuccess && st == JX_OK; ++i) {
+      if (i == parts.n && beside) st = pregen_beside(env, p, steps, s);
+      if (st == JX_OK) err = jx::rollout_launch(q, parts, i, env->draw_slots, s);
+      if (st == JX_OK && err == cudaSuccess) env->launches.fetch_add(1, std::memory_order_relaxed);
+      if (i == parts.n && beside && st == JX_OK) {
+        const cudaError_t joined = cudaStreamWaitEvent(s, env->join, 0);
+        if (err == cudaSuccess) err = joined;
+      }
+    }
+    if (st != JX_OK) return st;
     if (err != cudaSuccess) return cuda_fail(err, "rollout launch");
-    if (jx_status st = launch_env(env, w, jx::MODE_ROLLOUT, s)) return st;
+    if ((st = launch_env(env, w, jx::MODE_ROLLOUT, s, beside)) != JX_OK) return st;
   }
   return JX_OK;
 }
@@ -229,8 +266,9 @@ jx_status run(jx_env* env, const jx::Params& p, int mode, void* stream) {
   DeviceGuard g(env->device);
   if (g.err != cudaSuccess) return cuda_fail(g.err, "cudaSetDevice");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (jx::pregen_runs(p) && (mode == jx::MODE_STEP || mode == jx::MODE_ROLLOUT || mode == jx::MODE_RESET)) {
-    cudaError_t err = jx::pregen_launch(p, mode == jx::MODE_ROLLOUT ? p.steps : 1, mode == jx::MODE_RESET, s);
+  if (jx::pregen_runs(p) && !(mode == jx::MODE_ROLLOUT && pregen_beside_draw(env, p)) &&
+      (mode == jx::MODE_STEP || mode == jx::MODE_ROLLOUT || mode == jx::MODE_RESET)) {
+    cudaError_t err = jx::pregen_launch(p, mode == jx::MODE_ROLLOUT ? p.steps : 1, mode == jx::MODE_RESET, false, s);
     if (err != cudaSuccess) return cuda_fail(err, "pre-generation launch");
     env->launches.fetch_add(jx::kPregenKernels, std::memory_order_relaxed);
   }
@@ -304,7 +342,7 @@ bool takes_team(const jx_env* env, int mode) {
 
 cudaError_t launch_frame(const jx_env* env, const Params& p, int mode, cudaStream_t stream, int* launches) {
   *launches += 1;
-  if (!takes_team(env, mode)) return launch(p, mode, env->grid, stream);
+  if (!takes_team(env, mode)) return launch(p, mode, env->grid, false, stream);
   Params q = env->team;
   q.actions = p.actions;
   q.frames = p.frames;
@@ -314,7 +352,7 @@ cudaError_t launch_frame(const jx_env* env, const Params& p, int mode, cudaStrea
   cudaError_t err = team_launch(q, mode, stream);
   if (err != cudaSuccess || mode != MODE_STEP || !steps_end(env)) return err;
   *launches += 1;
-  return launch(p, MODE_BEGIN, env->grid, stream);
+  return launch(p, MODE_BEGIN, env->grid, false, stream);
 }
 
 }  // namespace host
@@ -629,6 +667,17 @@ jx_status create_impl(const jx_config* cfg, int device, void* ext, size_t ext_by
       // the launch pays once a launch would start mazes on about three times
       // as many envs as there are resident warps
       p.nx_min = 3 * env->num_sms * jx::kMinBlocksPerSm;
+      // without the stream, builds run before a rollout's walk; its blocks go
+      // ahead of the draw's, which are many and wait for nobody
+      int low = 0, high = 0;
+      if (jx::pregen_runs(p) &&
+          (cudaDeviceGetStreamPriorityRange(&low, &high) != cudaSuccess ||
+           cudaEventCreateWithFlags(&env->fork, cudaEventDisableTiming) != cudaSuccess ||
+           cudaEventCreateWithFlags(&env->join, cudaEventDisableTiming) != cudaSuccess ||
+           cudaStreamCreateWithPriority(&env->side, cudaStreamNonBlocking, high) != cudaSuccess)) {
+        env->side = nullptr;
+        (void)cudaGetLastError();
+      }
     } else {
       if (env->nx_mem) cudaFree(env->nx_mem);
       env->nx_mem = nullptr;
@@ -755,6 +804,9 @@ jx_status jx_destroy(jx_env* env) {
     if (env->owns_mem && env->mem) cudaFree(env->mem);
     if (env->nx_mem) cudaFree(env->nx_mem);
     if (env->stage) cudaFree(env->stage);
+    if (env->side) cudaStreamDestroy(env->side);
+    if (env->fork) cudaEventDestroy(env->fork);
+    if (env->join) cudaEventDestroy(env->join);
   }
   delete env;
   return JX_OK;

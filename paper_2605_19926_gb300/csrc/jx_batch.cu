@@ -194,7 +194,7 @@ jx_status batch_run(jx_batch* b, int mode, cudaStream_t stream, const uint8_t* a
   if (mode == jx::MODE_STEP || mode == jx::MODE_ROLLOUT || mode == jx::MODE_RESET) {
     for (int i = 0; i < bp.n_groups; ++i) {  // groups whose next episodes are built ahead
       if (!jx::pregen_runs(bp.g[i])) continue;
-      cudaError_t err = jx::pregen_launch(bp.g[i], mode == jx::MODE_ROLLOUT ? steps : 1, mode == jx::MODE_RESET, stream);
+      cudaError_t err = jx::pregen_launch(bp.g[i], mode == jx::MODE_ROLLOUT ? steps : 1, mode == jx::MODE_RESET, false, stream);
       if (err != cudaSuccess) return cuda_fail(err, "pre-generation launch");
       if (count) b->launches.fetch_add(jx::kPregenKernels, std::memory_order_relaxed);
     }

@@ -40,6 +40,9 @@ struct jx_env {
   // next-episode block and work slots of the lane-parallel pre-generation
   // (owned mazes of side >= 64), or null
   uint8_t* nx_mem = nullptr;
+  // the stream and the events with which a rollout's builds run beside its draw, or null
+  cudaStream_t side = nullptr;
+  cudaEvent_t fork = nullptr, join = nullptr;
   // staging buffers of jx_step_host
   uint8_t* stage = nullptr;
   size_t stage_frames_off = 0, stage_rewards_off = 0, stage_dones_off = 0;

@@ -186,7 +186,9 @@ size_t pregen_work_bytes(int S);
 size_t pregen_words_bytes(int S);  // per env: the saved walk words of a build in progress
 // Lanes of the pre-generation kernel resident at once on num_sms SMs (its grid).
 cudaError_t pregen_resident_lanes(int S, int num_sms, int* lanes);
-cudaError_t pregen_launch(const Params& p, int steps, bool reset, cudaStream_t stream);
+// The pre-generation kernels before a launch of `steps` steps, or (walked)
+// between its walk and the env kernel.
+cudaError_t pregen_launch(const Params& p, int steps, bool reset, bool walked, cudaStream_t stream);
 // Whether a launch over p builds next episodes ahead at all: batches of fewer
 // than nx_min envs never do, so their launches need none of the build's
 // kernels (a 1024-env step of side-64 mazes, 96 x 96 frames and a grayscale
@@ -204,8 +206,8 @@ cudaError_t team_launch(const Params& q, int mode, cudaStream_t stream);  // q.s
 
 // Configure (attributes) and query occupancy of the kernel for `mode`.
 cudaError_t kernel_blocks_per_sm(const Params& p, int mode, int* blocks);
-// Launch the fused kernel for `mode`.
-cudaError_t launch(const Params& p, int mode, int grid, cudaStream_t stream);
+// Launch the fused kernel for `mode`; joined: behind a wait for another stream.
+cudaError_t launch(const Params& p, int mode, int grid, bool joined, cudaStream_t stream);
 
 // Rollouts in two passes (jx_rollout.cu). Camera records are kept for at most
 // rollout_segment(n) steps: longer rollouts run in segments of that many.
@@ -221,9 +223,15 @@ void rollout_place(Params& p, uint8_t* mem);  // the pointers into rollout_bytes
 // Base parameters to those of the two passes, rows chosen as for the env kernel.
 void rollout_layout(Params& q, size_t smem_per_sm, size_t reserved);
 cudaError_t rollout_prepare(const Params& q);  // kernel attributes
-// The walk and the draw of q.steps steps with room for `slots` warps at once;
-// adds the kernels launched to *launches.
-cudaError_t rollout_launch(const Params& q, int slots, cudaStream_t stream, int* launches);
+// The parts of a rollout: part i ends before step ends[i].
+constexpr int kMaxParts = 4;
+struct RolloutParts {
+  int n, ends[kMaxParts];
+};
+RolloutParts rollout_parts(const Params& q);
+// Launch i of parts.n + 1: the walk of part i and the draw of part i - 1, with
+// room for `slots` warps at once.
+cudaError_t rollout_launch(const Params& q, const RolloutParts& parts, int i, int slots, cudaStream_t stream);
 
 // One launch of the two passes: steps walk_t0 .. walk_t1 - 1 are walked by the
 // first walk_blocks blocks, steps t0 .. t1 - 1 drawn by the others, in

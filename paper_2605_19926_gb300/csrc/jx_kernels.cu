@@ -221,7 +221,10 @@ __global__ void __launch_bounds__(256) pregen_walls_kernel(const __grid_constant
 // entry is published by its episode number (nx_ep). Each lane keeps the walk's words in shared memory while it runs
 // (kPregenThreads lanes a block, pregen_lane_words words each: under 48 KB a
 // block for side 128) and in the words array between launches.
-__global__ void __launch_bounds__(kPregenThreads) pregen_kernel(const __grid_constant__ Params p, int steps, int reset) {
+// `walked`: the launch's walk has run, so an env's step count is ahead by the
+// steps walked (p.stop).
+__global__ void __launch_bounds__(kPregenThreads)
+    pregen_kernel(const __grid_constant__ Params p, int steps, int reset, int walked) {
   extern __shared__ uint32_t pregen_sm[];
   if (*p.nx_count == 0u) return;  // the whole grid
   const LaneSlot L = lane_slot(p.S);
@@ -242,7 +245,7 @@ __global__ void __launch_bounds__(kPregenThreads) pregen_kernel(const __grid_con
       w = resume ? lane_walk_load(W, work, L, p.nx_words, e, p.n) : lane_walk_begin(p, e, ep, W, work, L);
       int launches = 1;  // the launches left for the remaining steps
       if (!reset) {
-        const int left = p.horizon - p.st.t[e];
+        const int left = p.horizon - (p.st.t[e] - (walked ? p.stop[e] : 0));
         launches = left > steps ? (left + steps - 1) / steps - 1 : 1;
       }
       // a build's steps go into at most kPregenLaunches launches after the
@@ -294,9 +297,10 @@ cudaError_t blocks_per_sm_mode(const Params& p, int* blocks) {
 
 // Programmatic stream serialisation: the launch may overlap the tail of the
 // kernel before it on the stream up to its griddepcontrol.wait (consecutive
-// steps in a CUDA graph then start without a launch gap).
+// steps in a CUDA graph then start without a launch gap). Not so behind a
+// joined stream, whose kernels that wait does not cover.
 template <int MODE>
-cudaError_t launch_mode(const Params& p, int grid, cudaStream_t stream) {
+cudaError_t launch_mode(const Params& p, int grid, bool joined, cudaStream_t stream) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid);
   cfg.blockDim = dim3(kThreads);
@@ -306,7 +310,7 @@ cudaError_t launch_mode(const Params& p, int grid, cudaStream_t stream) {
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = joined ? 0 : 1;
   return cudaLaunchKernelEx(&cfg, env_kernel_of<MODE>(p), p);
 }
 }  // namespace
@@ -369,7 +373,7 @@ size_t pregen_work_bytes(int S) {
   return ((size_t)lane_slot(S).bytes + 255) & ~(size_t)255;
 }
 
-cudaError_t pregen_launch(const Params& p, int steps, bool reset, cudaStream_t stream) {
+cudaError_t pregen_launch(const Params& p, int steps, bool reset, bool walked, cudaStream_t stream) {
   if (!pregen_runs(p)) return cudaSuccess;
   cudaError_t err = cudaMemsetAsync(p.nx_count, 0, 2 * sizeof(uint32_t), stream);
   if (err != cudaSuccess) return err;
@@ -378,7 +382,7 @@ cudaError_t pregen_launch(const Params& p, int steps, bool reset, cudaStream_t s
   pregen_walls_kernel<<<(unsigned)(wall_blocks < 4096 ? wall_blocks : 4096), 256, 0, stream>>>(p, reset ? 1 : 0);
   const size_t lane_bytes = (size_t)kPregenThreads * pregen_lane_words(p.S) * sizeof(uint32_t);
   pregen_kernel<<<(p.nx_lanes + kPregenThreads - 1) / kPregenThreads, kPregenThreads, lane_bytes, stream>>>(
-      p, steps, reset ? 1 : 0);  // nx_lanes: the resident lanes (pregen_resident_lanes)
+      p, steps, reset ? 1 : 0, walked ? 1 : 0);  // nx_lanes: the resident lanes (pregen_resident_lanes)
   return cudaGetLastError();
 }
 
@@ -421,14 +425,14 @@ cudaError_t kernel_blocks_per_sm(const Params& p, int mode, int* blocks) {
   }
 }
 
-cudaError_t launch(const Params& p, int mode, int grid, cudaStream_t stream) {
+cudaError_t launch(const Params& p, int mode, int grid, bool joined, cudaStream_t stream) {
   switch (mode) {
-    case MODE_STEP: return launch_mode<MODE_STEP>(p, grid, stream);
-    case MODE_RESET: return launch_mode<MODE_RESET>(p, grid, stream);
-    case MODE_RENDER: return launch_mode<MODE_RENDER>(p, grid, stream);
-    case MODE_ROLLOUT: return launch_mode<MODE_ROLLOUT>(p, grid, stream);
-    case MODE_BEGIN: return launch_mode<MODE_BEGIN>(p, grid, stream);
-    default: return launch_mode<MODE_RAYS>(p, grid, stream);
+    case MODE_STEP: return launch_mode<MODE_STEP>(p, grid, joined, stream);
+    case MODE_RESET: return launch_mode<MODE_RESET>(p, grid, joined, stream);
+    case MODE_RENDER: return launch_mode<MODE_RENDER>(p, grid, joined, stream);
+    case MODE_ROLLOUT: return launch_mode<MODE_ROLLOUT>(p, grid, joined, stream);
+    case MODE_BEGIN: return launch_mode<MODE_BEGIN>(p, grid, joined, stream);
+    default: return launch_mode<MODE_RAYS>(p, grid, joined, stream);
   }
 }
 }  // namespace jx

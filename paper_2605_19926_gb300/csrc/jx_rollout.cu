@@ -432,7 +432,6 @@ void choose_chunks(DrawPart& d, int n, int slots) {
 // 128 x 128, 8 steps, building next episodes: 1.41 ms whole, 1.49
 // in parts of 2 and 6.) Writes the parts' ends to `ends` and returns
 // their number.
-constexpr int kMaxParts = 4;
 int choose_parts(int steps, int64_t frame_bytes, int frame_px, int* ends) {
   const double walk_us = 1.2, ratio = (double)frame_bytes / 7.0e6 / walk_us;  // draw over walk of a step
   const double end_us = 3.0 * frame_px / 4096;
@@ -494,25 +493,22 @@ cudaError_t rollout_prepare(const Params& q) {
   return raise_smem_limit(q.gray ? rollout_kernel<1> : rollout_kernel<0>);
 }
 
-cudaError_t rollout_launch(const Params& q, int slots, cudaStream_t stream, int* launches) {
-  int ends[kMaxParts];
-  const int parts = choose_parts(q.steps, (int64_t)q.n * 3 * q.H * q.W, q.H * q.W, ends);
-  const int walk_blocks = (q.n + kEnvsPerWalkBlock - 1) / kEnvsPerWalkBlock;
-  const int pairs = (q.n + kWarpsPerBlock - 1) / kWarpsPerBlock;
-  for (int i = 0; i <= parts; ++i) {  // launch i walks part i and draws part i - 1
-    DrawPart d = {};
-    d.walk_blocks = i < parts ? walk_blocks : 0;
-    d.walk_t0 = i > 0 ? ends[i - 1] : 0;
-    d.walk_t1 = i < parts ? ends[i] : 0;
-    d.t0 = i > 1 ? ends[i - 2] : 0;
-    d.t1 = i > 0 ? ends[i - 1] : 0;
-    choose_chunks(d, q.n, slots);
-    const int64_t grid = d.walk_blocks + (int64_t)pairs * chunk_count(d);
-    cudaError_t err = launch_dependent(q.gray ? rollout_kernel<1> : rollout_kernel<0>, (int)grid, block_smem_bytes(q), stream, q, d);
-    if (err != cudaSuccess) return err;
-    ++*launches;
-  }
-  return cudaSuccess;
+RolloutParts rollout_parts(const Params& q) {
+  RolloutParts parts;
+  parts.n = choose_parts(q.steps, (int64_t)q.n * 3 * q.H * q.W, q.H * q.W, parts.ends);
+  return parts;
+}
+
+cudaError_t rollout_launch(const Params& q, const RolloutParts& parts, int i, int slots, cudaStream_t stream) {
+  DrawPart d = {};
+  d.walk_blocks = i < parts.n ? (q.n + kEnvsPerWalkBlock - 1) / kEnvsPerWalkBlock : 0;
+  d.walk_t0 = i > 0 ? parts.ends[i - 1] : 0;
+  d.walk_t1 = i < parts.n ? parts.ends[i] : 0;
+  d.t0 = i > 1 ? parts.ends[i - 2] : 0;
+  d.t1 = i > 0 ? parts.ends[i - 1] : 0;
+  choose_chunks(d, q.n, slots);
+  const int64_t grid = d.walk_blocks + (int64_t)((q.n + kWarpsPerBlock - 1) / kWarpsPerBlock) * chunk_count(d);
+  return launch_dependent(q.gray ? rollout_kernel<1> : rollout_kernel<0>, (int)grid, block_smem_bytes(q), stream, q, d);
 }
 
 cudaError_t batch_rollout_prepare(const BatchParams& bq) {

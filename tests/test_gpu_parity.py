@@ -766,6 +766,44 @@ def test_two_pass_rollout_equals_single_steps(case):
     b.env.sync_status()
 
 
+@pytest.mark.parametrize("T,captured", [(6, False), (6, True), (130, False)])
+def test_builds_beside_the_draw_equal_single_steps(T, captured):
+    """Large batches of large mazes build next episodes beside a rollout's draw:
+    rollouts in a row, over several horizons and (130 steps) two segments, give
+    the frames, outputs and state of single steps, also from a captured graph."""
+    cfg = dict(inputs.maze_keydoor(n_envs=12801, map_side=64, seed=71, horizon=17, frame_h=8, frame_w=16))
+    N = cfg["n_envs"]
+    a, b = Run(cfg), Run(cfg)
+    a.reset()
+    b.reset()
+    frames = torch.zeros((T, N, 8, 16, 3), dtype=torch.uint8, device=a.dev)
+    rewards = torch.zeros((T, N), dtype=torch.float32, device=a.dev)
+    dones = torch.zeros((T, N), dtype=torch.uint8, device=a.dev)
+    acts = torch.zeros((T, N), dtype=torch.uint8, device=a.dev)
+    graph = None
+    if captured:
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            b.env.rollout(acts, frames, rewards, dones)
+    for rep in range(2 if T > 100 else 5):
+        acts.copy_(torch.from_numpy(np.stack([forward_biased_actions(72 + rep, s, N) for s in range(T)])))
+        if graph is not None:
+            graph.replay()
+        else:
+            b.env.rollout(acts, frames, rewards, dones)
+        for t in range(T):
+            a.actions.copy_(acts[t])
+            a.env.step(a.actions, a.frames, a.rewards, a.dones)
+            assert torch.equal(a.frames, frames[t]), (rep, t)
+            assert torch.equal(a.rewards, rewards[t]) and torch.equal(a.dones, dones[t]), (rep, t)
+        torch.cuda.synchronize()
+        assert (a.env.get_state() == b.env.get_state()).all(), rep
+    assert (a.env.fields(a.env.get_state())["episode"] >= 1).all()
+    a.env.sync_status()
+    b.env.sync_status()
+
+
 def test_late_handoff_is_reported_and_later_rollouts_exact():
     """With the hand-off wait limit at 0 polls every hand-off of a chunked
     rollout counts as late: the launch still ends, the device error word says
