@@ -565,13 +565,16 @@ __device__ __forceinline__ void gen_rooms(const Params& p, int e, uint32_t ep, u
 
 // Work space of one maze generation of nn x nn nodes. The fast part is in the
 // walk's chain of dependent accesses:
-//   avail  [(nn + 2)^2] bytes, nodes with a border around them: the directions
-//          (bit 0 N, 1 E, 2 S, 3 W) in which an unvisited node lies
-//   stack  [n] the path to the current node, cells packed as y << 8 | x;
-//          afterwards each node's place in the visiting order
+//   avail  [(nn + 2) (nn + 1)] bytes, the rows of nodes with a border row above
+//          and below and a border column after each (which is the next row's
+//          left border too): the directions (bit 1 N, 2 E, 3 S, 4 W) in which
+//          an unvisited node lies
+//   stack  [n] the path to the current node, places in avail; afterwards each
+//          node's place in the visiting order
 // the slow part is written, or read ahead:
-//   seq    [n] visiting order: node | depth << 16
-//   pick   [n] per carve: the draw's choice among 2, 3 and 4 candidates
+//   seq    [n] visiting order: place in avail | depth << 16 | direction taken
+//          << 30, after the walk node | depth << 16
+//   pick   [n + 1] per carve (the last is read ahead only): the draw's choice among 2, 3 and 4 candidates
 struct MazeWork {
   uint8_t* avail;
   uint16_t* stack;
@@ -580,28 +583,28 @@ struct MazeWork {
 };
 __host__ __device__ __forceinline__ int maze_nodes(int S) { return (S - 2) / 2; }  // per side
 __host__ __device__ __forceinline__ size_t maze_fast_bytes(int nn) {
-  return (size_t)align16((nn + 2) * (nn + 2)) + align16(2 * nn * nn);
+  return (size_t)align16((nn + 2) * (nn + 1)) + align16(2 * nn * nn);
 }
 __host__ __device__ __forceinline__ size_t maze_slow_bytes(int nn) {
-  return (size_t)align16(4 * nn * nn) + align16(nn * nn);
+  return (size_t)align16(4 * nn * nn) + align16(nn * nn + 1);
 }
 __device__ __forceinline__ MazeWork maze_work(uint8_t* fast, uint8_t* slow, int nn) {
   MazeWork m;
   m.avail = fast;
-  m.stack = (uint16_t*)(fast + align16((nn + 2) * (nn + 2)));
+  m.stack = (uint16_t*)(fast + align16((nn + 2) * (nn + 1)));
   m.seq = (uint32_t*)slow;
   m.pick = slow + align16(4 * nn * nn);
   return m;
 }
 
-// The direction a carve takes: candidate r of the set `open` (bits in N, E, S,
-// W order), r the draw's choice for that many candidates (bit 0: of two, bits
-// 1-2: of three, bits 3-4: of four).
+// The directions a carve can take: for the draw's choice `pick` (bit 0: of two
+// candidates, bits 1-2: of three, bits 3-4: of four) one word with two bits
+// for each set `open` of candidates (bits in N, E, S, W order), at bit 2 open.
 struct MazePick {
-  uint8_t d[512];
+  uint32_t d[32];
   constexpr MazePick() : d() {
-    for (int open = 0; open < 16; ++open)
-      for (int pick = 0; pick < 32; ++pick) {
+    for (int pick = 0; pick < 32; ++pick)
+      for (int open = 0; open < 16; ++open) {
         int n = 0;
         for (int b = 0; b < 4; ++b) n += (open >> b) & 1;
         int r = n == 2 ? (pick & 1) : (n == 3 ? ((pick >> 1) & 3) : (n == 4 ? pick >> 3 : 0));
@@ -611,7 +614,7 @@ struct MazePick {
             dir = b;
             if (r-- == 0) break;
           }
-        d[open * 32 + pick] = (uint8_t)dir;
+        d[pick] |= (uint32_t)dir << (2 * open);
       }
   }
 };
@@ -625,20 +628,22 @@ __constant__ MazePick c_maze_pick = MazePick();
 // (deepest, ties to the smallest row-major index), the door's two path nodes
 // and the nodes reachable without crossing the door all come from the visiting
 // order, by the warp together.
-// The walk is a chain of dependent accesses, so it is kept short: all lanes
-// step it together (no divergence), one load says which neighbours are open
-// (the visits keep it up to date, four lanes at a time), one constant says
-// which of them the draw picks, and a dead end is left by looking at 32 nodes
-// of the path at once. (72 instructions a move on one lane, over two moves a
-// node, before; about 60 a node now. Resets of 4096 envs: 32 x 32 mazes 197 ->
-// 97 us, 64 x 64 968 -> 326; of 256 envs 90 -> 46 and 372 -> 138. With the
-// choice in a register table read by shuffles instead of the constant: 117.)
+// With many mazes at once the walk is bound by the instructions it issues,
+// alone by its chain of dependent accesses, so both are kept short: all lanes
+// step it together (no divergence, also where one value is stored), the four
+// directions' neighbours are read where they are marked, so that the next
+// node's open sides are a shuffle away, the draw's choice is a word read one
+// carve ahead, a dead end is left by looking at 32 nodes of the path at once,
+// and the floor is laid afterwards from the visiting order. (4096 envs, 32 x
+// 32: a reset takes 78 us, and 91 with the open sides loaded and the choice
+// and the map's bytes looked up and stored in each carve; 198 with one lane
+// walking and two moves a node.)
 // FAST_SMEM: the fast part lies in shared memory (an instance of its own, so
 // that the compiler knows the address space).
 template <bool FAST_SMEM>
 __device__ __forceinline__ void gen_maze(const Params& p, int e, uint32_t ep, uint8_t* smap, const MazeWork& m, int lane) {
   const int S = p.S, n_cells = S * S;
-  const int nn = maze_nodes(S), n = nn * nn, q = nn + 2;
+  const int nn = maze_nodes(S), n = nn * nn, q = nn + 1;
   const uint64_t kw = stream_key(p.seed, (uint32_t)e, ep, P_WALL);
   for (int i = 4 * lane; i < n_cells; i += 128) {  // S is even: whole words
     uint32_t w = 0x01010101u;
@@ -647,33 +652,31 @@ __device__ __forceinline__ void gen_maze(const Params& p, int e, uint32_t ep, ui
     *reinterpret_cast<uint32_t*>(smap + i) = w;
   }
   const uint64_t kd = stream_key(p.seed, (uint32_t)e, ep, P_DFS);
-  for (int j = lane; j < n; j += 32) {
+  for (int j = lane; j <= n; j += 32) {
     const uint32_t hi = (uint32_t)(draw_at(kd, (uint32_t)j) >> 32);
     m.pick[j] = (uint8_t)(hi >> 31 | below32(hi, 3u) << 1 | (hi >> 30) << 3);
   }
-  for (int i = lane; i < q * q; i += 32) {
+  for (int i = lane; i < (nn + 2) * q; i += 32) {
     const int y = i / q, x = i - y * q;
-    const bool node = x >= 1 && x <= nn && y >= 1 && y <= nn;
-    m.avail[i] = node ? (uint8_t)((y > 1 ? 1 : 0) | (x < nn ? 2 : 0) | (y < nn ? 4 : 0) | (x > 1 ? 8 : 0)) : (uint8_t)0;
+    const bool node = x < nn && y >= 1 && y <= nn;
+    m.avail[i] = node ? (uint8_t)((y > 1 ? 2 : 0) | (x < nn - 1 ? 4 : 0) | (y < nn ? 8 : 0) | (x > 0 ? 16 : 0)) : (uint8_t)0;
   }
   const int start = (int)below(draw_at(stream_key(p.seed, (uint32_t)e, ep, P_SPAWN), 0), (uint32_t)n);
   __syncwarp();
-  // lanes 0..3: the neighbour in direction `lane`, and all its directions but the one back
-  const int my_step = lane == 0 ? -q : (lane == 1 ? 1 : (lane == 2 ? q : -1));
-  const uint32_t my_keep = ~(1u << (lane ^ 2));
+  // lane & 3 is a direction: the neighbour in it, and all its directions but
+  // the one back. Lanes of one direction, and all lanes for the current node,
+  // store the same values: the walk has no divergent branch.
+  const int my_d = lane & 3, my_step = my_d == 0 ? -q : (my_d == 1 ? 1 : (my_d == 2 ? q : -1));
+  const uint32_t my_keep = ~(2u << (my_d ^ 2));
   {
-    int yx = (2 * (start / nn) + 1) << 8 | (2 * (start % nn) + 1);
-    int node = start, a = (start / nn + 1) * q + start % nn + 1, c = (yx >> 8) * S + (yx & 255);
-    int depth = 0;
-    if (lane < 4) m.avail[a + my_step] &= (uint8_t)my_keep;
-    if (lane == 0) {
-      smap[c] = 0;
-      m.stack[0] = (uint16_t)yx;
-      m.seq[0] = (uint32_t)node;
-    }
-    __syncwarp();
-    uint32_t pick = m.pick[0];
+    int a = (start / nn + 1) * q + start % nn, depth = 0;
     uint32_t open = m.avail[a];
+    uint32_t near = m.avail[a + my_step] & my_keep;  // the open directions of the neighbour
+    m.avail[a + my_step] = (uint8_t)near;
+    m.stack[0] = (uint16_t)a;
+    m.seq[0] = (uint32_t)a;
+    __syncwarp();
+    uint32_t dirs = c_maze_pick.d[m.pick[0]], pick = m.pick[1];  // of this carve, of the next
     for (int k = 1; k < n; ++k) {  // the k-th carve
       if (open == 0) {
         // a dead end: back to the deepest node of the path with an open side
@@ -681,45 +684,48 @@ __device__ __forceinline__ void gen_maze(const Params& p, int e, uint32_t ep, ui
         int from = depth;
         for (; from > 0; from -= 32) {
           const int i = from - 1 - lane;
-          uint32_t yx_i = 0u, open_i = 0u;
+          int a_i = 0;
+          uint32_t open_i = 0u;
           if (i >= 0) {
-            yx_i = m.stack[i];
-            open_i = m.avail[(((yx_i >> 8) + 1) >> 1) * q + (((yx_i & 255u) + 1) >> 1)];
+            a_i = m.stack[i];
+            open_i = m.avail[a_i];
           }
           const uint32_t b = __ballot_sync(0xffffffffu, open_i != 0u);
           if (b) {
             const int src = __ffs(b) - 1;
             depth = from - 1 - src;
-            yx = (int)__shfl_sync(0xffffffffu, yx_i, src);
+            a = __shfl_sync(0xffffffffu, a_i, src);
             open = __shfl_sync(0xffffffffu, open_i, src);
             break;
           }
         }
         if (from <= 0) break;
-        const int y = yx >> 8, x = yx & 255;
-        c = y * S + x;
-        a = ((y + 1) >> 1) * q + ((x + 1) >> 1);
-        node = (y >> 1) * nn + (x >> 1);
+        near = m.avail[a + my_step];
       }
-      const int d = c_maze_pick.d[open * 32 + pick];
-      pick = m.pick[k];  // for the next carve
-      const int sgn = ((d + 1) & 2) ? 1 : -1;
-      const bool row = d & 1;
-      const int dc = sgn * (row ? 1 : S);
-      if (lane < 2) smap[c + (lane + 1) * dc] = 0;  // the passage and the node
-      c += 2 * dc;
-      a += sgn * (row ? 1 : q);
-      node += sgn * (row ? 1 : nn);
-      yx += sgn * (row ? 2 : 512);
+      const int d = (int)(dirs >> open) & 3;
+      dirs = c_maze_pick.d[pick];
+      pick = m.pick[k + 1];
+      open = __shfl_sync(0xffffffffu, near, d);
+      a += __shfl_sync(0xffffffffu, my_step, d);
       ++depth;
-      open = m.avail[a];
-      if (lane < 4) m.avail[a + my_step] &= (uint8_t)my_keep;
-      if (lane == 0) {
-        m.stack[depth] = (uint16_t)yx;
-        m.seq[k] = (uint32_t)node | (uint32_t)depth << 16;
-      }
+      near = m.avail[a + my_step] & my_keep;
+      m.avail[a + my_step] = (uint8_t)near;
+      m.stack[depth] = (uint16_t)a;
+      m.seq[k] = (uint32_t)d << 30 | (uint32_t)depth << 16 | (uint32_t)a;
       __syncwarp();
     }
+  }
+  __syncwarp();
+  // the nodes and the passages to them become floor, all lanes on their own
+  // (a / q = a r >> 20: a < 2^13, q <= 64)
+  const uint32_t r_q = ((1u << 20) + (uint32_t)q - 1u) / (uint32_t)q;
+  for (int k = lane; k < n; k += 32) {
+    const uint32_t v = m.seq[k], a = v & 0xffffu;
+    const int y1 = (int)(a * r_q >> 20), x = (int)a - y1 * q, y = y1 - 1, d = (int)(v >> 30);
+    const int c = (2 * y + 1) * S + 2 * x + 1, dc = d & 1 ? 1 : S;
+    smap[c] = 0;
+    if (k > 0) smap[(d + 1) & 2 ? c - dc : c + dc] = 0;
+    m.seq[k] = (uint32_t)(y * nn + x) | (v & 0x0fff0000u);
   }
   __syncwarp();
   // the goal: the deepest node, ties to the smallest index (n < 4096)
