@@ -456,31 +456,72 @@ __device__ __forceinline__ bool stage(const Params& p, int e, uint8_t* smap, int
 }
 
 // ------------------------------------------------------------ generators --
-// Index of the r-th cell (row-major) of smap[0..n) satisfying pred, or -1.
+// The r-th set bit of b (r below its count), the lanes together.
+__device__ __forceinline__ int nth_bit(uint32_t b, uint32_t r, int lane) {
+  const bool me = ((b >> lane) & 1u) && (uint32_t)__popc(b & ((1u << lane) - 1u)) == r;
+  return __ffs(__ballot_sync(0xffffffffu, me)) - 1;
+}
+
+// Index of the r-th cell (row-major) of smap[from..n) satisfying pred, or -1.
 template <class Pred>
-__device__ __forceinline__ int nth_cell(int n, uint32_t r, int lane, Pred pred) {
-  for (int base = 0; base < n; base += 32) {
-    int i = base + lane;
-    bool f = i < n && pred(i);
-    uint32_t b = __ballot_sync(0xffffffffu, f);
-    uint32_t c = __popc(b);
-    if (r < c) {
-      for (uint32_t k = 0; k < r; ++k) b &= b - 1;
-      return base + __ffs(b) - 1;
-    }
+__device__ __forceinline__ int nth_cell(int from, int n, uint32_t r, int lane, Pred pred) {
+  for (int base = from; base < n; base += 32) {
+    const int i = base + lane;
+    const uint32_t b = __ballot_sync(0xffffffffu, i < n && pred(i));
+    const uint32_t c = __popc(b);
+    if (r < c) return base + nth_bit(b, r, lane);
     r -= c;
   }
   return -1;
 }
 
-template <class Pred>
-__device__ __forceinline__ int count_cells(int n, int lane, Pred pred) {
-  int total = 0;
-  for (int base = 0; base < n; base += 32) {
-    int i = base + lane;
-    total += __popc(__ballot_sync(0xffffffffu, i < n && pred(i)));
+// Counts of the cells of smap[0..n) that satisfy a predicate, by strips of
+// `words` x 32 cells, one a lane: the cells before the lane's strip, and all.
+// Looking up a cell by its number then reads one strip, not the map up to it.
+// (Rooms with up to 8 sprites, 64 x 64: a reset of 4096 envs takes 151 us
+// with a pass over the map for every sprite, 75 with the strips.)
+struct CellIndex {
+  uint32_t before, total;
+  int words;
+  // over the 32-cell words in order, the cells of each that count
+  int own = 0, left;
+  uint32_t mine = 0;
+  __device__ __forceinline__ explicit CellIndex(int n) : words((n + 1023) >> 10), left(words) {}
+  __device__ __forceinline__ void add(uint32_t bits, int lane) {
+    if (own == lane) mine += __popc(bits);
+    if (--left == 0) {
+      ++own;
+      left = words;
+    }
   }
-  return total;
+  __device__ __forceinline__ void finish(int lane) {
+    uint32_t v = mine;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const uint32_t o = __shfl_up_sync(0xffffffffu, v, d);
+      if (lane >= d) v += o;
+    }
+    total = __shfl_sync(0xffffffffu, v, 31);
+    before = v - mine;
+  }
+  // the r-th cell (r below total)
+  template <class Pred>
+  __device__ __forceinline__ int nth(int n, uint32_t r, int lane, Pred pred) const {
+    const int strip = 31 - __clz(__ballot_sync(0xffffffffu, before <= r));
+    return nth_cell(strip * words * 32, n, r - __shfl_sync(0xffffffffu, before, strip), lane, pred);
+  }
+};
+
+template <class Pred>
+__device__ __forceinline__ CellIndex index_cells(int n, int lane, Pred pred) {
+  CellIndex ix(n);
+#pragma unroll 4
+  for (int base = 0; base < n; base += 32) {
+    const int i = base + lane;
+    ix.add(__ballot_sync(0xffffffffu, i < n && pred(i)), lane);
+  }
+  ix.finish(lane);
+  return ix;
 }
 
 // Writes the scalar fields of a fresh episode (lane 0) and all K sprite slots
@@ -528,31 +569,42 @@ __device__ void write_episode_state(const Params& p, const State& st, int e, uin
 __device__ __forceinline__ void gen_rooms(const Params& p, int e, uint32_t ep, uint8_t* smap, int lane) {
   const int S = p.S, n = S * S;
   const uint64_t kw = stream_key(p.seed, (uint32_t)e, ep, P_WALL);
-  for (int i = lane; i < n; i += 32) {
-    uint64_t u = draw_at(kw, (uint32_t)i);
-    int x = i % S, y = i / S;
-    bool border = x == 0 || y == 0 || x == S - 1 || y == S - 1;
-    bool wall = border || (u >> 11) < p.wall_thr;
-    smap[i] = wall ? (uint8_t)(1 + (u & 3)) : (uint8_t)0;
+  CellIndex free_cells(n);
+  const int dy = 32 / S, dx = 32 - dy * S;
+  int y = lane / S, x = lane - y * S;
+  for (int base = 0; base < n; base += 32) {
+    const int i = base + lane;
+    const uint64_t u = draw_at(kw, (uint32_t)i);
+    const bool border = x == 0 || y == 0 || x == S - 1 || y == S - 1;
+    const bool wall = border || (u >> 11) < p.wall_thr;
+    if (i < n) smap[i] = wall ? (uint8_t)(1 + (u & 3)) : (uint8_t)0;
+    free_cells.add(__ballot_sync(0xffffffffu, i < n && !wall), lane);
+    x += dx;
+    y += dy;
+    if (x >= S) {
+      x -= S;
+      ++y;
+    }
   }
+  free_cells.finish(lane);
   __syncwarp();
   auto is_free = [&](int i) { return smap[i] == 0; };
-  int n_free = count_cells(n, lane, is_free);
-  if (n_free == 0) {
+  if (free_cells.total == 0) {
     if (lane == 0) smap[(S / 2) * S + S / 2] = 0;
     __syncwarp();
-    n_free = 1;
+    free_cells = index_cells(n, lane, is_free);
   }
-  uint32_t pick = below(draw_at(stream_key(p.seed, (uint32_t)e, ep, P_SPAWN), 0), (uint32_t)n_free);
-  int spawn = nth_cell(n, pick, lane, is_free);
+  const uint32_t n_free = free_cells.total;
+  const uint32_t pick = below(draw_at(stream_key(p.seed, (uint32_t)e, ep, P_SPAWN), 0), n_free);
+  const int spawn = free_cells.nth(n, pick, lane, is_free);
   int nspr = 0;
   int spr_cell[kMaxSprites], spr_type[kMaxSprites];
   if (p.K > 0) {
     nspr = (int)below(draw_at(stream_key(p.seed, (uint32_t)e, ep, P_NSPRITES), 0), (uint32_t)p.K + 1);
     const uint64_t kc = stream_key(p.seed, (uint32_t)e, ep, P_SPRITE_CELL);
     for (int k = 0; k < nspr; ++k) {
-      uint32_t c = below(draw_at(kc, (uint32_t)k), (uint32_t)n_free);
-      spr_cell[k] = nth_cell(n, c, lane, is_free);
+      const uint32_t c = below(draw_at(kc, (uint32_t)k), n_free);
+      spr_cell[k] = free_cells.nth(n, c, lane, is_free);
       spr_type[k] = 3;
     }
   }
@@ -767,7 +819,7 @@ __device__ __forceinline__ void gen_maze(const Params& p, int e, uint32_t ep, ui
   int key = start;
   if (n_side > 0) {
     uint32_t r = below(draw_at(stream_key(p.seed, (uint32_t)e, ep, P_KEY), 0), (uint32_t)n_side);
-    key = nth_cell(n, r, lane, side);
+    key = nth_cell(0, n, r, lane, side);
   }
   auto cell_of = [&](int v) { return (2 * (v / nn) + 1) * S + 2 * (v % nn) + 1; };
   const int kc = cell_of(key), gc = cell_of(goal);
@@ -793,12 +845,12 @@ __device__ __forceinline__ void gen_maze(const Params& p, int e, uint32_t ep, ui
     }
     __syncwarp();
     auto is_free = [&](int i) { return smap[i] == 0; };
-    const int n_free = count_cells(n_cells, lane, is_free);
+    const CellIndex free_cells = index_cells(n_cells, lane, is_free);
     const int nd = (int)below(draw_at(stream_key(p.seed, (uint32_t)e, ep, P_NSPRITES), 0), (uint32_t)(p.K - 1));
     const uint64_t ks = stream_key(p.seed, (uint32_t)e, ep, P_SPRITE_CELL);
     for (int k = 0; k < nd; ++k) {
-      const uint32_t c = below(draw_at(ks, (uint32_t)k), (uint32_t)n_free);
-      spr_cell[2 + k] = nth_cell(n_cells, c, lane, is_free);
+      const uint32_t c = below(draw_at(ks, (uint32_t)k), free_cells.total);
+      spr_cell[2 + k] = free_cells.nth(n_cells, c, lane, is_free);
       spr_type[2 + k] = 3;
     }
     nspr = 2 + nd;
@@ -1212,8 +1264,8 @@ __device__ __forceinline__ void gen_ascii(const Params& p, int e, uint32_t ep, u
   if (p.n_spawn > 0) {
     cell = p.cand[below(d, (uint32_t)p.n_spawn)];
   } else {
-    const int n_free = count_cells(n, lane, is_free);
-    cell = nth_cell(n, below(d, (uint32_t)n_free), lane, is_free);
+    const CellIndex free_cells = index_cells(n, lane, is_free);
+    cell = free_cells.nth(n, below(d, free_cells.total), lane, is_free);
   }
   int spr_cell[kMaxSprites], spr_type[kMaxSprites];
   int obj[6] = {-1, -1, -1, -1, -1, -1};

@@ -647,6 +647,19 @@ def test_pregenerated_episodes_equal_episodes_built_in_place():
     small.env.sync_status()
 
 
+@pytest.mark.parametrize("side,wall_prob", [(3, 0.0), (3, 1.0), (5, 0.5), (31, 0.3), (32, 0.97), (33, 0.25), (45, 1.0),
+                                            (64, 0.995), (100, 0.6), (128, 0.3)])
+def test_cells_found_by_strips_match_oracle(side, wall_prob):
+    """Spawns and sprites of rooms lie on the oracle's cells: maps of less than,
+    exactly and just over a word of 32 cells a lane, with strips that hold no
+    free cell, a single free cell, and none at all."""
+    run = Run(inputs.rooms(n_envs=40, map_side=side, wall_prob=wall_prob, seed=81 + side, max_sprites=9, frame_h=8,
+                           frame_w=16))
+    stats = Stats()
+    check_reset(run, stats)
+    stats.check()
+
+
 def _corridor(text, n=8):
     cfg = dict(inputs.ascii_env("simple", n_envs=n, map_side=16, horizon=0), ascii_map=text)
     run = Run(cfg)
