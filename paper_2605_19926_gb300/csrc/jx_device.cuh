@@ -687,8 +687,9 @@ __constant__ MazePick c_maze_pick = MazePick();
 // node's open sides are a shuffle away, the draw's choice is a word read one
 // carve ahead, a dead end is left by looking at 32 nodes of the path at once,
 // and the floor is laid afterwards from the visiting order. (4096 envs, 32 x
-// 32: a reset takes 78 us, and 91 with the open sides loaded and the choice
-// and the map's bytes looked up and stored in each carve; 198 with one lane
+// 32: a reset takes 72 us, 78 with the goal and the places in the order found in
+// passes of their own, 91 with the open sides loaded and the choice and the
+// map's bytes looked up and stored in each carve; 198 with one lane
 // walking and two moves a node.)
 // FAST_SMEM: the fast part lies in shared memory (an instance of its own, so
 // that the compiler knows the address space).
@@ -768,33 +769,39 @@ __device__ __forceinline__ void gen_maze(const Params& p, int e, uint32_t ep, ui
     }
   }
   __syncwarp();
-  // the nodes and the passages to them become floor, all lanes on their own
-  // (a / q = a r >> 20: a < 2^13, q <= 64)
+  // The nodes and the passages to them become floor, each node learns its
+  // place in the visiting order, and the goal is found: the deepest node, ties
+  // to the smallest index (n < 4096). All lanes on their own, four nodes at a
+  // time (the order may lie in global memory); a / q = a r >> 20: a < 2^13, q <= 64.
   const uint32_t r_q = ((1u << 20) + (uint32_t)q - 1u) / (uint32_t)q;
-  for (int k = lane; k < n; k += 32) {
-    const uint32_t v = m.seq[k], a = v & 0xffffu;
-    const int y1 = (int)(a * r_q >> 20), x = (int)a - y1 * q, y = y1 - 1, d = (int)(v >> 30);
-    const int c = (2 * y + 1) * S + 2 * x + 1, dc = d & 1 ? 1 : S;
-    smap[c] = 0;
-    if (k > 0) smap[(d + 1) & 2 ? c - dc : c + dc] = 0;
-    m.seq[k] = (uint32_t)(y * nn + x) | (v & 0x0fff0000u);
-  }
-  __syncwarp();
-  // the goal: the deepest node, ties to the smallest index (n < 4096)
+  uint16_t* const disc = m.stack;
   uint32_t top = 0u;
-  for (int k = lane; k < n; k += 32) {
-    const uint32_t v = m.seq[k], key = (v >> 16) << 12 | (4095u - (v & 0xffffu));
-    top = key > top ? key : top;
+  for (int k0 = lane; k0 < n; k0 += 128) {
+    uint32_t v[4];
+#pragma unroll
+    for (int h = 0; h < 4; ++h) v[h] = k0 + 32 * h < n ? m.seq[k0 + 32 * h] : 0u;
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+      const int k = k0 + 32 * h;
+      if (k >= n) break;
+      const uint32_t a = v[h] & 0xffffu, depth = v[h] & 0x0fff0000u;
+      const int y1 = (int)(a * r_q >> 20), x = (int)a - y1 * q, y = y1 - 1, d = (int)(v[h] >> 30);
+      const int c = (2 * y + 1) * S + 2 * x + 1, dc = d & 1 ? 1 : S;
+      const uint32_t node = (uint32_t)(y * nn + x), key = depth >> 4 | (4095u - node);
+      smap[c] = 0;
+      if (k > 0) smap[(d + 1) & 2 ? c - dc : c + dc] = 0;
+      m.seq[k] = node | depth;
+      disc[node] = (uint16_t)k;
+      top = key > top ? key : top;
+    }
   }
   top = __reduce_max_sync(0xffffffffu, top);
-  const int goal = 4095 - (int)(top & 4095u), goal_d = (int)(top >> 12);
-  // the nodes' places in the visiting order
-  uint16_t* const disc = m.stack;
-  for (int k = lane; k < n; k += 32) disc[m.seq[k] & 0xffffu] = (uint16_t)k;
   __syncwarp();
+  const int goal = 4095 - (int)(top & 4095u), goal_d = (int)(top >> 12);
   // the door sits on edge ceil(d / 2) of the path to the goal: between its nodes at depths j - 1 and j
   const int j = (goal_d + 1) / 2, k_goal = disc[goal];
   uint32_t ka = 0u, kb = 0u;
+#pragma unroll 4
   for (int k = lane; k <= k_goal; k += 32) {
     const int depth = (int)(m.seq[k] >> 16);
     if (depth == j) kb = (uint32_t)k;
@@ -804,8 +811,9 @@ __device__ __forceinline__ void gen_maze(const Params& p, int e, uint32_t ep, ui
   kb = __reduce_max_sync(0xffffffffu, kb);
   // the door's subtree: visits kb .. d1 - 1
   uint32_t d1_min = (uint32_t)n;
-  for (int k = lane; k < n; k += 32)
-    if (k > (int)kb && (int)(m.seq[k] >> 16) <= j && (uint32_t)k < d1_min) d1_min = (uint32_t)k;
+#pragma unroll 4
+  for (int k = (int)kb + 1 + lane; k < n; k += 32)
+    if ((int)(m.seq[k] >> 16) <= j && (uint32_t)k < d1_min) d1_min = (uint32_t)k;
   const int d0 = (int)kb, d1 = (int)__reduce_min_sync(0xffffffffu, d1_min);
   const int node_a = (int)(m.seq[ka] & 0xffffu), node_b = (int)(m.seq[kb] & 0xffffu);
   const int dxc = node_a % nn + node_b % nn + 1, dyc = node_a / nn + node_b / nn + 1;
