@@ -353,7 +353,8 @@ jx_status jx_launch_shape(const jx_env* env, int32_t* grid, int32_t* block, int3
 /* Launch shape of the env kernel in a jx_rollout of `steps` steps (see
  * jx_rollout): as jx_launch_shape, plus the steps per hand-off chunk (0: every
  * warp runs whole envs). For an env routed
- * through the batched kernel (jx_autotune), the batch's shape and chunk 0.
+ * through the batched kernel (jx_autotune) whose rollouts do not take two passes,
+ * the batch's shape and chunk 0.
  * JX_EINVAL for steps < 1. */
 jx_status jx_rollout_shape(const jx_env* env, int32_t steps, int32_t* grid, int32_t* block, int32_t* smem_bytes,
                            int32_t* chunk);
@@ -440,7 +441,9 @@ jx_status jx_batch_render(jx_batch* batch, void* stream, uint8_t* d_frames);
  * 8, 16, 32 x staging_buffers 1, 2; the first max_trials of them, the
  * default first) on this batch
  * and keeps the fastest. mode 0 times `steps` jx_batch_step launches, mode 1
- * one jx_batch_rollout launch of `steps` steps; each trial starts from
+ * one jx_batch_rollout launch of `steps` steps, or where its time does not
+ * depend on the tiling (2 or more steps, every group rolls out in two passes)
+ * the `steps` steps as in mode 0; each trial starts from
  * jx_batch_reset and is timed with CUDA events after one untimed launch.
  * Uses uniform random actions and allocates its own buffers. Every env is
  * RESET (episode 0) when it returns. trials / ms_per_step (optional, room for
@@ -450,12 +453,12 @@ jx_status jx_batch_autotune(jx_batch* batch, void* stream, int32_t mode, int32_t
                             int32_t* n_trials, jx_tiling* trials, float* ms_per_step);
 
 /* Autotuner of a single env: times the env's own kernel (trial 0, reported as
- * the all-zero tiling; for mode 1, the launch jx_rollout makes for `steps`,
- * in hand-off chunks from 64 steps) and the batched kernel over this env alone under every
+ * the all-zero tiling; for mode 1, what jx_batch_autotune times then: the
+ * launch jx_rollout makes for `steps`, or single steps) and the batched kernel over this env alone under every
  * tiling of jx_batch_autotune's search space (the first max_trials - 1), with
  * jx_batch_autotune's protocol, and keeps the fastest: afterwards jx_reset,
  * jx_step, jx_rollout and jx_render of the env launch the chosen kernel
- * (results are identical either way; jx_debug_rays always uses the env's own
+ * (rollouts in two passes are the same kernels either way; results are identical either way; jx_debug_rays always uses the env's own
  * kernel). Every env is RESET (episode 0) when it returns. Waits for `stream`. */
 jx_status jx_autotune(jx_env* env, void* stream, int32_t mode, int32_t steps, int32_t max_trials,
                       int32_t* n_trials, jx_tiling* trials, float* ms_per_step);

@@ -214,6 +214,11 @@ jx_status pregen_beside(jx_env* env, const jx::Params& p, int steps, cudaStream_
   return JX_OK;
 }
 
+// Whether a rollout walks first and draws afterwards: the same on every route,
+// so that it never takes the batched one (which has neither the builds beside
+// the draw nor the hand-off).
+bool two_passes(const jx_env* env, int steps) { return env->base.stop && steps >= jx::kRolloutMinSteps; }
+
 // A rollout of p.steps steps: walk, draw and the env kernel for what they left,
 // in segments that the camera records hold; envs without records in the env
 // kernel alone.
@@ -838,7 +843,7 @@ jx_status jx_step(jx_env* env, void* stream, const uint8_t* d_actions, uint8_t* 
 jx_status jx_rollout(jx_env* env, void* stream, const uint8_t* d_actions, int32_t steps, uint8_t* d_frames,
                      float* d_rewards, uint8_t* d_dones) {
   if (jx_status st = check_env(env)) return st;
-  if (env->use_batch) return jx_batch_rollout(env->tuned, stream, d_actions, steps, d_frames, d_rewards, d_dones);
+  if (env->use_batch && !two_passes(env, steps)) return jx_batch_rollout(env->tuned, stream, d_actions, steps, d_frames, d_rewards, d_dones);
   if (steps < 1) return fail(JX_EINVAL, "steps must be >= 1 (got %d)", steps);
   if (!d_actions || !d_rewards || !d_dones) return fail(JX_EINVAL, "NULL device pointer");
   if (!d_frames || !aligned16(d_frames)) return fail(JX_EINVAL, "d_frames must be a 16-byte aligned device pointer");
@@ -977,7 +982,8 @@ jx_status jx_autotune(jx_env* env, void* stream, int32_t mode, int32_t steps, in
       jx::Params p = env->base;
       p.rewards = rewards;
       p.dones = dones;
-      if (mode == 1) {
+      // as jx_batch_autotune: the walk and the draw are the same on both routes
+      if (mode == 1 && !two_passes(env, steps)) {
         p.actions = base;
         p.frames = frames;
         p.steps = steps;
@@ -1193,7 +1199,7 @@ jx_status jx_rollout_shape(const jx_env* env, int32_t steps, int32_t* grid, int3
                            int32_t* chunk) {
   if (jx_status st = check_env(env)) return st;
   if (steps < 1) return fail(JX_EINVAL, "steps must be >= 1 (got %d)", steps);
-  if (env->use_batch) {
+  if (env->use_batch && !two_passes(env, steps)) {
     if (chunk) *chunk = 0;
     return jx_batch_launch_shape(env->tuned, grid, block, smem_bytes);
   }

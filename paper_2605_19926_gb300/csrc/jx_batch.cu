@@ -454,6 +454,13 @@ jx_status jx_batch_autotune(jx_batch* batch, void* stream, int32_t mode, int32_t
   if (dg.err != cudaSuccess) return cuda_fail(dg.err, "cudaSetDevice");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const size_t N = (size_t)batch->n_total, F = (size_t)batch->frame_total, T = (size_t)steps;
+  // rollouts of two passes in every group take the same time with every tiling
+  // (prepare_draw): single steps tell the tilings apart. (Uneven rooms of 16,384
+  // envs: a tiling picked among equal rollouts stepped at 205 us in a graph, the
+  // tiling picked by steps at 76.)
+  bool two_pass = mode == 1 && steps >= jx::kRolloutMinSteps;
+  for (const jx_env* env : batch->envs) two_pass = two_pass && env->base.stop;
+  const bool rollouts = mode == 1 && !two_pass;
   TuneBuffers buf;
   const size_t off_frames = jx::host::align256(T * N);
   const size_t off_rewards = off_frames + jx::host::align256(T * F);
@@ -488,7 +495,7 @@ jx_status jx_batch_autotune(jx_batch* batch, void* stream, int32_t mode, int32_t
     if (done >= max_trials) break;
     if (apply_tiling(batch, t) != JX_OK) continue;  // does not fit: not a candidate
     auto run = [&]() -> jx_status {
-      if (mode == 1)
+      if (rollouts)
         return batch_run(batch, jx::MODE_ROLLOUT, s, buf.actions, buf.frames, buf.rewards, buf.dones, steps, false);
       for (size_t k = 0; k < T; ++k)
         if (jx_status r = batch_run(batch, jx::MODE_STEP, s, buf.actions + k * N, buf.frames + k * F,
