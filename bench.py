@@ -548,7 +548,7 @@ def large_record(g: Gpu, n_envs: int, slots: int, steps: int, tiling_text: str, 
     # launches whose steps end episodes (the horizon), against the others
     ends = [int(done_steps[c * T: (c + 1) * T].sum()) for c in range(K // T)]
     normal = [per_launch[c] for c in range(1, K // T) if ends[c] == 0]
-    per_es = recorded_traffic_per_env_step(N, TRAFFIC_LARGE_FILE, BATCH_KERNEL_SOURCES, tiling.as_tuple())
+    per_es = recorded_traffic_per_env_step(N, TRAFFIC_LARGE_FILE, KERNEL_SOURCES, tiling.as_tuple())
     return {
         "metric": "env-steps/s incl. render (frames/s), 128x128 RGB + gray stack",
         "value": g.world * N * K / (ms / 1e3), "unit": "env-steps/s", "n_gpus": g.world, "steps": K, "warmup": 0,

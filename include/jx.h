@@ -210,7 +210,9 @@ jx_status jx_step(jx_env* env, void* stream, const uint8_t* d_actions, uint8_t* 
  * its episode, one lane per env, and leaves a camera record per env and step;
  * a draw renders the records' frames in any order. The env kernel, launched
  * last, then runs the envs whose episode ends in the rollout from that step
- * on. Other rollouts run in the env kernel alone. In the env kernel each env's
+ * on. Next episodes of large mazes in large batches are built beside the draw,
+ * on a stream of the env's own that `stream` waits for (also under capture).
+ * Other rollouts run in the env kernel alone. In the env kernel each env's
  * pose stays in registers and its map in shared memory across its steps. For
  * 64 steps or more (envs without a grayscale stack) they are cut into chunks
  * of 12 steps that the launch's warps take in turn: a warp that finishes a
@@ -364,10 +366,10 @@ jx_status jx_rollout_shape(const jx_env* env, int32_t steps, int32_t* grid, int3
  *
  * A batch ties together G existing envs ("groups"; each is homogeneous, the
  * groups differ in map side, frame size, sprite count, task, seed, ...) and
- * steps all of their environments in ONE launch of a persistent kernel:
- * every warp drains per-group work queues (counters of handed-out envs), the
- * groups taken largest frames first, so warps that finish early move on to
- * the remaining envs. Results are bit-identical to stepping each group alone
+ * steps all of their environments in ONE launch: blocks of a few envs each, the
+ * groups taken largest frames first (resets, renders and what rollouts leave
+ * after their walk and draw run on a persistent kernel whose warps drain
+ * per-group work queues). Results are bit-identical to stepping each group alone
  * with jx_step / jx_rollout / jx_reset / jx_render.
  *
  * Layout of a batch's arrays (the batch's env order): group g's envs occupy
@@ -427,7 +429,7 @@ jx_status jx_batch_launch_shape(const jx_batch* batch, int32_t* grid, int32_t* b
 jx_status jx_batch_launch_count(const jx_batch* batch, uint64_t* count);
 
 /* jx_reset / jx_step / jx_rollout / jx_render of every env of every group in
- * one launch each, with the batch's array layout (above). Asynchronous on
+ * one launch each (a rollout in a few: see jx_rollout), with the batch's array layout (above). Asynchronous on
  * `stream`; allocate nothing; capturable in a CUDA graph. */
 jx_status jx_batch_reset(jx_batch* batch, void* stream, uint8_t* d_frames);
 jx_status jx_batch_step(jx_batch* batch, void* stream, const uint8_t* d_actions, uint8_t* d_frames,
@@ -486,8 +488,8 @@ jx_status jx_graph_destroy(jx_graph* graph);
  * session's life. They submit step requests (one step of all the session's
  * envs, actions from host memory) as they arrive. A dispatcher thread inside
  * the server merges the oldest pending request of every idle session (up to
- * 32 sessions and 2^20 envs per launch) into one launch of the batched
- * persistent kernel (see jx_batch_*), on one of `max_inflight` launch slots,
+ * 32 sessions and 2^20 envs per launch) into one launch (see jx_batch_*; a
+ * single session's is that of jx_step), on one of `max_inflight` launch slots,
  * each with its own stream; requests that arrive while launches run go into
  * the next launch on a free slot, so their work overlaps on the device. A
  * session has at most one request on the device; its later requests wait in

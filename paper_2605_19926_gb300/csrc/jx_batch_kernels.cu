@@ -1,5 +1,6 @@
-// jx_batch_kernels.cu — the batched kernel (env groups of different sizes in
-// one persistent launch over per-group work queues) and its launches.
+// jx_batch_kernels.cu — the batched kernels (env groups of different sizes in one
+// launch: steps by blocks of a few envs, the rest persistent over per-group
+// work queues) and their launches.
 #include "jx_device.cuh"
 
 namespace jx {

@@ -1,5 +1,6 @@
-// jx_kernels.cu — the env kernel (one env config per launch, rollouts in
-// hand-off chunks), the kernels that build next episodes ahead (a count, the
+// jx_kernels.cu — the env kernel (one env config per launch, rollouts or what a
+// walk left of them in hand-off chunks), the team kernel (a block of warps per
+// env), the kernels that build next episodes ahead (a count, the
 // walls of the builds that start, then one lane per env advancing its build),
 // and their host side: launch shape queries, launches, the per-warp shared
 // memory layout.
