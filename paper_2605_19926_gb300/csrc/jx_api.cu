@@ -337,18 +337,30 @@ void choose_rows(Params& p, int max_rows, int warps, int blocks, size_t smem_per
 // take a team where a frame has more than 64 x 64 pixels (a grayscale plane
 // counted as a third more); one room env whose episode never ends takes 5.4 /
 // 4.4 us a call. Renders begin nothing: 55 envs, 128 x 128, 18.8 / 6.4 us.
-bool steps_end(const jx_env* env) { return env->cfg.task != JX_TASK_ROOMS || env->cfg.horizon > 0; }
-
-bool takes_team(const jx_env* env, int mode) {
+bool takes_team(const jx_env* env, int mode, bool ends) {
   if (env->team.staging == 0) return false;
   if (mode == MODE_RENDER) return true;
   const int px = env->cfg.frame_h * env->cfg.frame_w * (env->cfg.gray_stack ? 4 : 3);
-  return mode == MODE_STEP && (!steps_end(env) || px > 3 * 64 * 64);
+  return mode == MODE_STEP && (!ends || px > 3 * 64 * 64);
+}
+
+// Generated rooms hold no goal; a state set by the host may.
+bool steps_end(const jx_env* env) {
+  return env->cfg.task != JX_TASK_ROOMS || env->cfg.horizon > 0 || env->goals_set.load(std::memory_order_relaxed);
+}
+
+// A captured step is replayed on whatever state is set after the capture.
+bool captured(cudaStream_t stream) {
+  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(stream, &status) == cudaSuccess) return status != cudaStreamCaptureStatusNone;
+  (void)cudaGetLastError();  // the legacy stream while another stream is captured: the launch reports it
+  return true;
 }
 
 cudaError_t launch_frame(const jx_env* env, const Params& p, int mode, cudaStream_t stream, int* launches) {
   *launches += 1;
-  if (!takes_team(env, mode)) return launch(p, mode, env->grid, false, stream);
+  const bool ends = mode == MODE_STEP && (steps_end(env) || (env->team.staging > 0 && captured(stream)));
+  if (!takes_team(env, mode, ends)) return launch(p, mode, env->grid, false, stream);
   Params q = env->team;
   q.actions = p.actions;
   q.frames = p.frames;
@@ -356,7 +368,7 @@ cudaError_t launch_frame(const jx_env* env, const Params& p, int mode, cudaStrea
   q.dones = p.dones;
   q.bulk_wait_rounds = p.bulk_wait_rounds;
   cudaError_t err = team_launch(q, mode, stream);
-  if (err != cudaSuccess || mode != MODE_STEP || !steps_end(env)) return err;
+  if (err != cudaSuccess || !ends) return err;
   *launches += 1;
   return launch(p, MODE_BEGIN, env->grid, false, stream);
 }
@@ -1121,6 +1133,8 @@ jx_status jx_set_state(jx_env* env, const void* h_buf, size_t bytes) {
   const uint8_t* nspr = reinterpret_cast<const uint8_t*>(fld(JX_F_NSPR));
   float* c0 = reinterpret_cast<float*>(fld(JX_F_COS0));
   float* s0 = reinterpret_cast<float*>(fld(JX_F_SIN0));
+  const uint8_t* type = reinterpret_cast<const uint8_t*>(fld(JX_F_SPR_TYPE));
+  bool goals = false;
   for (int i = 0; i < N; ++i) {
     if (cx[i] < 0 || cx[i] >= S || cy[i] < 0 || cy[i] >= S || !(fx[i] >= 0.f && fx[i] < 1.f) ||
         !(fy[i] >= 0.f && fy[i] < 1.f))
@@ -1132,13 +1146,17 @@ jx_status jx_set_state(jx_env* env, const void* h_buf, size_t bytes) {
       return fail(JX_EINVAL, "env %d: %d sprites in use, at most %d", i, nspr[i], env->cfg.max_sprites);
     c0[i] = (float)std::cos((double)th[i]);
     s0[i] = (float)std::sin((double)th[i]);
+    for (int k = 0; k < nspr[i]; ++k) goals = goals || type[(size_t)i * env->cfg.max_sprites + k] == jx::kSprGoal;
   }
   DeviceGuard g(env->device);
   cudaError_t err = cudaDeviceSynchronize();
+  if (goals) env->goals_set.store(true, std::memory_order_relaxed);
   if (err == cudaSuccess) err = cudaMemcpy(env->state, blob.data(), bytes, cudaMemcpyHostToDevice);
   if (err == cudaSuccess) err = jx::plane_launch(env->base, 0);
   if (err == cudaSuccess) err = cudaDeviceSynchronize();
-  return err == cudaSuccess ? JX_OK : cuda_fail(err, "set_state");
+  if (err != cudaSuccess) return cuda_fail(err, "set_state");
+  env->goals_set.store(goals, std::memory_order_relaxed);
+  return JX_OK;
 }
 
 jx_status jx_sync_status(jx_env* env, void* stream) {
@@ -1189,7 +1207,7 @@ jx_status jx_launch_count(const jx_env* env, uint64_t* count) {
 jx_status jx_launch_shape(const jx_env* env, int32_t* grid, int32_t* block, int32_t* smem_bytes) {
   if (jx_status st = check_env(env)) return st;
   if (env->use_batch) return jx_batch_launch_shape(env->tuned, grid, block, smem_bytes);
-  const bool team = jx::host::takes_team(env, jx::MODE_STEP);
+  const bool team = jx::host::takes_team(env, jx::MODE_STEP, jx::host::steps_end(env));
   if (grid) *grid = team ? env->cfg.n_envs : env->grid;
   if (block) *block = team ? 32 * env->team.staging : jx::kThreads;
   if (smem_bytes) *smem_bytes = team ? jx::team_block_bytes(env->team) : env->smem_block;

@@ -31,7 +31,6 @@ constexpr int kUnlocked = 20;  // + colour: unlocked doors
 constexpr int kDoor = kLocked;  // the red locked door of the generated mazes
 constexpr int kTaskAscii = 3;
 constexpr int kSprKey = 1;
-constexpr int kSprGoal = 2;
 constexpr int kSprKeyBlue = 4;
 constexpr int kSprKeyYellow = 5;
 // colour of a key sprite type, -1 for other types

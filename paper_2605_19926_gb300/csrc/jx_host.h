@@ -47,6 +47,8 @@ struct jx_env {
   uint8_t* stage = nullptr;
   size_t stage_frames_off = 0, stage_rewards_off = 0, stage_dones_off = 0;
   std::atomic<uint64_t> launches{0};
+  // whether the state last set by the host (jx_set_state) holds a goal sprite
+  std::atomic<bool> goals_set{false};
   // jx_autotune: a private one-group batch over this env, and whether the
   // env's launches go through it (the batched kernel with tuned tiles)
   jx_batch* tuned = nullptr;
@@ -103,7 +105,9 @@ void choose_rows(Params& p, int max_rows, int warps, int blocks, size_t smem_per
 // The launch of a step, render, reset or ray query over p (env's parameters
 // with the call's pointers): a team per env for small batches, else the env
 // kernel. Adds the kernels launched to *launches.
-bool takes_team(const jx_env* env, int mode);
+// ends: the step's episodes can end.
+bool takes_team(const jx_env* env, int mode, bool ends);
+bool steps_end(const jx_env* env);
 cudaError_t launch_frame(const jx_env* env, const Params& p, int mode, cudaStream_t stream, int* launches);
 
 // jx_env_bytes / jx_create_in, for the ASCII task too (ascii: the map text, or null).

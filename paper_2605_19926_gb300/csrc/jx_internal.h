@@ -10,6 +10,7 @@
 namespace jx {
 
 constexpr int kMaxSprites = 16;
+constexpr int kSprGoal = 2;
 constexpr int kBulkWaitRounds = 1 << 16;  // default try_wait polls before a bulk map copy counts as late
 constexpr int kMaxSide = 128;
 constexpr int kMaxH = 256;

@@ -853,3 +853,48 @@ def test_late_handoff_is_reported_and_later_rollouts_exact():
     torch.cuda.synchronize()
     assert (ref.env.get_state() == run.env.get_state()).all()
     run.env.sync_status()
+
+
+@pytest.mark.parametrize("call", ["step", "captured", "rollout", "host"])
+def test_goal_in_endless_rooms_ends_the_episode(call):
+    """Rooms without a horizon whose state, set by the host, holds a goal: the
+    agent that walks onto it starts its next episode, in lockstep with the
+    oracle, in single steps, in steps captured before the state was set, in
+    rollouts of one step and in host steps."""
+    cfg = inputs.rooms(n_envs=6, map_side=16, wall_prob=0.0, seed=78, max_sprites=2)
+    run = Run(cfg)
+    run.reset()
+    graph = torch.cuda.CUDAGraph()
+    if call == "captured":
+        with torch.cuda.graph(graph):
+            run.env.step(run.actions, run.frames, run.rewards, run.dones)
+    blob = run.env.get_state()
+    f = run.env.fields(blob)
+    f["cell_x"][:], f["cell_y"][:], f["frac_x"][:], f["frac_y"][:] = 3, 5, 0.45, 0.5
+    f["theta0"][:], f["turn"][:] = 0.0, 0
+    f["nspr"][:], f["spr_x"][:], f["spr_y"][:] = 2, 9.5, 9.5
+    f["spr_type"][:] = 3
+    f["spr_x"][::2, 1], f["spr_y"][::2, 1], f["spr_type"][::2, 1] = 4.5, 5.5, 2  # a goal on the cell ahead
+    run.env.set_state(blob)
+
+    def step(actions):
+        run.actions.copy_(torch.from_numpy(actions))
+        if call == "captured":
+            graph.replay()
+        elif call == "rollout":
+            run.env.rollout(run.actions[None], run.frames[None], run.rewards[None], run.dones[None])
+        elif call == "host":
+            fr, rw, dn = (np.empty(tuple(t.shape), d) for t, d in ((run.frames, np.uint8), (run.rewards, np.float32),
+                                                                 (run.dones, np.uint8)))
+            run.env.step_host(actions, fr, rw, dn)
+            return fr, rw, dn
+        else:
+            run.env.step(run.actions, run.frames, run.rewards, run.dones)
+        torch.cuda.synchronize()
+        return run.frames.cpu().numpy(), run.rewards.cpu().numpy(), run.dones.cpu().numpy()
+
+    run.step = step
+    stats = Stats()
+    lockstep(run, stats, 12, seed=0, action_fn=lambda seed, step, n: np.ones(n, np.uint8))
+    stats.check()
+    assert stats.goal_events == 3 and stats.resets == 3, stats
