@@ -30,8 +30,13 @@ struct jx_batch {
   int block_smem = 0;
   int grid[5] = {};  // per mode
   uint32_t* queue = nullptr;
+  // Maze work spaces of the groups' largest map, then the bits of those in use
+  // (null without mazes). Laid out once: captured steps keep these pointers
+  // when the tiling changes, and find the bits where later steps find them.
   uint8_t* scratch = nullptr;
-  size_t scratch_bytes = 0;
+  size_t scratch_stride = 0;
+  int work_spaces = 0;
+  uint32_t* gen_slots = nullptr;
   std::atomic<uint64_t> launches{0};
 };
 
@@ -60,13 +65,12 @@ jx_status check_tiling(const jx_tiling& t) {
   return JX_OK;
 }
 
-// Lay out every group for tiling t, size the launch and (re)allocate the
-// maze work space. Leaves the batch unchanged on failure.
+// Lay out every group for tiling t and size the launches. Leaves the batch
+// unchanged on failure.
 jx_status apply_tiling(jx_batch* b, const jx_tiling& t) {
   if (jx_status st = check_tiling(t)) return st;
   jx::BatchParams bp{};
   bp.n_groups = (int32_t)b->order.size();
-  size_t stride = 0;
   int warp_bytes = 0;
   for (int i = 0; i < bp.n_groups; ++i) {
     const jx_env* env = b->envs[b->order[i]];
@@ -78,7 +82,10 @@ jx_status apply_tiling(jx_batch* b, const jx_tiling& t) {
                           b->reserved);
     p.out_stride = (int32_t)b->n_total;
     p.frame_step = (size_t)b->frame_total;
-    stride = std::max(stride, jx::gen_scratch_bytes(env->cfg.task, S));
+    p.gen_scratch = b->scratch;
+    p.gen_scratch_stride = b->scratch_stride;
+    p.gen_slots = b->gen_slots;
+    p.n_gen_slots = b->work_spaces;
     warp_bytes = std::max(warp_bytes, p.warp_bytes);
     bp.g[i] = p;
   }
@@ -87,49 +94,20 @@ jx_status apply_tiling(jx_batch* b, const jx_tiling& t) {
   if ((size_t)smem > b->optin)
     return fail(JX_EINVAL, "tiling needs %d bytes of shared memory per block (limit %zu)", smem, b->optin);
   int grid[5] = {};
-  int64_t max_resident = 0;  // blocks
   for (int mode : kModes) {
     int bps = 0;
     cudaError_t err = jx::batch_blocks_per_sm(mode, t.cols_per_lane, jx::batch_spec(bp), t.warps_per_block, smem, &bps);
     if (err != cudaSuccess) return cuda_fail(err, "occupancy query");
     if (bps < 1) return fail(JX_EINVAL, "batched kernel cannot be resident with %d bytes of shared memory", smem);
     const int64_t need = (b->n_total + t.warps_per_block - 1) / t.warps_per_block;
-    const int64_t cap = (int64_t)bps * b->num_sms;
+    int64_t cap = (int64_t)bps * b->num_sms;
+    if (b->scratch) cap = std::min<int64_t>(cap, b->work_spaces / t.warps_per_block);  // a space per warp
     grid[mode] = (int)std::min(need, cap);
     if (mode == jx::MODE_STEP) {  // not persistent: a block per warps_per_block envs of a group
       int64_t blocks = 0;
       for (int i = 0; i < bp.n_groups; ++i) blocks += (bp.g[i].n + t.warps_per_block - 1) / t.warps_per_block;
       grid[mode] = (int)blocks;
     }
-    max_resident = std::max(max_resident, cap);
-  }
-  // the work space of each resident warp, then the bits of the spaces in use
-  const size_t warps = (size_t)max_resident * t.warps_per_block;
-  const size_t slots_off = jx::host::align256(stride * warps);
-  const size_t scratch_need = stride > 0 ? slots_off + jx::gen_slot_bytes((int64_t)warps) : 0;
-  if (scratch_need > b->scratch_bytes) {
-    uint8_t* fresh = nullptr;
-    cudaError_t err = cudaMalloc(&fresh, scratch_need);
-    if (err != cudaSuccess) return fail(JX_ENOMEM, "cudaMalloc of %zu scratch bytes failed", scratch_need);
-    if (b->scratch) {
-      cudaDeviceSynchronize();  // launches in flight may still use the old work space
-      cudaFree(b->scratch);
-    }
-    b->scratch = fresh;
-    b->scratch_bytes = scratch_need;
-  }
-  uint32_t* slots = stride > 0 ? reinterpret_cast<uint32_t*>(b->scratch + slots_off) : nullptr;
-  if (slots) {
-    cudaError_t err = cudaDeviceSynchronize();  // steps in flight hold spaces of the former layout
-    if (err == cudaSuccess) err = cudaMemset(slots, 0, jx::gen_slot_bytes((int64_t)warps));
-    if (err == cudaSuccess) err = cudaDeviceSynchronize();
-    if (err != cudaSuccess) return cuda_fail(err, "clearing the maze work spaces");
-  }
-  for (int i = 0; i < bp.n_groups; ++i) {
-    bp.g[i].gen_scratch = stride > 0 ? b->scratch : nullptr;
-    bp.g[i].gen_scratch_stride = stride;
-    bp.g[i].gen_slots = slots;
-    bp.g[i].n_gen_slots = (int32_t)warps;
   }
   bp.queue = b->queue;
   b->bp = bp;
@@ -158,6 +136,27 @@ jx_status prepare_draw(jx_batch* b) {
   cudaError_t err = jx::batch_rollout_prepare(bq);
   if (err != cudaSuccess) return cuda_fail(err, "kernel attributes");
   b->draw_slots = jx::kMinBlocksPerSm * b->num_sms;
+  return JX_OK;
+}
+
+// The maze work spaces of the batch and their bits, all free.
+jx_status alloc_work_spaces(jx_batch* b) {
+  size_t stride = 0;
+  for (const jx_env* env : b->envs) stride = std::max(stride, jx::gen_scratch_bytes(env->cfg.task, env->cfg.map_side));
+  if (stride == 0) return JX_OK;
+  const int spaces = jx::kWorkSpacesPerSm * b->num_sms;
+  const size_t bits_off = jx::host::align256(stride * (size_t)spaces);
+  const size_t bytes = bits_off + jx::gen_slot_bytes(spaces);
+  cudaError_t err = cudaMalloc(&b->scratch, bytes);
+  if (err != cudaSuccess) {
+    b->scratch = nullptr;
+    return fail(JX_ENOMEM, "cudaMalloc of %zu maze work bytes failed", bytes);
+  }
+  if ((err = cudaMemset(b->scratch + bits_off, 0, bytes - bits_off)) != cudaSuccess)
+    return cuda_fail(err, "clearing the maze work spaces");
+  b->scratch_stride = stride;
+  b->work_spaces = spaces;
+  b->gen_slots = reinterpret_cast<uint32_t*>(b->scratch + bits_off);
   return JX_OK;
 }
 
@@ -340,11 +339,10 @@ jx_status jx_batch_create(jx_env* const* groups, int32_t n_groups, const jx_tili
     jx_batch_destroy(b);
     return cuda_fail(err, "cudaMemset of the work queues");
   }
-  if (jx_status st = apply_tiling(b, t)) {
-    jx_batch_destroy(b);
-    return st;
-  }
-  if (jx_status st = prepare_draw(b)) {
+  jx_status st = alloc_work_spaces(b);
+  if (st == JX_OK) st = apply_tiling(b, t);
+  if (st == JX_OK) st = prepare_draw(b);
+  if (st != JX_OK) {
     jx_batch_destroy(b);
     return st;
   }

@@ -36,6 +36,10 @@ enum MapKind { MAP_BYTES = 0, MAP_BITS = 1, MAP_RUNTIME = 2 };
 constexpr int kMaxGroups = 32;
 constexpr int kBatchMaxThreads = 128;  // up to 4 warps (envs in flight) per block
 constexpr int kBatchMinBlocks = kMinBlocksPerSm * 32 / kBatchMaxThreads;
+// Maze work spaces per SM of a batch or a server's launch slot: one for each
+// warp of a batched kernel that can be resident (they take 64 registers a
+// thread or more).
+constexpr int kWorkSpacesPerSm = 32;
 
 enum Purpose : uint32_t {
   P_WALL = 1,

@@ -396,7 +396,7 @@ jx_status jx_server_create(int device, uint64_t budget_bytes, int32_t max_sessio
   sv->tiling = t;
   sv->max_map_side = max_map_side;
   sv->scratch_stride = jx::gen_scratch_bytes(JX_TASK_MAZE_KEYDOOR, max_map_side & ~1);
-  sv->max_warps = 32 * sv->num_sms;  // at least the resident warps of a step
+  sv->max_warps = jx::kWorkSpacesPerSm * sv->num_sms;
   sv->max_launch_envs = 1 << 20;
   sv->budget = (size_t)budget_bytes;
   sv->max_sessions = max_sessions;

@@ -325,3 +325,44 @@ def test_env_autotune_and_pinned_tilings_give_identical_results(cfg):
         fb, rb, db = tuned.step(act)
         assert (fa == fb).all() and (ra == rb).all() and (da == db).all(), s
     assert (ref.env.get_state() == tuned.env.get_state()).all()
+
+
+@pytest.mark.parametrize("order", [0, 1])
+def test_captured_steps_replay_after_the_tiling_changed(order):
+    """Steps captured under one tiling, replayed in turn with steps under
+    another that keeps more or fewer warps resident: maze groups whose builds
+    take a work space, all of whose episodes end every few steps, give the
+    frames, outputs and state of single steps, and no build goes without a
+    space."""
+    cfgs = [inputs.maze_keydoor(n_envs=2500, map_side=64, seed=111, horizon=3),
+            inputs.maze_rooms(n_envs=300, map_side=128, seed=112, horizon=2, frame_h=32, frame_w=48, gray_stack=0)]
+    tilings = [tiling(1, 1, 8, 8), tiling(4, 1, 0, 64, 2)]
+    first, second = tilings[order], tilings[1 - order]
+    ref, run = BatchRun(cfgs), BatchRun(cfgs, first)
+    ref.reset()
+    run.reset()
+    T = 3
+    acts = torch.zeros((T, run.batch.n), dtype=torch.uint8, device=run.dev)
+    frames = torch.zeros((T, run.batch.frame_bytes), dtype=torch.uint8, device=run.dev)
+    rewards = torch.zeros((T, run.batch.n), dtype=torch.float32, device=run.dev)
+    dones = torch.zeros((T, run.batch.n), dtype=torch.uint8, device=run.dev)
+    graph = run.batch.capture(acts, frames, rewards, dones)
+    run.batch.tiling = second
+    for rep in range(3):
+        acts.copy_(torch.from_numpy(np.stack([inputs.actions(113 + rep, s, run.batch.n) for s in range(T)])))
+        graph.launch()
+        for t in range(T):
+            ref.actions.copy_(acts[t])
+            ref.batch.step(ref.actions, ref.frames, ref.rewards, ref.dones)
+            assert torch.equal(ref.frames, frames[t]), (rep, t)
+            assert torch.equal(ref.rewards, rewards[t]) and torch.equal(ref.dones, dones[t]), (rep, t)
+        for s in range(2):
+            act = inputs.actions(119 + rep, s, run.batch.n)
+            fa, ra, da = ref.step(act)
+            fb, rb, db = run.step(act)
+            assert (fa == fb).all() and (ra == rb).all() and (da == db).all(), (rep, s)
+    for a, b in zip(ref.envs, run.envs):
+        assert (a.get_state() == b.get_state()).all()
+        a.sync_status()
+        b.sync_status()
+    graph.close()
