@@ -144,7 +144,9 @@ jx_status alloc_work_spaces(jx_batch* b) {
   size_t stride = 0;
   for (const jx_env* env : b->envs) stride = std::max(stride, jx::gen_scratch_bytes(env->cfg.task, env->cfg.map_side));
   if (stride == 0) return JX_OK;
-  const int spaces = jx::kWorkSpacesPerSm * b->num_sms;
+  // never more mazes at once than envs; the persistent modes' last block may be short of envs
+  const int spaces = (int)std::min<int64_t>(b->n_total + jx::kBatchMaxThreads / 32 - 1,
+                                            (int64_t)jx::kWorkSpacesPerSm * b->num_sms);
   const size_t bits_off = jx::host::align256(stride * (size_t)spaces);
   const size_t bytes = bits_off + jx::gen_slot_bytes(spaces);
   cudaError_t err = cudaMalloc(&b->scratch, bytes);

@@ -366,3 +366,17 @@ def test_captured_steps_replay_after_the_tiling_changed(order):
         a.sync_status()
         b.sync_status()
     graph.close()
+
+
+def test_small_batch_takes_little_maze_work_space():
+    """A batch of one 128 x 128 maze env (32 KB of work a build) takes work
+    spaces for its envs, not for every warp the chip holds; so does the private
+    batch of an env pinned to a tiling. (Allocations are counted in pieces of
+    2 MB: two of them each.)"""
+    env = jx.Env(inputs.maze_rooms(n_envs=1, map_side=128, seed=121, gray_stack=0, frame_h=32, frame_w=32))
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    batch = jx.Batch([env])
+    env.tiling = tiling(1, 1, 8, 8)
+    assert free - torch.cuda.mem_get_info()[0] <= 8 << 20
+    del batch
