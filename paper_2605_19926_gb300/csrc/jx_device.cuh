@@ -1313,10 +1313,11 @@ __device__ __forceinline__ void gen_ascii(const Params& p, int e, uint32_t ep, u
 }
 
 // A free work space of Params::gen_slots, or -1 after a bounded search (there
-// are as many as resident warps, so one is always free). Every lane gets it.
+// is one per warp that can be building, so one is always free), or in a launch
+// that has none. Every lane gets it.
 __device__ __forceinline__ int take_gen_slot(const Params& p, int lane) {
   int slot = -1;
-  if (lane == 0) {
+  if (lane == 0 && p.n_gen_slots > 0) {
     const int words = (p.n_gen_slots + 31) >> 5;
     int w = (int)((blockIdx.x * 37u) % (unsigned)words);
     for (int it = 0; it < 1 << 20 && slot < 0; ++it, w = w + 1 == words ? 0 : w + 1) {

@@ -86,7 +86,8 @@ struct Params {
   size_t gen_scratch_stride;
   // Batched steps (blocks handed out in order, no warp index to tell work
   // spaces apart): one bit per slot of gen_scratch, taken and given back by
-  // the warps that build a maze; there are as many slots as resident warps.
+  // the warps that build a maze; there is a slot per warp that can be building
+  // (in an env's own launches, which index gen_scratch by warp, none).
   uint32_t* gen_slots;
   int32_t n_gen_slots;
   // The next episode of each env, built ahead by the lane-parallel
