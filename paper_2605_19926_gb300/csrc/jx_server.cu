@@ -145,10 +145,11 @@ struct jx_server {
   std::map<int, int> occupancy;  // 2 x block shared memory bytes + kernel spec -> blocks per SM
   std::mutex mu;
   std::mutex open_mu;  // serialises the admin stream
-  std::condition_variable cv_work, cv_done;
+  std::condition_variable cv_work, cv_done, cv_issued;
   std::thread worker;
   bool stop = false;
   bool paused = false;
+  bool issuing = false;  // the dispatcher issues a launch (without the lock)
   jx_status worker_status = JX_OK;
   std::string worker_msg;
   // counters
@@ -225,9 +226,10 @@ jx_status issue(jx_server* sv, Slot& sl, const std::vector<Session*>& chosen) {
 }
 
 // Takes the head requests of `chosen` for one launch on slot `sl`. The lock is
-// held while the requests are taken and given up while the launch is issued
-// (some 5 us that every submitting client would wait for): sessions in flight
-// are not freed, and the slots are the dispatcher's alone.
+// held while the requests are taken and the launch is counted, and given up
+// while it is issued (some 5 us that every submitting client would wait for):
+// sessions in flight are not freed, the slots are the dispatcher's alone, and
+// a pause waits until the launch is out.
 jx_status dispatch(jx_server* sv, Slot& sl, std::vector<Session*>& chosen, std::unique_lock<std::mutex>& lk) {
   std::stable_sort(chosen.begin(), chosen.end(), [](const Session* a, const Session* b) {
     const int64_t fa = (int64_t)a->p.H * a->p.W, fb = (int64_t)b->p.H * b->p.W;
@@ -245,17 +247,27 @@ jx_status dispatch(jx_server* sv, Slot& sl, std::vector<Session*>& chosen, std::
     s->pending.pop_front();
     s->in_flight = true;
   }
-  lk.unlock();
-  const jx_status st = issue(sv, sl, chosen);
-  lk.lock();
-  if (st != JX_OK) return st;
   sl.busy = true;
   sv->inflight++;
-  sv->peak_inflight = std::max(sv->peak_inflight, sv->inflight);
   sv->launches++;
   sv->env_steps += (uint64_t)total;
   sv->groups += chosen.size();
-  return JX_OK;
+  sv->issuing = true;
+  lk.unlock();
+  const jx_status st = issue(sv, sl, chosen);
+  lk.lock();
+  sv->issuing = false;
+  sv->cv_issued.notify_all();
+  if (st == JX_OK) {
+    sv->peak_inflight = std::max(sv->peak_inflight, sv->inflight);
+    return JX_OK;
+  }
+  sl.busy = false;  // not launched
+  sv->inflight--;
+  sv->launches--;
+  sv->env_steps -= (uint64_t)total;
+  sv->groups -= chosen.size();
+  return st;
 }
 
 void worker_loop(jx_server* sv) {
@@ -296,6 +308,7 @@ void worker_loop(jx_server* sv) {
     if (progress) sv->cv_done.notify_all();
     if (sv->worker_status == JX_OK && !sv->paused) {
       for (Slot& sl : sv->slots) {
+        if (sv->paused || sv->stop) break;  // while the lock was given up
         if (sl.busy) continue;
         ready.clear();
         for (auto& kv : sv->sessions) {
@@ -611,8 +624,9 @@ jx_status jx_server_wait(jx_server* sv, uint64_t ticket, double timeout_s) {
 jx_status jx_server_pause(jx_server* sv, int32_t paused) {
   if (jx_status st = check_server(sv)) return st;
   {
-    std::lock_guard<std::mutex> lk(sv->mu);
+    std::unique_lock<std::mutex> lk(sv->mu);
     sv->paused = paused != 0;
+    if (paused) sv->cv_issued.wait(lk, [&]() { return !sv->issuing || !sv->paused; });
   }
   sv->cv_work.notify_all();
   return JX_OK;

@@ -161,3 +161,30 @@ def test_served_frames_match_oracle():
             compare_frames(s.frames.cpu().numpy(), ref, stats)
         s.close()
     stats.check()
+
+
+def test_pause_holds_the_dispatcher_when_it_returns():
+    """Once a pause has returned no further request is launched, and what the
+    counters say is in flight is all there is: requests submitted while it is
+    held stay queued, whatever the dispatcher was doing when it came."""
+    cfgs = [inputs.maze_keydoor(n_envs=8, map_side=32, seed=97 + i, horizon=500) for i in range(2)]
+    act = np.zeros(8, np.uint8)
+    with jx.Server(budget_bytes=1 << 28, max_inflight=4) as server:
+        a, b = (server.open(c) for c in cfgs)
+        for r in range(400):
+            ta = a.submit(act)
+            t0 = time.perf_counter()
+            while time.perf_counter() - t0 < (r % 80) * 1e-6:
+                pass
+            server.pause(True)
+            n0 = server.stats()["launches"]
+            tb = b.submit(act)
+            t0 = time.perf_counter()
+            while time.perf_counter() - t0 < 3e-4:
+                pass
+            assert server.stats()["launches"] == n0, r
+            server.pause(False)
+            server.wait(ta, timeout=30.0)
+            server.wait(tb, timeout=30.0)
+        a.close()
+        b.close()
