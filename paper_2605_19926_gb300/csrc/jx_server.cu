@@ -95,7 +95,10 @@ struct Request {
 struct Session {
   int32_t id = 0;
   jx_env* env = nullptr;
-  jx::Params p{};  // laid out for the server's tiling; outputs point at the session buffers
+  // The session's step as it was opened, so that the dispatcher never reads
+  // what a client may set through the env handle: laid out for the server's
+  // tiling (outputs point at the session buffers), and the env's own.
+  jx::Params p{}, own{};
   uint8_t* block = nullptr;
   size_t block_bytes = 0;
   uint8_t* d_frames = nullptr;
@@ -197,7 +200,7 @@ jx_status issue(jx_server* sv, Slot& sl, const std::vector<Session*>& chosen) {
   cudaError_t err;
   size_t off = 0;
   if (chosen.size() == 1) {
-    jx::Params p = chosen[0]->env->base;
+    jx::Params p = chosen[0]->own;
     step_params(sl, chosen[0], 0, p);
     int launches = 0;
     err = jx::host::launch_frame(chosen[0]->env, p, jx::MODE_STEP, sl.stream, &launches);
@@ -528,7 +531,8 @@ jx_status open_session(jx_server* sv, const jx_config* cfg, const char* ascii, i
     free_session(sv, s);
     return st;
   }
-  jx::Params p = s->env->base;
+  s->own = s->env->base;
+  jx::Params p = s->own;
   p.map_bits = sv->tiling.bits_min_side > 0 && cfg->map_side >= sv->tiling.bits_min_side && cfg->map_side % 8 == 0;
   p.staging = sv->tiling.staging_buffers;
   jx::host::choose_rows(p, sv->tiling.max_rows_per_block, sv->tiling.warps_per_block, jx::kMinBlocksPerSm,

@@ -188,3 +188,24 @@ def test_pause_holds_the_dispatcher_when_it_returns():
             server.wait(tb, timeout=30.0)
         a.close()
         b.close()
+
+
+def test_limits_set_on_a_session_leave_its_requests_alone():
+    """The dispatcher launches a session as it was opened, alone or in the mix:
+    a copy-wait limit that a client sets on the session's env meanwhile (every
+    copy counts as late, see jx_debug_wait_limit) reaches no request."""
+    cfgs = [inputs.rooms(n_envs=12, map_side=68, wall_prob=0.3, seed=99 + i) for i in range(2)]  # byte maps, bulk copies
+    act = np.ones(12, np.uint8)
+    with jx.Server(budget_bytes=1 << 28, max_map_side=128) as server:
+        sessions = [server.open(c) for c in cfgs]
+        for s in sessions:
+            s.env.debug_wait_limit(0)
+        server.wait(sessions[0].submit(act), timeout=30.0)  # alone
+        server.pause(True)
+        tickets = [s.submit(act) for s in sessions]  # together
+        server.pause(False)
+        for t in tickets:
+            server.wait(t, timeout=30.0)
+        for s in sessions:
+            s.env.sync_status()
+            s.close()
