@@ -68,7 +68,10 @@ __device__ __forceinline__ void walk_envs(const Params& p, int e, int t_begin, i
 #pragma unroll
   for (int i = 0; i < kActAhead; ++i) ahead[i] = t_begin + i < t_end ? act[i * stride] : 0u;
   Env r = load_env(p, es);
-  int stop = t_begin == 0 ? p.steps : p.stop[es];  // an earlier part may have stopped the env
+  // An earlier part may have stopped the env. A grayscale stack whose step count
+  // comes from below zero (a state set by the host) is left to the env kernel:
+  // the frame of step 0 writes all four planes, which no order of drawing keeps.
+  int stop = t_begin == 0 ? (p.gray && r.t < 0 ? 0 : p.steps) : p.stop[es];
   const int door_x = p.st.obj[6 * (size_t)es + 4], door_y = p.st.obj[6 * (size_t)es + 5];
   // the sprites that make events: cell x | cell y << 8 | type << 16
   int n_ev = 0;
@@ -157,7 +160,7 @@ __device__ __forceinline__ void walk_envs(const Params& p, int e, int t_begin, i
     return turn < 0 ? tpr - 1 : (turn == tpr ? 0 : turn);
   };
   bool fresh = true;  // the agent's cell has not been looked at for events in this launch
-  bool go = on && stop >= t_begin, bad = false;
+  bool go = on && stop > t_begin, bad = false;  // a stop lies in an earlier part, or at the first step of all
   const size_t first = (size_t)t_begin * stride + e, first_cam = (size_t)t_begin * p.n + e;
   float* rewards = p.rewards + first;
   uint8_t* dones = p.dones + first;

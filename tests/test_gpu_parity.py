@@ -898,3 +898,31 @@ def test_goal_in_endless_rooms_ends_the_episode(call):
     lockstep(run, stats, 12, seed=0, action_fn=lambda seed, step, n: np.ones(n, np.uint8))
     stats.check()
     assert stats.goal_events == 3 and stats.resets == 3, stats
+
+
+@pytest.mark.parametrize("T", [3, 40])
+def test_rollout_from_a_negative_step_count_equals_single_steps(T):
+    """A state set by the host may count an episode's steps from below zero: the
+    step that arrives at 0 writes all four grayscale planes, like an episode's
+    first frame. Rollouts equal single steps, planes included, beside envs with
+    ordinary counts."""
+    cfg = dict(inputs.maze_keydoor(n_envs=40, map_side=16, seed=81, horizon=60), gray_stack=1)
+    N, H, W = cfg["n_envs"], cfg["frame_h"], cfg["frame_w"]
+    a, b = Run(cfg), Run(cfg)
+    a.reset()
+    blob = a.env.get_state()
+    a.env.fields(blob)["t"][:] = np.where(np.arange(N) % 2 == 0, np.arange(N), -1 - np.arange(N) % 5)
+    acts = torch.from_numpy(np.stack([forward_biased_actions(82, s, N) for s in range(T)])).to(a.dev)
+    frames = torch.zeros((T, N, H, W, 3), dtype=torch.uint8, device=a.dev)
+    rewards = torch.zeros((T, N), dtype=torch.float32, device=a.dev)
+    dones = torch.zeros((T, N), dtype=torch.uint8, device=a.dev)
+    for run in (a, b):
+        run.env.set_state(blob)
+    b.env.rollout(acts, frames, rewards, dones)
+    for t in range(T):
+        a.actions.copy_(acts[t])
+        a.env.step(a.actions, a.frames, a.rewards, a.dones)
+        assert torch.equal(a.frames, frames[t]), t
+        assert torch.equal(a.rewards, rewards[t]) and torch.equal(a.dones, dones[t]), t
+    torch.cuda.synchronize()
+    assert (a.env.get_state() == b.env.get_state()).all()
