@@ -380,3 +380,43 @@ def test_small_batch_takes_little_maze_work_space():
     env.tiling = tiling(1, 1, 8, 8)
     assert free - torch.cuda.mem_get_info()[0] <= 8 << 20
     del batch
+
+
+def _long_groups():
+    """Groups with a grayscale stack, of sizes that leave ragged warps; an ASCII
+    group, whose rollouts keep to the batched kernel; mazes enough for next
+    episodes to be built ahead; 256-wide frames; rooms whose episodes never end."""
+    return [
+        dict(inputs.maze_keydoor(n_envs=33, map_side=32, seed=131, horizon=50, frame_h=24, frame_w=32), gray_stack=1),
+        inputs.ascii_env("coloured-rooms", n_envs=7, map_side=24, seed=132, horizon=40, frame_h=16, frame_w=48),
+        inputs.maze_rooms(n_envs=3, map_side=64, seed=133, horizon=200, max_sprites=16, frame_h=5, frame_w=256),
+        inputs.maze_keydoor(n_envs=12801, map_side=64, seed=134, horizon=37, frame_h=8, frame_w=16),
+        inputs.rooms(n_envs=65, map_side=9, seed=135, max_sprites=3, frame_h=21, frame_w=16),
+    ]
+
+
+@pytest.mark.parametrize("groups,T", [((0, 1, 2, 4), 6), ((0, 2), 40), ((0, 1, 2, 3, 4), 129), ((2, 3), 131),
+                                      ((0, 1, 2, 4), 257)])
+def test_batch_rollouts_of_gray_groups_and_over_segments(groups, T):
+    """Rollouts of batches with grayscale stacks, with groups that walk first
+    beside groups that do not, and longer than the 128 steps a walk records
+    (129 and 257 leave a single step at the end): frames, outputs, planes and
+    state equal those of batched steps, from a second rollout too."""
+    cfgs = [_long_groups()[g] for g in groups]
+    ref, run = BatchRun(cfgs), BatchRun(cfgs, tiling(2, 1, 8, 16))
+    ref.reset()
+    run.reset()
+    for rep in range(2):
+        acts = torch.from_numpy(np.stack([forward_biased_actions(137 + rep, s, run.batch.n) for s in range(T)]))
+        acts = acts.to(run.dev)
+        frames, rewards, dones = _rollout(run, acts)
+        for t in range(T):
+            ref.actions.copy_(acts[t])
+            ref.batch.step(ref.actions, ref.frames, ref.rewards, ref.dones)
+            assert torch.equal(ref.frames, frames[t]), (rep, t)
+            assert torch.equal(ref.rewards, rewards[t]) and torch.equal(ref.dones, dones[t]), (rep, t)
+        torch.cuda.synchronize()
+        for a, b in zip(ref.envs, run.envs):
+            assert (a.get_state() == b.get_state()).all(), rep
+    for env in ref.envs + run.envs:
+        env.sync_status()
