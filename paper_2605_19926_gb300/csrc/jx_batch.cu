@@ -219,8 +219,9 @@ jx_status batch_run(jx_batch* b, int mode, cudaStream_t stream, const uint8_t* a
       for (int i = 0; i < bp.n_groups; ++i) bp.g[i].stop = nullptr;
     }
   }
-  cudaError_t err = jx::batch_launch(bp, mode, b->tiling.cols_per_lane, b->tiling.warps_per_block, b->grid[mode],
-                                     stream);
+  const int cols = b->tiling.cols_per_lane, warps = b->tiling.warps_per_block;
+  cudaError_t err = mode == jx::MODE_STEP ? jx::batch_step_launch(bp, cols, warps, stream)
+                                          : jx::batch_launch(bp, mode, cols, warps, b->grid[mode], stream);
   if (err != cudaSuccess) {
     // The kernel's last warp clears the work-queue counters for the next
     // launch; a launch that failed may not have got there, so clear them here

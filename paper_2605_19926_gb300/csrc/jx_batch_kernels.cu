@@ -140,27 +140,27 @@ cudaError_t batch_blocks_per_sm(int mode, int cols, int spec, int warps, int sme
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, k, 32 * warps, smem_bytes);
 }
 
-cudaError_t batch_launch(BatchParams& bp, int mode, int cols, int warps, int grid, cudaStream_t stream) {
-  auto k = batch_kernel_of(mode, cols, batch_spec(bp));
-  if (mode == MODE_STEP) {
-    int64_t blocks = 0;
-    for (int g = 0; g < bp.n_groups; ++g) {
-      bp.first_block[g] = (int32_t)blocks;
-      blocks += (bp.g[g].n + warps - 1) / warps;
-    }
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)blocks);
-    cfg.blockDim = dim3((unsigned)(32 * warps));
-    cfg.dynamicSmemBytes = (size_t)bp.warp_bytes * warps;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k, bp);
+cudaError_t batch_step_launch(BatchParams& bp, int cols, int warps, cudaStream_t stream) {
+  int64_t blocks = 0;
+  for (int g = 0; g < bp.n_groups; ++g) {
+    bp.first_block[g] = (int32_t)blocks;
+    blocks += (bp.g[g].n + warps - 1) / warps;
   }
-  k<<<grid, 32 * warps, (size_t)bp.warp_bytes * warps, stream>>>(bp);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)blocks);
+  cfg.blockDim = dim3((unsigned)(32 * warps));
+  cfg.dynamicSmemBytes = (size_t)bp.warp_bytes * warps;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, batch_step_kernel_of(cols, batch_spec(bp)), bp);
+}
+
+cudaError_t batch_launch(const BatchParams& bp, int mode, int cols, int warps, int grid, cudaStream_t stream) {
+  batch_kernel_of(mode, cols, batch_spec(bp))<<<grid, 32 * warps, (size_t)bp.warp_bytes * warps, stream>>>(bp);
   return cudaGetLastError();
 }
 }  // namespace jx

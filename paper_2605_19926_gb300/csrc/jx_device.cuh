@@ -868,12 +868,6 @@ __device__ __forceinline__ void gen_maze(const Params& p, int e, uint32_t ep, ui
   __syncwarp();
 }
 
-// Zero (floor) bytes among the 16 at q (16-byte aligned).
-__device__ __forceinline__ int floor_bytes16(const uint8_t* q) {
-  const uint4 v = *reinterpret_cast<const uint4*>(q);
-  return 16 - __popc(nonzero4(v.x) | nonzero4(v.y) << 4 | nonzero4(v.z) << 8 | nonzero4(v.w) << 12);
-}
-
 // Shared-memory words one pre-generation lane needs for mazes of side S: the
 // walk's visited bits (one per node) and parent directions (two bits per node).
 __host__ __device__ __forceinline__ int pregen_lane_words(int S) {

@@ -262,9 +262,10 @@ cudaError_t batch_rollout_launch(const BatchParams& bq, int steps, int slots, cu
 // specialised instance, 0 the general one (batch_spec gives it for a launch).
 int batch_spec(const BatchParams& bp);
 cudaError_t batch_blocks_per_sm(int mode, int cols, int spec, int warps, int smem_bytes, int* blocks);
-// `grid` resident blocks; MODE_STEP launches one block per `warps` envs of a
-// group instead (and fills in bp.first_block).
-cudaError_t batch_launch(BatchParams& bp, int mode, int cols, int warps, int grid, cudaStream_t stream);
+// A step: one block per `warps` envs of a group (fills in bp.first_block).
+cudaError_t batch_step_launch(BatchParams& bp, int cols, int warps, cudaStream_t stream);
+// A reset, render or rollout: `grid` resident blocks over the work queues.
+cudaError_t batch_launch(const BatchParams& bp, int mode, int cols, int warps, int grid, cudaStream_t stream);
 inline size_t gen_slot_bytes(int64_t warps) { return 4 * (size_t)((warps + 31) / 32); }  // Params::gen_slots
 
 }  // namespace jx

@@ -421,7 +421,6 @@ cudaError_t kernel_blocks_per_sm(const Params& p, int mode, int* blocks) {
     case MODE_RESET: return blocks_per_sm_mode<MODE_RESET>(p, blocks);
     case MODE_RENDER: return blocks_per_sm_mode<MODE_RENDER>(p, blocks);
     case MODE_ROLLOUT: return blocks_per_sm_mode<MODE_ROLLOUT>(p, blocks);
-    case MODE_BEGIN: return blocks_per_sm_mode<MODE_BEGIN>(p, blocks);
     default: return blocks_per_sm_mode<MODE_RAYS>(p, blocks);
   }
 }

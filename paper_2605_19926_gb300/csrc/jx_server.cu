@@ -221,7 +221,7 @@ jx_status issue(jx_server* sv, Slot& sl, const std::vector<Session*>& chosen) {
     const int wpb = sv->tiling.warps_per_block, smem = bp.warp_bytes * wpb;
     if (blocks_per_sm(sv, smem, jx::batch_spec(bp)) < 1)
       return fail(JX_ECUDA, "batched kernel cannot be resident with %d bytes of shared memory", smem);
-    err = jx::batch_launch(bp, jx::MODE_STEP, sv->tiling.cols_per_lane, wpb, 0, sl.stream);
+    err = jx::batch_step_launch(bp, sv->tiling.cols_per_lane, wpb, sl.stream);
   }
   if (err != cudaSuccess) return cuda_fail(err, "step launch");
   if ((err = cudaEventRecord(sl.done, sl.stream)) != cudaSuccess) return cuda_fail(err, "cudaEventRecord");
