@@ -56,6 +56,8 @@ __host__ __device__ __forceinline__ int walk_warp_bytes(int K) { return 32 * (4 
 // of the env's bit plane that registers hold, the actions of 8 steps come with one round of loads, and the
 // next step's turn-table entry is fetched a step ahead (turns depend on the
 // actions alone).
+// GRAY: as render_env's.
+template <int GRAY>
 __device__ __forceinline__ void walk_envs(const Params& p, int e, int t_begin, int t_end, uint32_t* sm, int lane) {
   const bool on = e < p.n;
   const int es = on ? e : p.n - 1;  // lanes past the last env load its state and store nothing
@@ -71,7 +73,7 @@ __device__ __forceinline__ void walk_envs(const Params& p, int e, int t_begin, i
   // An earlier part may have stopped the env. A grayscale stack whose step count
   // comes from below zero (a state set by the host) is left to the env kernel:
   // the frame of step 0 writes all four planes, which no order of drawing keeps.
-  int stop = t_begin == 0 ? (p.gray && r.t < 0 ? 0 : p.steps) : p.stop[es];
+  int stop = t_begin == 0 ? (GRAY != 0 && p.gray && r.t < 0 ? 0 : p.steps) : p.stop[es];
   const int door_x = p.st.obj[6 * (size_t)es + 4], door_y = p.st.obj[6 * (size_t)es + 5];
   // the sprites that make events: cell x | cell y << 8 | type << 16
   int n_ev = 0;
@@ -346,7 +348,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocksPerSm / kWarpsPerBlock)
   if ((int)blockIdx.x < part.walk_blocks) {
     wait_and_release();
     const int e = ((int)blockIdx.x * kWarpsPerBlock + warp) * 32 + lane;
-    walk_envs(p, e, part.walk_t0, part.walk_t1, reinterpret_cast<uint32_t*>(wbase), lane);
+    walk_envs<GRAY>(p, e, part.walk_t0, part.walk_t1, reinterpret_cast<uint32_t*>(wbase), lane);
     return;
   }
   write_palette(p, WarpSmem{wbase, FillLane{}}, lane);
@@ -372,7 +374,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocksPerSm / kWarpsPerBlock)
     while (g + 1 < bp.n_groups && (int)blockIdx.x >= parts.first_walk[g + 1]) ++g;
     wait_and_release();
     const int e = (((int)blockIdx.x - parts.first_walk[g]) * kWarpsPerBlock + warp) * 32 + lane;
-    walk_envs(bp.g[g], e, parts.g[g].walk_t0, parts.g[g].walk_t1, reinterpret_cast<uint32_t*>(wbase), lane);
+    walk_envs<GRAY>(bp.g[g], e, parts.g[g].walk_t0, parts.g[g].walk_t1, reinterpret_cast<uint32_t*>(wbase), lane);
     return;
   }
   while (g + 1 < bp.n_groups && (int)blockIdx.x >= parts.first_draw[g + 1]) ++g;
