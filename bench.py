@@ -331,7 +331,8 @@ def run_reference(args, cfg: dict):
 
 
 def tiling_dict(t) -> dict:
-    """A launch choice as JSON: all zero means the env's own kernel."""
+    """A launch choice of resets, steps and renders as JSON: all zero means the
+    env's own kernel (rollouts in two passes have kernels of their own)."""
     names = ("warps_per_block", "cols_per_lane", "bits_min_side", "max_rows_per_block", "staging_buffers")
     d = dict(zip(names, t.as_tuple()))
     d["kernel"] = "env kernel" if not any(t.as_tuple()) else "batched kernel"
@@ -392,7 +393,7 @@ class Gpu:
 
 def uneven_record(g: Gpu, n_envs: int, slots: int, steps: int, tiling_text: str, tune_trials: int) -> dict | None:
     """Uneven batching: n_envs envs of 16 (map side, frame size) groups in one
-    persistent launch per rollout of `slots` steps; fixed tiles against
+    call per rollout of `slots` steps; fixed tiles against
     autotuned tiles, and the autotuned step sequence replayed as a CUDA graph
     of `slots` single-step launches. Returns rank 0's record."""
     torch, jx = g.torch, g.jx
@@ -875,7 +876,7 @@ def headline(g: Gpu, args) -> dict | None:
                              traffic_unit="DRAM bytes per launch (ncu record, scaled by env-steps)",
                              algorithmic_bytes_per_step=bytes_total / args.steps,
                              algorithmic_bytes_per_launch=bytes_total / len(plan.launches),
-                             kernel="jx_rollout (env kernel, or the batched kernel when autotuned to it)"),
+                             kernel="rollout_kernel (walk and draw), env_kernel for what they left"),
         "cpu_baseline": cpu,
         "e2e": {"value": e2e_value, "unit": "env-steps/s", "h2d_bytes_per_step": N,
                 "d2h_bytes_per_step": N * H * W * 3 + 4 * N + N,

@@ -159,8 +159,9 @@ jx_status jx_create_ascii(const jx_config* cfg, const char* ascii, int device, j
 
 /* Device bytes of an env of cfg on `device`: one block holding the state, the
  * per-env tables, the maps' bit planes and the maze work space (jx_create also
- * allocates the camera records of its rollouts, at most 24 bytes per env for
- * 128 steps). Validates cfg like jx_create. */
+ * allocates the camera records of its rollouts, ASCII task excepted: 3 KB an
+ * env up to 21,845 envs, 64 MB from there, 384 bytes an env above 174,762).
+ * Validates cfg like jx_create. */
 jx_status jx_env_bytes(const jx_config* cfg, int device, size_t* bytes);
 
 /* jx_create with the env's device block placed in caller memory d_mem
@@ -197,7 +198,7 @@ jx_status jx_reset(jx_env* env, void* stream, uint8_t* d_frames);
 jx_status jx_step(jx_env* env, void* stream, const uint8_t* d_actions, uint8_t* d_frames, float* d_rewards,
                   uint8_t* d_dones);
 
-/* `steps` consecutive calls of jx_step in one kernel launch, for action
+/* `steps` consecutive calls of jx_step in one call (and a few launches), for action
  * streams known in advance (uniform random policies, as the paper's speed
  * measurements use, App. A.1; replayed or scripted actions): step t reads
  * d_actions + t*N and writes d_frames + t*N*H*W*3,
@@ -339,12 +340,15 @@ jx_status jx_sync_status(jx_env* env, void* stream);
 
 /* Number of kernel launches this env has issued since creation. For maze
  * configs with a next-episode block (see jx_create) and batches of many envs
- * (at least 3 x 28 per SM), jx_reset, jx_step and jx_rollout each also launch the three kernels that build episodes ahead (a
- * count, the walls of builds that start, then the build's share of the launch,
- * after a 4-byte cudaMemsetAsync on the same stream; all capturable in a CUDA
- * graph). A jx_rollout in two passes (see there) counts its walk and draw
- * launches and the env kernel's, per 128 steps. Steps of small batches with
- * large frames count a second launch, which begins the next episodes. */
+ * (at least 3 x 28 per SM), jx_reset, jx_step and jx_rollout each also launch
+ * the three kernels that build episodes ahead (a count, the walls of builds
+ * that start, then the build's share of the launch, after an 8-byte
+ * cudaMemsetAsync; on the same stream, or for a rollout in two passes on the
+ * env's side stream beside its draw; all capturable in a CUDA graph). A
+ * jx_rollout in two passes (see there) counts its walk and draw launches and
+ * the env kernel's, per segment of 16 to 128 steps (as many as the camera
+ * records hold, see jx_env_bytes). Steps of small batches with large frames
+ * count a second launch, which begins the next episodes. */
 jx_status jx_launch_count(const jx_env* env, uint64_t* count);
 
 /* Launch shape of the fused step kernel: grid blocks, threads per block,
@@ -474,7 +478,8 @@ jx_status jx_env_set_tiling(jx_env* env, const jx_tiling* tiling);
  * d_actions + t*n_envs and writes step t's slice of d_frames, d_rewards,
  * d_dones, laid out as for jx_batch_rollout). jx_graph_launch replays it on
  * a stream: one submission for all the steps. The graph keeps the batch's
- * tiling and the pointers of the capture; it must not outlive the batch. */
+ * tiling and the pointers of the capture, and stays valid when the batch's
+ * tiling changes; it must not outlive the batch. */
 jx_status jx_batch_capture(jx_batch* batch, int32_t steps, const uint8_t* d_actions, uint8_t* d_frames,
                            float* d_rewards, uint8_t* d_dones, jx_graph** out);
 jx_status jx_graph_launch(jx_graph* graph, void* stream);
@@ -551,7 +556,8 @@ jx_status jx_server_submit(jx_server* server, int32_t session, const uint8_t* h_
  * completed on the device. */
 jx_status jx_server_wait(jx_server* server, uint64_t ticket, double timeout_s);
 /* Hold (paused != 0) or resume the dispatcher: while held, submitted
- * requests queue and launches already on the device complete. */
+ * requests queue and launches already on the device complete. A hold waits
+ * until the launch that the dispatcher is issuing, if any, is out. */
 jx_status jx_server_pause(jx_server* server, int32_t paused);
 jx_status jx_server_stats(jx_server* server, jx_server_counters* out);
 /* Move up to `capacity` latencies (seconds from submit to completion seen

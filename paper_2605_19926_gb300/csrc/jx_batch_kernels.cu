@@ -78,11 +78,11 @@ __global__ void __launch_bounds__(kBatchMaxThreads, kBatchMinBlocks)
 }
 
 // One step of every env of a batch: a warp an env, the blocks of the groups one
-// after another, handed out as slots free. (The queues above serialise on
-// their counters, which every warp tries for every group: 16 groups of 1024
-// envs took 138 us per step, 74 here; and a warp's group, known from the
-// block index, is uniform, so its parameters are read without indexing.) A
-// step is a programmatic dependent like the env kernel's.
+// after another, handed out as slots free: 74 us a step of 16 groups of 1024
+// envs, 138 through the queues above, which serialise on their counters (every
+// warp tries every group's). A warp's group, known from the block index, is
+// uniform, so its parameters are read without indexing. A step is a
+// programmatic dependent like the env kernel's.
 template <int COLS, int SPEC>
 __global__ void __launch_bounds__(kBatchMaxThreads, kBatchMinBlocks)
     batch_step_kernel(const __grid_constant__ BatchParams bp) {

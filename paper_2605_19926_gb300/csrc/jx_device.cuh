@@ -685,11 +685,8 @@ __constant__ MazePick c_maze_pick = MazePick();
 // directions' neighbours are read where they are marked, so that the next
 // node's open sides are a shuffle away, the draw's choice is a word read one
 // carve ahead, a dead end is left by looking at 32 nodes of the path at once,
-// and the floor is laid afterwards from the visiting order. (4096 envs, 32 x
-// 32: a reset takes 72 us, 78 with the goal and the places in the order found in
-// passes of their own, 91 with the open sides loaded and the choice and the
-// map's bytes looked up and stored in each carve; 198 with one lane
-// walking and two moves a node.)
+// and the floor is laid afterwards from the visiting order. A reset of 4096 envs,
+// 32 x 32, takes 73 us, 69% of it issuing (198 us with one lane walking).
 // FAST_SMEM: the fast part lies in shared memory (an instance of its own, so
 // that the compiler knows the address space).
 template <bool FAST_SMEM>
@@ -1648,10 +1645,8 @@ struct Hit {
 // most 2 S of them the ray stands on a border cell. Lanes leave it as their
 // rays hit; no ballot is needed. Otherwise each crossing also tests the
 // bounds (a cell outside the map ends the ray, as wall 1), at most 4 S + 8.
-// (Recomputing only the crossed side, indexing cells instead of (x, y) pairs
-// and leaving without a ballot, with the depth test of project_sprites, took
-// the 4096-env rollout of 128 steps from 8.82 to 7.98 us per step, the one of
-// 20 steps from 9.67 to 9.33, and the single step from 13.4 to 12.9 us.)
+// What bounds it is the instructions a crossing issues: only the crossed side
+// is recomputed, and cells are indexed by one number.
 template <int MODE, int MAPK, int COLS>
 __device__ __forceinline__ void march(const Params& p, int e, const Env& r, Ray (&q)[COLS], Hit (&h)[COLS],
                                       const WarpSmem& ws, bool inside, const bool (&valid)[COLS]) {

@@ -462,7 +462,8 @@ int choose_parts(int steps, int64_t frame_bytes, int frame_px, int* ends) {
 }  // namespace
 
 int rollout_segment(int n) {
-  const int64_t fit = ((int64_t)64 << 20) / (24 * (int64_t)n);  // 64 MB of camera records
+  // 64 MB of camera records, but at least 16 steps (more than that above 174,762 envs: 384 bytes an env)
+  const int64_t fit = ((int64_t)64 << 20) / (24 * (int64_t)n);
   return fit > 128 ? 128 : (fit < 16 ? 16 : (int)fit);
 }
 

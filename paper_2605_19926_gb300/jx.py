@@ -281,7 +281,7 @@ class Env:
         _check(lib.jx_step(self._h, _stream(stream), _ptr(actions), _ptr(frames), _ptr(rewards), _ptr(dones)))
 
     def rollout(self, actions, frames, rewards, dones, stream=None):
-        """``actions.shape[0]`` steps in one launch (outputs shaped [steps, N, ...])."""
+        """``actions.shape[0]`` steps in one call (outputs shaped [steps, N, ...])."""
         steps = int(actions.shape[0])
         _check(lib.jx_rollout(self._h, _stream(stream), _ptr(actions), steps, _ptr(frames), _ptr(rewards),
                               _ptr(dones)))
