@@ -876,7 +876,7 @@ def headline(g: Gpu, args) -> dict | None:
                              traffic_unit="DRAM bytes per launch (ncu record, scaled by env-steps)",
                              algorithmic_bytes_per_step=bytes_total / args.steps,
                              algorithmic_bytes_per_launch=bytes_total / len(plan.launches),
-                             kernel="rollout_kernel (walk and draw), env_kernel for what they left"),
+                             kernel="rollout_kernel (walk and draw), env_kernel or handoff_kernel for what they left"),
         "cpu_baseline": cpu,
         "e2e": {"value": e2e_value, "unit": "env-steps/s", "h2d_bytes_per_step": N,
                 "d2h_bytes_per_step": N * H * W * 3 + 4 * N + N,

@@ -213,10 +213,10 @@ jx_status jx_step(jx_env* env, void* stream, const uint8_t* d_actions, uint8_t* 
  * last, then runs the envs whose episode ends in the rollout from that step
  * on. Next episodes of large mazes in large batches are built beside the draw,
  * on a stream of the env's own that `stream` waits for (also under capture).
- * Other rollouts run in the env kernel alone. In the env kernel each env's
- * pose stays in registers and its map in shared memory across its steps. For
- * 64 steps or more (envs without a grayscale stack) they are cut into chunks
- * of 12 steps that the launch's warps take in turn: a warp that finishes a
+ * Other rollouts run in the env kernel alone. There each env's pose stays in
+ * registers and its map in shared memory across its steps. For 64 steps or
+ * more (envs without a grayscale stack) a hand-off kernel takes its place: the
+ * steps are cut into chunks of 12 that the launch's warps take in turn: a warp that finishes a
  * chunk takes the next free one, of any env, and the chunk after it starts
  * once its env's previous chunk has stored the state (a hand-off through
  * device memory that a late partner cannot stall for more than a bounded wait;
@@ -356,7 +356,7 @@ jx_status jx_launch_count(const jx_env* env, uint64_t* count);
  * chip idle step and render with a block of 2 or 4 warps per env.) */
 jx_status jx_launch_shape(const jx_env* env, int32_t* grid, int32_t* block, int32_t* smem_bytes);
 
-/* Launch shape of the env kernel in a jx_rollout of `steps` steps (see
+/* Launch shape of the env (or hand-off) kernel in a jx_rollout of `steps` steps (see
  * jx_rollout): as jx_launch_shape, plus the steps per hand-off chunk (0: every
  * warp runs whole envs). For an env routed
  * through the batched kernel (jx_autotune) whose rollouts do not take two passes,

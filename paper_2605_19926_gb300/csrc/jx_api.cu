@@ -152,11 +152,11 @@ jx_status check_env(const jx_env* env) {
   return JX_OK;
 }
 
-// Steps per hand-off chunk of a rollout launch of the env kernel (0: each
-// warp runs whole envs). Measured on the 4096-env maze workload (10,000 steps
-// in 128-step launches) while all its steps ran in the env kernel, as those
-// after a horizon still do: chunks of 12 steps on 5/8 of the resident warps run
-// at 9.10-9.16 us per step against 9.44-9.46 us for whole envs on all of
+// Steps per hand-off chunk of a rollout launch (handoff_kernel; 0: the env
+// kernel, each warp whole envs). Measured on the 4096-env maze workload (10,000
+// steps in 128-step launches) before rollouts took two passes (the steps after
+// a horizon still run so): chunks of 12 steps on 5/8 of the resident warps
+// ran at 9.10-9.16 us per step against 9.44-9.46 us for whole envs on all of
 // them (the warps of an SM are served unequally, and the hand-off lets the
 // faster ones take more chunks; with fewer warps than envs a warp always finds
 // an item whose env is free). Rollouts of 20 steps lose more to the hand-off

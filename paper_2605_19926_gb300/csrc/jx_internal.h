@@ -22,6 +22,8 @@ constexpr int kMinBlocksPerSm = 28;  // register budget: 28 warps resident per S
 constexpr int kHandoffPolls = 1 << 22;  // default polls (about 0.25 us apart) before a rollout hand-off counts as late
 constexpr int kHandoffMinSteps = 64;    // rollouts of at least this many steps run in hand-off chunks
 constexpr int kHandoffChunk = 12;       // steps per hand-off chunk
+// blocks of a hand-off launch per SM: 5/8 of the env kernel's resident warps (see rollout_chunk)
+constexpr int kHandoffBlocksPerSm = (kMinBlocksPerSm * 5 / 8 + kWarpsPerBlock) / kWarpsPerBlock;
 
 // MODE_BEGIN starts the next episode of the envs whose done flag is set (after a
 // team's step) and draws its first frame.

@@ -1,6 +1,6 @@
-// jx_kernels.cu — the env kernel (one env config per launch, rollouts or what a
-// walk left of them in hand-off chunks), the team kernel (a block of warps per
-// env), the kernels that build next episodes ahead (a count, the
+// jx_kernels.cu — the env kernel (one env config per launch), the hand-off
+// kernel (rollouts or what a walk left of them in chunks), the team kernel (a
+// block of warps per env), the kernels that build next episodes ahead (a count, the
 // walls of the builds that start, then one lane per env advancing its build),
 // and their host side: launch shape queries, launches, the per-warp shared
 // memory layout.
@@ -88,40 +88,6 @@ __global__ void __launch_bounds__(kThreads, kMinBlocksPerSm / kWarpsPerBlock)
   const int nw = gridDim.x * kWarpsPerBlock;
   uint8_t* scratch = p.gen_scratch ? p.gen_scratch + (size_t)gw * p.gen_scratch_stride : nullptr;
   int slot = 0;
-  if (MODE == MODE_ROLLOUT && p.chunk > 0) {
-    if (p.stop != nullptr) {  // after the walk and the draw: only the envs they left
-      uint32_t left = 0u;
-      for (int i = lane; i < (p.n + 31) >> 5; i += 32) left |= p.ended[i];
-      if (!__any_sync(0xffffffffu, left != 0u)) return;  // the whole grid
-    }
-    const uint32_t nch = (uint32_t)((p.steps + p.chunk - 1) / p.chunk);
-    const uint32_t items = (uint32_t)p.n * nch;  // below 2^31 (the host caps it)
-    bool lost = false;
-    for (uint32_t item = take_item(p, lane); item < items;) {
-      const uint32_t next = take_item(p, lane);  // its latency overlaps this item
-      const int e = (int)(item % (uint32_t)p.n);
-      const uint32_t k = item / (uint32_t)p.n;
-      int t0 = (int)k * p.chunk;
-      const int t1 = t0 + p.chunk < p.steps ? t0 + p.chunk : p.steps;
-      const int first = p.stop != nullptr ? p.stop[e] : 0;  // the env's first step in this kernel
-      if (first >= t1) {
-        item = next;
-        continue;
-      }
-      if (first >= t0)
-        t0 = first;  // its first chunk: nothing to wait for
-      else if (!await_chunk(p, e, k) && lane == 0)
-        atomicOr(p.err, 4u);
-      // after a lost map copy the warp only passes its items on (their envs
-      // keep their state; the error word says so) and never touches the ring
-      if (!lost) lost = !run_env<MODE, MAPK, 1, GRAY>(p, e, wbase, scratch, lane, slot, t0, t1);
-      publish_chunk(p, e, k + 1 == nch ? 0u : k + 1, lane);
-      item = next;
-    }
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    finish_items(p, nw, lane);
-    return;
-  }
   for (int e = gw; e < p.n; e += nw) {
     const int first = MODE == MODE_ROLLOUT && p.stop != nullptr ? p.stop[e] : 0;
     if (MODE == MODE_ROLLOUT && first >= p.steps) continue;
@@ -130,6 +96,56 @@ __global__ void __launch_bounds__(kThreads, kMinBlocksPerSm / kWarpsPerBlock)
   if (!kEarlyRelease) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   // shared memory stays allocated until the bulk stores have read it
   if (lane == 0) bulk_wait_read_all();
+}
+
+// A rollout, or what a walk left of one, in hand-off chunks (envs without a
+// grayscale stack). A kernel of its own, on 5/8 of the warps that the env
+// kernel keeps resident, so that each may hold 96 registers: in one kernel
+// with the loop over whole envs, under its 72, the step loop spilled (128 steps
+// of 4096 ASCII envs, 24 x 24: 1323 us, 1097 here; of 600: 940, 800).
+template <int MAPK>
+__global__ void __launch_bounds__(kThreads, kHandoffBlocksPerSm) handoff_kernel(const __grid_constant__ Params p) {
+  extern __shared__ __align__(128) uint8_t smem_raw[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  uint8_t* const wbase = smem_raw + warp * p.warp_bytes;
+  write_palette(p, WarpSmem{wbase, FillLane{}}, lane);
+  if (!p.map_bits && p.S * p.S >= 4096) init_warp_header(wbase, lane);
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const int gw = blockIdx.x * kWarpsPerBlock + warp;
+  const int nw = gridDim.x * kWarpsPerBlock;
+  uint8_t* scratch = p.gen_scratch ? p.gen_scratch + (size_t)gw * p.gen_scratch_stride : nullptr;
+  int slot = 0;
+  if (p.stop != nullptr) {  // after the walk and the draw: only the envs they left
+    uint32_t left = 0u;
+    for (int i = lane; i < (p.n + 31) >> 5; i += 32) left |= p.ended[i];
+    if (!__any_sync(0xffffffffu, left != 0u)) return;  // the whole grid
+  }
+  const uint32_t nch = (uint32_t)((p.steps + p.chunk - 1) / p.chunk);
+  const uint32_t items = (uint32_t)p.n * nch;  // below 2^31 (the host caps it)
+  bool lost = false;
+  for (uint32_t item = take_item(p, lane); item < items;) {
+    const uint32_t next = take_item(p, lane);  // its latency overlaps this item
+    const int e = (int)(item % (uint32_t)p.n);
+    const uint32_t k = item / (uint32_t)p.n;
+    int t0 = (int)k * p.chunk;
+    const int t1 = t0 + p.chunk < p.steps ? t0 + p.chunk : p.steps;
+    const int first = p.stop != nullptr ? p.stop[e] : 0;  // the env's first step in this kernel
+    if (first >= t1) {
+      item = next;
+      continue;
+    }
+    if (first >= t0)
+      t0 = first;  // its first chunk: nothing to wait for
+    else if (!await_chunk(p, e, k) && lane == 0)
+      atomicOr(p.err, 4u);
+    // after a lost map copy the warp only passes its items on (their envs
+    // keep their state; the error word says so) and never touches the ring
+    if (!lost) lost = !run_env<MODE_ROLLOUT, MAPK, 1, 0>(p, e, wbase, scratch, lane, slot, t0, t1);
+    publish_chunk(p, e, k + 1 == nch ? 0u : k + 1, lane);
+    item = next;
+  }
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  finish_items(p, nw, lane);
 }
 
 // One plane word a thread.
@@ -281,6 +297,8 @@ __global__ void __launch_bounds__(kPregenThreads)
   }
 }
 
+auto handoff_kernel_of(const Params& p) { return p.map_bits ? handoff_kernel<MAP_BITS> : handoff_kernel<MAP_BYTES>; }
+
 // The env kernel of a mode for p's map kind and grayscale stack.
 template <int MODE>
 auto env_kernel_of(const Params& p) {
@@ -312,7 +330,7 @@ cudaError_t launch_mode(const Params& p, int grid, bool joined, cudaStream_t str
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = joined ? 0 : 1;
-  return cudaLaunchKernelEx(&cfg, env_kernel_of<MODE>(p), p);
+  return cudaLaunchKernelEx(&cfg, MODE == MODE_ROLLOUT && p.chunk > 0 ? handoff_kernel_of(p) : env_kernel_of<MODE>(p), p);
 }
 }  // namespace
 
@@ -416,6 +434,10 @@ cudaError_t team_launch(const Params& q, int mode, cudaStream_t stream) {
 }
 
 cudaError_t kernel_blocks_per_sm(const Params& p, int mode, int* blocks) {
+  if (mode == MODE_ROLLOUT) {
+    cudaError_t err = raise_smem_limit(handoff_kernel_of(p));
+    if (err != cudaSuccess) return err;
+  }
   switch (mode) {
     case MODE_STEP: return blocks_per_sm_mode<MODE_STEP>(p, blocks);
     case MODE_RESET: return blocks_per_sm_mode<MODE_RESET>(p, blocks);
