@@ -206,19 +206,20 @@ jx_status jx_step(jx_env* env, void* stream, const uint8_t* d_actions, uint8_t* 
  * sequence of jx_step calls.
  *  d_actions [steps][N] uint8; d_frames [steps][N][H][W][3] uint8;
  *  d_rewards [steps][N] float32; d_dones [steps][N] uint8.
- * Rollouts of 2 steps or more (of envs that jx_create made, except the ASCII
- * task) run in two passes: a walk steps every agent up to the step that ends
- * its episode, one lane per env, and leaves a camera record per env and step;
- * a draw renders the records' frames in any order. The env kernel, launched
- * last, then runs the envs whose episode ends in the rollout from that step
- * on. Next episodes of large mazes in large batches are built beside the draw,
- * on a stream of the env's own that `stream` waits for (also under capture).
+ * Rollouts of 2 steps or more (of 3 to 12 or more for small frames; of envs
+ * that jx_create made, except the ASCII task) run in two passes: a walk steps
+ * every agent up to the step that ends its episode, one lane per env, and
+ * leaves a camera record per env and step; a draw renders the records' frames
+ * in any order. The env kernel, launched last, then runs the envs whose episode
+ * ends in the rollout from that step on. Next episodes of large mazes in large
+ * batches are built beside the draw, on a stream of the env's own that `stream`
+ * waits for (also under capture).
  * Other rollouts run in the env kernel alone. There each env's pose stays in
- * registers and its map in shared memory across its steps. For 64 steps or
- * more (envs without a grayscale stack) a hand-off kernel takes its place: the
- * steps are cut into chunks of 12 that the launch's warps take in turn: a warp that finishes a
- * chunk takes the next free one, of any env, and the chunk after it starts
- * once its env's previous chunk has stored the state (a hand-off through
+ * registers and its map in shared memory across its steps. For 64 steps or more
+ * (envs without a grayscale stack) a hand-off kernel takes its place: the steps
+ * are cut into chunks of 12 that the launch's warps take in turn: a warp that
+ * finishes a chunk takes the next free one, of any env, and the chunk after it
+ * starts once its env's previous chunk has stored the state (a hand-off through
  * device memory that a late partner cannot stall for more than a bounded wait;
  * bit 2 of the device error word records one that ran out).
  * Asynchronous on `stream`; allocates nothing. steps >= 1. Launches of one

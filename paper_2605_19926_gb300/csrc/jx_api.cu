@@ -191,11 +191,18 @@ jx_status launch_env(jx_env* env, const jx::Params& p, int mode, cudaStream_t s,
   return JX_OK;
 }
 
+// Whether a rollout walks first and draws afterwards.
+bool walks_first(const jx_env* env, int steps) {
+  return env->base.stop &&
+         steps >= jx::rollout_min_steps(env->cfg.task, env->cfg.map_side, env->cfg.n_envs,
+                                        env->cfg.frame_h * env->cfg.frame_w, env->draw_slots);
+}
+
 // Whether the next episodes of a rollout of p.steps steps are built beside its
 // draw. (16,384 envs of 128 x 128 cells and pixels, 8 steps: 1312 us a
 // launch before the walk, 1234 beside the draw.)
 bool pregen_beside_draw(const jx_env* env, const jx::Params& p) {
-  return env->side && p.stop && p.steps >= jx::kRolloutMinSteps && jx::pregen_runs(p);
+  return env->side && walks_first(env, p.steps) && jx::pregen_runs(p);
 }
 
 // The pre-generation of a rollout of `steps` steps on the env's side stream,
@@ -215,18 +222,19 @@ jx_status pregen_beside(jx_env* env, const jx::Params& p, int steps, cudaStream_
   return JX_OK;
 }
 
-// Whether a rollout walks first and draws afterwards: the same on every route,
-// so that it never takes the batched one (which has neither the builds beside
-// the draw nor the hand-off).
+// Whether a rollout keeps the env's own route where an env is tuned to the
+// batched one, which has neither the builds beside the draw nor the hand-off:
+// the walk and the draw are the same on both.
 bool two_passes(const jx_env* env, int steps) { return env->base.stop && steps >= jx::kRolloutMinSteps; }
 
 // A rollout of p.steps steps: walk, draw and the env kernel for what they left,
-// in segments that the camera records hold; envs without records in the env
-// kernel alone.
+// in segments that the camera records hold; envs without records, and rollouts
+// too short to gain from it, in the env kernel alone.
 jx_status run_rollout(jx_env* env, jx::Params p, cudaStream_t s) {
   const int steps = p.steps;
   if (steps < jx::kRolloutMinSteps) return launch_env(env, p, jx::MODE_STEP, s);
-  if (!p.stop) {
+  if (!walks_first(env, steps)) {
+    p.stop = nullptr;
     p.chunk = rollout_chunk(env, steps);
     return launch_env(env, p, jx::MODE_ROLLOUT, s);
   }

@@ -219,11 +219,14 @@ cudaError_t launch(const Params& p, int mode, int grid, bool joined, cudaStream_
 
 // Rollouts in two passes (jx_rollout.cu). Camera records are kept for at most
 // rollout_segment(n) steps: longer rollouts run in segments of that many.
-// A rollout of one step is a step. From two steps on the two passes and the
-// env kernel's last look take less than stepping and drawing in turn (alone, from a cold stream: 89 envs,
-// 96 x 96, 3 steps 27.7 us against 49.2; 5562 uneven envs, 3 steps 97 against 321;
-// 4096 envs, 64 x 64, 2 steps 34.9 against 34.4).
+// A rollout of one step is a step. From two steps on batches roll out in two
+// passes (5562 uneven envs, 3 steps: 97 us against 321 in the batched kernel),
+// single envs from rollout_min_steps on.
 constexpr int kRolloutMinSteps = 2;
+// The fewest steps that n envs of a task with maps of the given side and frames
+// of px pixels roll out in two passes (slots: warps resident at once); shorter
+// rollouts run in the env kernel alone.
+int rollout_min_steps(int task, int side, int n, int px, int slots);
 int rollout_segment(int n);
 bool rollout_wanted(int task);  // whether envs of a task roll out in two passes
 size_t rollout_bytes(int n);    // camera records, stop steps and end words of n envs

@@ -461,6 +461,37 @@ int choose_parts(int steps, int64_t frame_bytes, int frame_px, int* ends) {
 }
 }  // namespace
 
+// Two passes take two launches more and the walk's chain, some 6 us a call, and
+// save per step what a warp's frame takes beyond its share of a full chip. So
+// the line lies higher where frames are small, in mazes, whose rays are short,
+// and where a step's warps just fill the chip (one round, none waiting), which
+// suits the env kernel best. Calls back to back, us, env kernel / two passes:
+//   mazes of side 32, 32 x 32: 600 envs 3 steps 11.9 / 12.3, 4 14.1 / 13.1;
+//     4096 envs 4 steps 22.9 / 27.8, 8 40.9 / 44.6, 10 51.5 / 52.8; 64 x 64: 1200
+//     envs 2 steps 13.4 / 15.0, 3 19.3 / 17.4; 4096 envs 3 steps 30.3 / 34.0, 6
+//     55.9 / 55.6; 128 x 128: 2400 envs 2 steps 43.4 / 54.9, 4 81.3 / 82.1; 4096
+//     envs 2 steps 70.1 / 71.7, 3 102.4 / 98.1
+//   rooms of side 64 with sprites, 32 x 32: 1200 envs 2 steps 12.0 / 13.1, 3
+//     16.3 / 14.1; 64 x 64: 4096 envs 3 steps 35.8 / 38.9, 5 56.2 / 56.2
+// In mazes of four nodes an episode lasts a few dozen steps, so most envs leave
+// the walk, and their rest runs as in the env kernel alone: 64 x 64, 4096 envs
+// 8 steps 80 / 101, 20 steps 194 / 223, 48 454 / 478; 600 envs 8 steps 47 / 41.
+int rollout_min_steps(int task, int side, int n, int px, int slots) {
+  const bool small = px <= 32 * 32, maze = task != 0;
+  const bool fits = n <= slots, fills = fits && n > slots * 3 / 10;
+  if (maze && side < 8) {
+    if (px > 64 * 64) return fits && n > slots * 2 / 5 ? 32 : 2;
+    return !fits ? 16 : (n > slots / 4 ? 48 : (small ? 12 : 4));
+  }
+  if (px > 64 * 64) return fits && n > slots * 2 / 5 ? 3 : 2;
+  if (!fits) return small ? (maze ? 6 : 4) : 3;
+  const int few = (small ? 3 : 2) + (maze ? 1 : 0);
+  if (!fills) return few;
+  const int at = maze ? 2 : (small ? 3 : 1), slope = maze && small ? 9 : 4;  // from few envs to a full chip
+  const int line = at + (int)((int64_t)slope * n / slots);
+  return line > few ? line : few;
+}
+
 int rollout_segment(int n) {
   // 64 MB of camera records, but at least 16 steps (more than that above 174,762 envs: 384 bytes an env)
   const int64_t fit = ((int64_t)64 << 20) / (24 * (int64_t)n);

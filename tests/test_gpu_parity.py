@@ -926,3 +926,43 @@ def test_rollout_from_a_negative_step_count_equals_single_steps(T):
         assert torch.equal(a.rewards, rewards[t]) and torch.equal(a.dones, dones[t]), t
     torch.cuda.synchronize()
     assert (a.env.get_state() == b.env.get_state()).all()
+
+
+@pytest.mark.parametrize("task,fill,hw,line", [("maze", 0.01, (32, 32), 4), ("rooms", 0.01, (32, 32), 3),
+                                               ("maze", 0.01, (64, 64), 3), ("rooms", 0.01, (48, 64), 2),
+                                               ("maze", 0.01, (64, 80), 2), ("maze", 0.6, (16, 32), 7),
+                                               ("rooms", 0.6, (16, 32), 5), ("maze", 0.9, (33, 32), 5),
+                                               ("rooms", 0.9, (33, 32), 4), ("maze", 0.6, (66, 64), 3),
+                                               ("maze", 1.1, (8, 16), 6), ("rooms", 1.1, (8, 16), 4),
+                                               ("maze", 1.1, (33, 32), 3), ("maze6", 0.6, (8, 16), 48),
+                                               ("maze6", 0.1, (33, 32), 4), ("maze6", 1.1, (8, 16), 16)])
+def test_short_rollouts_keep_the_env_kernel(task, fill, hw, line):
+    """Rollouts of fewer steps than gain from two passes are one launch of the env
+    kernel, from there on several launches; on both sides of the line they equal
+    single steps. `fill`: envs over the warps resident at once."""
+    slots = 28 * torch.cuda.get_device_properties(0).multi_processor_count
+    n, (h, w) = int(fill * slots), hw
+    if task != "rooms":
+        cfg = inputs.maze_keydoor(n_envs=n, map_side=6 if task == "maze6" else 16, seed=84, horizon=5, frame_h=h,
+                                  frame_w=w)
+    else:
+        cfg = dict(inputs.rooms(n_envs=n, map_side=16, seed=85, max_sprites=2, frame_h=h, frame_w=w), horizon=5)
+    a, b = Run(cfg), Run(cfg)
+    a.reset()
+    b.reset()
+    for T in (line - 1, line):
+        acts = torch.from_numpy(np.stack([forward_biased_actions(86 + T, s, n) for s in range(T)])).to(a.dev)
+        frames = torch.zeros((T, n, h, w, 3), dtype=torch.uint8, device=a.dev)
+        rewards = torch.zeros((T, n), dtype=torch.float32, device=a.dev)
+        dones = torch.zeros((T, n), dtype=torch.uint8, device=a.dev)
+        before = b.env.launch_count()
+        b.env.rollout(acts, frames, rewards, dones)
+        launches = b.env.launch_count() - before
+        assert T == 1 or (launches == 1) == (T < line), (T, launches)
+        for t in range(T):
+            a.actions.copy_(acts[t])
+            a.env.step(a.actions, a.frames, a.rewards, a.dones)
+            assert torch.equal(a.frames, frames[t]), (T, t)
+            assert torch.equal(a.rewards, rewards[t]) and torch.equal(a.dones, dones[t]), (T, t)
+        torch.cuda.synchronize()
+        assert (a.env.get_state() == b.env.get_state()).all(), T
